@@ -728,6 +728,7 @@ int run_layers_few(asr_spec* h) {
 // LayerNorm -> the target's tied LM head with argmax (when `lm`).
 int draft_block(asr_spec* h, const RowPlan& plan, int rows, bool lm) {
   const int d = h->d, F2 = 2 * h->d;
+  const int rows_per_utt = (rows + h->B - 1) / h->B;
   DraftW& w = h->dw;
   Epi base{};
   base.n_valid = plan.n_rows;
@@ -776,7 +777,7 @@ int draft_block(asr_spec* h, const RowPlan& plan, int rows, bool lm) {
   at.vc = static_cast<const __nv_bfloat16*>(h->d_vs);
   at.t_alloc = h->maxpos;
   at.causal = 1;
-  launch_draft_attn(at, h->st);
+  launch_draft_attn(at, rows_per_utt, h->st);
   e = base;
   e.bias = w.bo;
   e.x = h->d_x;
@@ -792,7 +793,7 @@ int draft_block(asr_spec* h, const RowPlan& plan, int rows, bool lm) {
   at.vc = static_cast<const __nv_bfloat16*>(h->d_xkv) + half;
   at.t_alloc = h->Tmax;
   at.causal = 0;
-  launch_draft_attn(at, h->st);
+  launch_draft_attn(at, rows_per_utt, h->st);
   e = base;
   e.bias = w.bco;
   e.x = h->d_x;

@@ -323,62 +323,149 @@ __global__ void draft_finish_kernel(DraftArgs A, int* lens_out) {
   if (b < A.B) lens_out[b] = A.lens[b] < 0 ? -1 : A.n_prop[b];
 }
 
-// Attention of the draft's block for the rows of one (utterance, head):
+// Attention of the draft's block for up to NR rows of one (utterance, head):
 // keys [0, pos + 1) of the self cache (causal) or [row_lo, row_hi) of the
 // encoder K/V (cross); fp32 scores, softmax and sums over the bf16 caches.
 // Cache layout [B_max][H][t_alloc][64]; q [R][d] fp32; out [R][d] bf16.
-__global__ void __launch_bounds__(128) draft_attn_kernel(DraftAttn a) {
-  extern __shared__ float s_p[];   // [t_alloc] scores / probabilities
-  __shared__ float s_q[64], s_red[8], s_o[2][64];
-  const int hh = blockIdx.x, b = blockIdx.y, tid = threadIdx.x;
-  const int n = a.plan.n_utt_rows[b];
-  const int r0 = a.plan.row_start[b];
+//
+// Bound by the latency of the key and value loads: a catch-up row reads every
+// frame (192 KB of keys per head), a proposal row a window of 41.  Eight lanes
+// hold one key (16 bytes each, coalesced), a warp four keys, the CTA 32 keys
+// and DA_U of those steps in flight, keys and values requested together; each
+// eight-lane group keeps its own online softmax, merged in a fixed order at
+// the end.  Rows of one utterance share the loads (NR = 4 for catch-up passes,
+// 1 where every utterance has one row).  The row-by-row kernel
+// with four-byte loads before it took 55 us a launch on average over two
+// rounds of the cached loop at batch 1 (d = 1280, k = 8, 1500 frames).
+constexpr int DA_T = 256, DA_U = 4;
+
+template <int NR>
+__global__ void __launch_bounds__(DA_T) draft_attn_kernel(DraftAttn a) {
+  __shared__ float s_m[DA_T / 32][NR], s_l[DA_T / 32][NR], s_o[DA_T / 32][NR][64];
+  __shared__ int s_ok[NR];   // 0: a row refused by the bounds-check mode
+  const int hh = blockIdx.x, b = blockIdx.y, tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int i0 = blockIdx.z * NR, nr = min(NR, a.plan.n_utt_rows[b] - i0);
+  if (nr <= 0) return;
+  const int r0 = a.plan.row_start[b] + i0;
   const size_t head = ((size_t)b * a.H + hh) * a.t_alloc;
-  const __nv_bfloat16* K = a.kc + head * 64;
-  const __nv_bfloat16* V = a.vc + head * 64;
-  for (int i = 0; i < n; ++i) {
-    const int r = r0 + i;
-    const int lo = a.causal ? 0 : a.row_lo[r];
-    const int hi = a.causal ? a.plan.row_pos[r] + 1 : a.row_hi[r];
-    if (bounds_bad(a.status, lo < 0 || hi > a.t_alloc || hi <= lo)) continue;   // uniform over the CTA
-    if (tid < 64) s_q[tid] = a.q[(size_t)r * a.d + hh * 64 + tid] * 0.125f;
-    __syncthreads();
-    float m = -INFINITY;
-    for (int j = lo + tid; j < hi; j += 128) {
-      const __nv_bfloat162* kr = reinterpret_cast<const __nv_bfloat162*>(K + (size_t)j * 64);
-      float s = 0.f;
-#pragma unroll 8
-      for (int c = 0; c < 32; ++c) {
-        const float2 kv = __bfloat1622float2(kr[c]);
-        s = fmaf(s_q[2 * c], kv.x, fmaf(s_q[2 * c + 1], kv.y, s));
-      }
-      s_p[j - lo] = s;
-      m = fmaxf(m, s);
+  const int grp = tid >> 3, sub = tid & 7;   // 32 groups of eight lanes, 8 dimensions per lane
+  const __nv_bfloat16* K = a.kc + head * 64 + 8 * sub;
+  const __nv_bfloat16* V = a.vc + head * 64 + 8 * sub;
+  int lo[NR], hi[NR], jlo = 0x7fffffff, jhi = 0;
+  float q[NR][8], o[NR][8], m[NR], l[NR];
+#pragma unroll
+  for (int i = 0; i < NR; ++i) {
+    lo[i] = hi[i] = 0;
+    if (i < nr) {
+      lo[i] = a.causal ? 0 : a.row_lo[r0 + i];
+      hi[i] = a.causal ? a.plan.row_pos[r0 + i] + 1 : a.row_hi[r0 + i];
+      if (bounds_bad(a.status, lo[i] < 0 || hi[i] > a.t_alloc || hi[i] <= lo[i])) lo[i] = hi[i] = 0;
     }
-    m = warp_max(m);
-    if ((tid & 31) == 0) s_red[tid >> 5] = m;
-    __syncthreads();
-    m = fmaxf(fmaxf(s_red[0], s_red[1]), fmaxf(s_red[2], s_red[3]));
-    float l = 0.f;
-    for (int j = lo + tid; j < hi; j += 128) {
-      const float p = expf(s_p[j - lo] - m);
-      s_p[j - lo] = p;
-      l += p;
+    if (tid == 0) s_ok[i] = hi[i] > lo[i];
+    if (hi[i] > lo[i]) {
+      jlo = min(jlo, lo[i]);
+      jhi = max(jhi, hi[i]);
     }
-    l = warp_sum(l);
-    __syncthreads();
-    if ((tid & 31) == 0) s_red[4 + (tid >> 5)] = l;
-    __syncthreads();
-    l = (s_red[4] + s_red[5]) + (s_red[6] + s_red[7]);
-    // output column c = tid & 63 over the keys of half tid >> 6
-    const int c = tid & 63, half = tid >> 6;
-    float o = 0.f;
-    for (int j = lo + half; j < hi; j += 2) o = fmaf(s_p[j - lo], __bfloat162float(V[(size_t)j * 64 + c]), o);
-    s_o[half][c] = o;
-    __syncthreads();
-    if (tid < 64) a.out[(size_t)r * a.d + hh * 64 + tid] = __float2bfloat16_rn((s_o[0][tid] + s_o[1][tid]) / l);
-    __syncthreads();
+    const float* qr = a.q + (size_t)(r0 + (i < nr ? i : 0)) * a.d + hh * 64 + 8 * sub;
+    const float4 q0 = *reinterpret_cast<const float4*>(qr), q1 = *reinterpret_cast<const float4*>(qr + 4);
+    q[i][0] = q0.x * 0.125f; q[i][1] = q0.y * 0.125f; q[i][2] = q0.z * 0.125f; q[i][3] = q0.w * 0.125f;
+    q[i][4] = q1.x * 0.125f; q[i][5] = q1.y * 0.125f; q[i][6] = q1.z * 0.125f; q[i][7] = q1.w * 0.125f;
+    m[i] = -INFINITY;
+    l[i] = 0.f;
+#pragma unroll
+    for (int e = 0; e < 8; ++e) o[i][e] = 0.f;
   }
+  auto unpack = [](const uint4& w, float* f) {
+    const uint32_t u[4] = {w.x, w.y, w.z, w.w};
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {   // bf16 pairs: low half first
+      f[2 * e] = __uint_as_float(u[e] << 16);
+      f[2 * e + 1] = __uint_as_float(u[e] & 0xffff0000u);
+    }
+  };
+  for (int j0 = jlo; j0 < jhi; j0 += 32 * DA_U) {   // uniform over the CTA
+    uint4 kw[DA_U], vw[DA_U];
+#pragma unroll
+    for (int u = 0; u < DA_U; ++u) {
+      const int j = min(j0 + 32 * u + grp, jhi - 1);   // in range; masked below
+      kw[u] = *reinterpret_cast<const uint4*>(K + (size_t)j * 64);
+      vw[u] = *reinterpret_cast<const uint4*>(V + (size_t)j * 64);
+    }
+    float s[NR][DA_U];
+#pragma unroll
+    for (int u = 0; u < DA_U; ++u) {
+      float kf[8];
+      unpack(kw[u], kf);
+      const int j = j0 + 32 * u + grp;
+#pragma unroll
+      for (int i = 0; i < NR; ++i) {
+        float t = 0.f;
+#pragma unroll
+        for (int e = 0; e < 8; ++e) t = fmaf(q[i][e], kf[e], t);
+        t += __shfl_xor_sync(0xffffffffu, t, 1);
+        t += __shfl_xor_sync(0xffffffffu, t, 2);
+        t += __shfl_xor_sync(0xffffffffu, t, 4);
+        s[i][u] = j >= lo[i] && j < hi[i] ? t : -INFINITY;
+      }
+    }
+#pragma unroll
+    for (int i = 0; i < NR; ++i) {
+      float mx = m[i];
+#pragma unroll
+      for (int u = 0; u < DA_U; ++u) mx = fmaxf(mx, s[i][u]);
+      const float c = mx == -INFINITY ? 0.f : expf(m[i] - mx);
+      m[i] = mx;
+      l[i] *= c;
+#pragma unroll
+      for (int e = 0; e < 8; ++e) o[i][e] *= c;
+#pragma unroll
+      for (int u = 0; u < DA_U; ++u) s[i][u] = mx == -INFINITY ? 0.f : expf(s[i][u] - mx);
+    }
+#pragma unroll
+    for (int u = 0; u < DA_U; ++u) {
+      float vf[8];
+      unpack(vw[u], vf);
+#pragma unroll
+      for (int i = 0; i < NR; ++i) {
+        l[i] += s[i][u];
+#pragma unroll
+        for (int e = 0; e < 8; ++e) o[i][e] = fmaf(s[i][u], vf[e], o[i][e]);
+      }
+    }
+  }
+  // merge the warp's four groups, then the warps, in a fixed order
+#pragma unroll
+  for (int i = 0; i < NR; ++i) {
+#pragma unroll
+    for (int x = 8; x <= 16; x <<= 1) {
+      const float om = __shfl_xor_sync(0xffffffffu, m[i], x), ol = __shfl_xor_sync(0xffffffffu, l[i], x);
+      const float mx = fmaxf(m[i], om);
+      const float c0 = mx == -INFINITY ? 0.f : expf(m[i] - mx), c1 = mx == -INFINITY ? 0.f : expf(om - mx);
+      m[i] = mx;
+      l[i] = l[i] * c0 + ol * c1;
+#pragma unroll
+      for (int e = 0; e < 8; ++e) o[i][e] = o[i][e] * c0 + __shfl_xor_sync(0xffffffffu, o[i][e], x) * c1;
+    }
+    if (lane < 8) {
+#pragma unroll
+      for (int e = 0; e < 8; ++e) s_o[warp][i][8 * sub + e] = o[i][e];
+      if (lane == 0) {
+        s_m[warp][i] = m[i];
+        s_l[warp][i] = l[i];
+      }
+    }
+  }
+  __syncthreads();
+  const int i = tid >> 6, c = tid & 63;   // one output column of one row per thread
+  if (i >= nr || !s_ok[i]) return;
+  float mx = -INFINITY, lt = 0.f, ot = 0.f;
+  for (int w = 0; w < DA_T / 32; ++w) mx = fmaxf(mx, s_m[w][i]);
+  for (int w = 0; w < DA_T / 32; ++w) {
+    const float f = expf(s_m[w][i] - mx);
+    lt += s_l[w][i] * f;
+    ot += s_o[w][i][c] * f;
+  }
+  a.out[(size_t)(r0 + i) * a.d + hh * 64 + c] = __float2bfloat16_rn(ot / lt);
 }
 
 }  // namespace
@@ -414,13 +501,11 @@ void launch_draft_softmax(const float* logits, int V, const int* n_rows, int row
                           float* row_p, cudaStream_t st) {
   draft_softmax_kernel<<<std::max(1, rows_max), 256, 0, st>>>(logits, V, n_rows, row_key, row_p);
 }
-void launch_draft_attn(const DraftAttn& a, cudaStream_t st) {
-  static bool configured = false;
-  if (!configured) {
-    cudaFuncSetAttribute(draft_attn_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 64 * 1024);
-    configured = true;
-  }
-  draft_attn_kernel<<<dim3(a.H, a.B), 128, (size_t)a.t_alloc * 4, st>>>(a);
+// One row per utterance (every continuation pass): a CTA per row and head.
+// More: groups of four rows share the key and value loads.
+void launch_draft_attn(const DraftAttn& a, int rows_per_utt, cudaStream_t st) {
+  if (rows_per_utt <= 1) draft_attn_kernel<1><<<dim3(a.H, a.B), DA_T, 0, st>>>(a);
+  else draft_attn_kernel<4><<<dim3(a.H, a.B, (rows_per_utt + 3) / 4), DA_T, 0, st>>>(a);
 }
 
 }  // namespace asrspec

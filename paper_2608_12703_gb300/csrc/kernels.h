@@ -282,7 +282,8 @@ void launch_draft_embed(const DraftArgs& a, int rows_max, const void* tok_emb, c
                         cudaStream_t st);
 void launch_draft_take(const DraftArgs& a, cudaStream_t st);
 void launch_draft_finish(const DraftArgs& a, int* lens_out, cudaStream_t st);
-void launch_draft_attn(const DraftAttn& a, cudaStream_t st);
+// rows_per_utt: the most rows of one utterance in the pass
+void launch_draft_attn(const DraftAttn& a, int rows_per_utt, cudaStream_t st);
 // Per row of logits [rows][V] (fp32): the argmax key (as the LM-head epilogue
 // writes it: lowest index on ties) and the softmax probability of the argmax.
 void launch_draft_softmax(const float* logits, int V, const int* n_rows, int rows_max, unsigned long long* row_key,

@@ -206,6 +206,17 @@ def test_draft_ragged_batch_windows(built_lib, cuda, kind):
     assert ds.proposals > 60
 
 
+@pytest.mark.parametrize("k", [3, 4])
+def test_draft_attention_edges(built_lib, cuda, k):
+    """Encoder lengths at the edges of the draft attention's 32- and 128-key
+    steps, and catch-up passes that fill one group of four rows (k = 3) or
+    leave one over (k = 4), whole-audio restarts included."""
+    enc_lens = [32, 33, 128, 129, 31]
+    total = [W.PROMPT_LEN + n for n in (15, 12, 16, 9, 14)]
+    st, ds, seqs, truth, _ = run_lockstep(enc_lens, total, k, None, seed=5)
+    _check(f"attention edges k{k}", st, ds, seqs, truth, total)
+
+
 def test_draft_edges(built_lib, cuda):
     """A one-token prompt (zero representations for the first restart), k = 0
     rounds between full ones, an utterance whose only round offers no draft
