@@ -82,7 +82,7 @@ struct asr_spec {
   int* attn_tickets = nullptr;                       // [B_max * H], tensor-core attention merge
   CUtensorMap m_kself[2], m_vself[2], m_xkv[2];      // boxes of 128 and 256 rows
   std::map<std::pair<int, int>, CUtensorMap> bmaps;  // (buffer id, BN) -> map
-  std::map<int, CUtensorMap> xmaps;                   // BN -> map of the residual stream (fp32, box 128 x BN)
+  std::map<std::pair<int, int>, CUtensorMap> xmaps;   // (target 0 / draft 1, BN) -> map of its residual stream (fp32, box 128 x BN)
   int n_sms = 0;
   bool use_wide = true;   // many-row projections on the one-tile-per-SM kernel (ASRSPEC_WIDE=0: the split-K chain)
   int fr_prefetch = 3;    // few-row launches prefetch the weights of the launch this many ahead into L2 (0: none)
@@ -270,12 +270,14 @@ const CUtensorMap* bmap(asr_spec* h, int id, const void* buf, int rows, int cols
   return &(h->bmaps[key] = m);
 }
 
-const CUtensorMap* xmap(asr_spec* h, int bn) {
-  auto it = h->xmaps.find(bn);
+// x: the target's residual stream or the draft's (both the handle's own, [R_pad][d])
+const CUtensorMap* xmap(asr_spec* h, const float* x, int bn) {
+  auto key = std::make_pair(x == h->x ? 0 : 1, bn);
+  auto it = h->xmaps.find(key);
   if (it != h->xmaps.end()) return &it->second;
   CUtensorMap m;
-  if (!make_tmap_f32(&m, h->x, h->R_pad, h->d, 128, bn)) return nullptr;
-  return &(h->xmaps[bn] = m);
+  if (!make_tmap_f32(&m, x, h->R_pad, h->d, 128, bn)) return nullptr;
+  return &(h->xmaps[key] = m);
 }
 
 // The next launch's slot of the per-CTA phase trace, or null (tracing off or the buffer full).
@@ -304,10 +306,9 @@ int gemm_rows(asr_spec* h, const void* W, const CUtensorMap* mW, int M, int K, c
     return 0;
   }
   WideGemm w{};
-  if (N > 64 && h->use_wide && wide_pick(M, N, K, mode, h->n_sms, &w.bn, &w.split) &&
-      (mode != EPI_RESID || epi.x == h->x)) {
+  if (h->use_wide && wide_pick(M, N, K, mode, h->n_sms, &w.bn, &w.split)) {
     const CUtensorMap* mb = bmap(h, x_id, X, h->R_pad, K, w.bn);
-    const CUtensorMap* mx = mode == EPI_RESID ? xmap(h, w.bn) : mW;
+    const CUtensorMap* mx = mode == EPI_RESID ? xmap(h, epi.x, w.bn) : mW;
     if (!mb || !mx) return fail(h, ASR_E_CUDA, "tensor map encode failed");
     w.mapA = *mW;
     w.mapB = *mb;

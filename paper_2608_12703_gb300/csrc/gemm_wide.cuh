@@ -1,7 +1,7 @@
-// tcgen05 GEMM for the projections of many verify rows (more than 64): one
-// 128 x BN output tile per CTA and about one CTA per SM, so that every SM
-// streams with a deep pipeline and the weights are re-read as few times as the
-// SM count allows (BN is picked from the rows and the SM count).
+// tcgen05 GEMM for the projections of the verify rows: one 128 x BN output tile
+// per CTA and at most about one CTA per SM, so that every SM streams with a
+// deep pipeline and the weights are re-read as few times as the SM count
+// allows (BN and the K split are picked from the rows and the SM count).
 //
 //   P = WG_PIPES pipelines, each over every P-th k-block with its own ring of
 //   (A, B) stages and its own accumulator in tensor memory:
@@ -17,10 +17,21 @@
 //                     order, out of tensor memory into shared memory
 //   warps 0 - 7     : the epilogue, one row per warp at a time, 4 features per lane
 //
-// Long K (at least 48 k-blocks) splits in two over a cluster pair: both CTAs
-// stage their partial tile, and each sums half of the rows in rank order
-// (rank 0 + rank 1, reading the peer's half through distributed shared
-// memory), so that results do not depend on timing.
+// What bounds it: many rows, the 64 bytes per clock that an SM takes from L2
+// (a k-block of a 128 x 32 tile is 20 KB, 155 ns of the 170 measured); few
+// rows, latency: 0.55 us to the first k-block, 0.2 us per k-block, the
+// epilogue.  So where the tiles leave SMs idle, K splits over a cluster of 2
+// or 4: each CTA stages its partial tile, sends the rows that another rank
+// owns into that rank's shared memory with st.async (bytes counted on the
+// owner's mbarrier) and sums its own rows over the ranks in a fixed order, so
+// that results do not depend on timing; the epilogue's rows are split too.
+// One projection of 35 rows (d = 1280, K split over 4) takes 3.2 - 4.8 us;
+// one CTA per tile took 6.3 - 9.3, the earlier 8- and 16-way split of narrow
+// tiles 8.5 - 16.7; exchange 0.9 us, against 1.5 by a bulk copy of the staged
+// rows and 1.15 plus a second cluster barrier by reading the peers' tiles.
+// Tiles too large for a receive buffer (BN 96 split in two) still read the
+// peer's staged rows through distributed shared memory between two cluster
+// barriers.
 #pragma once
 
 #include "kernels.h"
@@ -36,17 +47,25 @@ constexpr int WG_DYN_MAX = 220 * 1024;   // dynamic shared memory budget of one 
 constexpr int WG_PIPES = 3;
 static_assert(2 * WG_PIPES <= 6, "warps 0 .. 2 P - 1 hold the pipeline roles; at least two warps stay free");
 
-template <int BN, int MODE>
+template <int BN, int MODE, int SPLIT = 1>
 struct WideCfg {
   static constexpr int A_BYTES = 128 * 64 * 2;
   static constexpr int B_BYTES = BN * 64 * 2;
   static constexpr int STAGE_BYTES = A_BYTES + B_BYTES;
   static constexpr int XT_BYTES = MODE == EPI_RESID ? BN * 128 * 4 : 0;   // residual tile [BN][128] fp32
   static constexpr int LDS = 128 + 4;                                     // staged tile row stride (floats)
-  static constexpr int FIT = (WG_DYN_MAX - 1024 - 256 - XT_BYTES) / STAGE_BYTES;
+  static constexpr int ROWS = BN / SPLIT;   // rows of the tile that a CTA of a split writes
+  // receive buffer of a split: the other ranks' partials of this CTA's rows,
+  // where it fits beside two stages per pipeline (else the owners read the
+  // peers' staged tiles)
+  static constexpr int PUSH_BYTES = (SPLIT - 1) * ROWS * LDS * 4;
+  static constexpr bool PUSH =
+      SPLIT > 1 && WG_DYN_MAX - 1024 - 256 - XT_BYTES - PUSH_BYTES >= 2 * WG_PIPES * STAGE_BYTES;
+  static constexpr int RECV_BYTES = PUSH ? PUSH_BYTES : 0;
+  static constexpr int FIT = (WG_DYN_MAX - 1024 - 256 - XT_BYTES - RECV_BYTES) / STAGE_BYTES;
   static constexpr int STAGES = FIT < 8 ? FIT : 8;
   // dynamic shared memory for s stages per pipeline (the staged tile reuses the ring)
-  static constexpr int smem_bytes(int s) { return 1024 + WG_PIPES * s * STAGE_BYTES + XT_BYTES + 256; }
+  static constexpr int smem_bytes(int s) { return 1024 + WG_PIPES * s * STAGE_BYTES + XT_BYTES + RECV_BYTES + 256; }
   static constexpr int SMEM = smem_bytes(STAGES / WG_PIPES);
   // accumulators, split over the pipelines (within a pipeline the K = 16
   // steps of a k-block rotate over its share)
@@ -81,7 +100,7 @@ template <int BN, int MODE, int SPLIT>
 __global__ void __launch_bounds__(WG_THREADS, 1)
 gemm_wide_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUtensorMap mapB,
                  const __grid_constant__ CUtensorMap mapX, int K, int S, Epi epi, int* status) {
-  using C = WideCfg<BN, MODE>;
+  using C = WideCfg<BN, MODE, SPLIT>;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   // layout for S stages per pipeline: A ring, B ring, residual tile, barriers
@@ -89,11 +108,13 @@ gemm_wide_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant
   uint8_t* sA = smem;
   uint8_t* sB = smem + NS * C::A_BYTES;
   float* xt = reinterpret_cast<float*>(smem + NS * C::STAGE_BYTES);
-  uint64_t* full = reinterpret_cast<uint64_t*>(smem + NS * C::STAGE_BYTES + C::XT_BYTES);
+  float* recv = reinterpret_cast<float*>(smem + NS * C::STAGE_BYTES + C::XT_BYTES);   // split: [rank][ROWS][LDS]
+  uint64_t* full = reinterpret_cast<uint64_t*>(smem + NS * C::STAGE_BYTES + C::XT_BYTES + C::RECV_BYTES);
   uint64_t* empty = full + NS;
   uint64_t* done = empty + NS;   // [WG_PIPES]
   uint64_t* xbar = done + WG_PIPES;
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(xbar + 1);
+  uint64_t* rbar = xbar + 1;     // split: the other ranks' partials have landed
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(rbar + 1);
   __shared__ float ln_mu[BN], ln_rs[BN];   // folded LayerNorm: statistics of the tile's rows
   __shared__ int s_rb[BN], s_rp[BN];       // QKV: utterance and position of the tile's rows
   __shared__ __align__(16) float s_op[4][128];   // the tile's bias, folded-LayerNorm c1, c2, next gain
@@ -127,11 +148,19 @@ gemm_wide_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant
     }
     for (int p = 0; p < WG_PIPES; ++p) mbar_init(&done[p], 1);
     mbar_init(xbar, 1);
+    if constexpr (C::PUSH) {
+      mbar_init(rbar, 1);
+      const int mine = min(C::ROWS, n_valid - n0 - split * C::ROWS);   // rows this CTA will write
+      mbar_arrive_expect_tx(rbar, (uint32_t)(mine > 0 ? (SPLIT - 1) * mine * 512 : 0));
+    }
     fence_mbar_init();
   }
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
+  // split: announce the receive barrier; the matching wait comes just before
+  // the first remote copy, long after every peer has arrived
+  if constexpr (C::PUSH) cluster_arrive_relaxed();
   const uint32_t tmem = *tmem_slot;
   if (tr && threadIdx.x == 0) tr[1] = global_ns();
 
@@ -199,12 +228,10 @@ gemm_wide_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant
     }
     umma_commit(&done[pipe]);
   } else {
-    pdl_wait();
-    pdl_launch();
-    if (warp >= 2 * WG_PIPES) {   // the warps without a pipeline role
-      constexpr int NT = WG_THREADS - 64 * WG_PIPES;
-      const int t = threadIdx.x - 64 * WG_PIPES;
-      // the epilogue's per-feature operands of this tile
+    constexpr int NT = WG_THREADS - 64 * WG_PIPES;   // threads of the warps without a pipeline role
+    const int t = (int)threadIdx.x - 64 * WG_PIPES;
+    if (warp >= 2 * WG_PIPES) {
+      // the epilogue's per-feature operands of this tile (constants: before the wait)
       for (int f = t; f < 128; f += NT) {
         s_op[0][f] = __ldg(epi.bias + m0 + f);
         if (epi.ln_part != nullptr && MODE != EPI_RESID) {
@@ -213,6 +240,10 @@ gemm_wide_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant
         }
         if (MODE == EPI_RESID && epi.xg != nullptr) s_op[3][f] = __ldg(epi.xg_gain + m0 + f);
       }
+    }
+    pdl_wait();
+    pdl_launch();
+    if (warp >= 2 * WG_PIPES) {
       // Folded LayerNorm: row statistics combined from the producer's equal
       // slices, one pass shifted by the first slice's mean:
       // mean = shift + E / S, M2 = sum M2_s + c (sum e_s^2 - E^2 / S)
@@ -225,12 +256,18 @@ gemm_wide_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant
           const float shift = ok ? pr[0].x : 0.f;
           float e1 = 0.f, e2 = 0.f, m2 = 0.f;
           if (ok)
-            for (int j = 0; j < S; ++j) {
-              const float2 p = pr[(size_t)j * epi.ln_stride];
-              const float es = p.x - shift;
-              e1 += es;
-              e2 += es * es;
-              m2 += p.y;
+            for (int j0 = 0; j0 < S; j0 += 8) {   // eight slices' loads in flight
+              float2 p[8];
+#pragma unroll
+              for (int u = 0; u < 8; ++u)
+                p[u] = j0 + u < S ? pr[(size_t)(j0 + u) * epi.ln_stride] : make_float2(shift, 0.f);
+#pragma unroll
+              for (int u = 0; u < 8; ++u) {
+                const float es = p[u].x - shift;
+                e1 += es;
+                e2 += es * es;
+                m2 += p[u].y;
+              }
             }
           const float mean = shift + e1 / (float)S;
           const float q = m2 + (float)epi.ln_c * fmaxf(e2 - e1 * e1 / (float)S, 0.f);
@@ -292,8 +329,27 @@ gemm_wide_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant
     }
   }
   if (tr && threadIdx.x == 0) tr[5] = global_ns();
-  __syncthreads();
-  if constexpr (SPLIT > 1) cluster_sync();   // the peer's partial tile is staged too
+  if constexpr (C::PUSH) {
+    __syncthreads();
+    cluster_wait();   // every peer's receive barrier is initialised
+    // the staged rows that the other ranks own, whole rows per warp: row rr of
+    // rank (split + 1 + rr / ROWS) mod SPLIT
+    for (int rr = warp; rr < (SPLIT - 1) * C::ROWS; rr += WG_THREADS / 32) {
+      const int to = (split + 1 + rr / C::ROWS) % SPLIT, row = rr % C::ROWS;
+      if (to * C::ROWS + row >= n_valid - n0) continue;
+      const int slot = (split - to + SPLIT) % SPLIT - 1;   // this rank's place in the owner's buffer
+      st_async_f4(dsmem_addr(recv + (slot * C::ROWS + row) * C::LDS + 4 * lane, (uint32_t)to),
+                  *reinterpret_cast<const float4*>(stg + (to * C::ROWS + row) * C::LDS + 4 * lane),
+                  dsmem_addr(rbar, (uint32_t)to));
+    }
+    mbar_wait(rbar, 0, status);
+    __syncwarp();
+    // no CTA leaves before its peers' rows have landed (the wait at the end)
+    cluster_arrive_relaxed();
+  } else {
+    __syncthreads();
+    if constexpr (SPLIT > 1) cluster_sync();   // the peers' partial tiles are staged too
+  }
   if (tr && threadIdx.x == 0) tr[6] = global_ns();
 
   if constexpr (MODE == EPI_RESID) mbar_wait(xbar, 0, status);   // the residual tile has landed
@@ -303,9 +359,8 @@ gemm_wide_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant
   const float4 gain = (MODE == EPI_RESID && epi.xg) ? *reinterpret_cast<const float4*>(&s_op[3][4 * lane])
                                                     : make_float4(0.f, 0.f, 0.f, 0.f);
   if (tr && threadIdx.x == 0) tr[10] = global_ns();
-  const int r_lo = SPLIT > 1 ? split * (BN / 2) : 0;
-  const int r_end = min(SPLIT > 1 ? r_lo + BN / 2 : BN, n_valid - n0);
-  const uint32_t peer = (uint32_t)(split ^ 1);
+  const int r_lo = split * (BN / SPLIT);
+  const int r_end = min(r_lo + BN / SPLIT, n_valid - n0);
   constexpr int RB = 4;   // rows per batch per warp, loads in flight together
   for (int j0 = r_lo + warp; j0 < r_end; j0 += 8 * RB) {
     if (tr && threadIdx.x == 0 && j0 == r_lo + 8 * RB) tr[11] = global_ns();
@@ -315,11 +370,24 @@ gemm_wide_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant
       const int nl = j0 + 8 * r;
       a[r] = nl < r_end ? *reinterpret_cast<const float4*>(stg + nl * C::LDS + 4 * lane)
                         : make_float4(0.f, 0.f, 0.f, 0.f);
-      if constexpr (SPLIT > 1) {   // rank 0's partial + rank 1's, in that order
+      if constexpr (SPLIT > 1) {   // the ranks' partials, pairwise
         if (nl < r_end) {
-          const float4 p = ld_dsmem_f4(dsmem_addr(stg + nl * C::LDS + 4 * lane, peer));
-          a[r] = split == 0 ? make_float4(a[r].x + p.x, a[r].y + p.y, a[r].z + p.z, a[r].w + p.w)
-                            : make_float4(p.x + a[r].x, p.y + a[r].y, p.z + a[r].z, p.w + a[r].w);
+          float4 p[SPLIT];
+#pragma unroll
+          for (int s = 0; s < SPLIT; ++s) {
+            if constexpr (C::PUSH) {
+              const int slot = (s - split + SPLIT) % SPLIT - 1;
+              p[s] = s == split ? a[r]
+                                : *reinterpret_cast<const float4*>(recv + (slot * C::ROWS + nl - r_lo) * C::LDS + 4 * lane);
+            } else {
+              p[s] = ld_dsmem_f4(dsmem_addr(stg + nl * C::LDS + 4 * lane, (uint32_t)s));
+            }
+          }
+          auto add = [](const float4& u, const float4& v) {
+            return make_float4(u.x + v.x, u.y + v.y, u.z + v.z, u.w + v.w);
+          };
+          a[r] = add(p[0], p[1]);
+          if constexpr (SPLIT == 4) a[r] = add(a[r], add(p[2], p[3]));
         }
       }
     }
@@ -372,7 +440,8 @@ gemm_wide_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant
     }
   }
   if (tr && threadIdx.x == 0) tr[7] = global_ns();
-  if constexpr (SPLIT > 1) cluster_sync();   // the peer has read this CTA's partial
+  if constexpr (C::PUSH) cluster_wait();   // the peers have this CTA's partials
+  else if constexpr (SPLIT > 1) cluster_sync();   // the peers have read this CTA's partial
   if (tr && threadIdx.x == 0) tr[4] = global_ns();
   tc_fence_before();
   __syncthreads();

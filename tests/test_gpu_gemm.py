@@ -67,3 +67,16 @@ def test_wide_gemm_matches_torch(built_lib, cuda, impl, M, N, K):
     else:
         err = (c - ref).abs().max().item()
         assert err <= 1e-4 * K ** 0.5, err
+
+
+# K split over 4, 2 or 1 CTAs by the number of tiles and k-blocks; rows at the edges of the 32-row tiles
+FEW_SHAPES = [(1280, 1, 1280), (1280, 31, 5120), (1280, 32, 832), (3840, 33, 1280), (5120, 12, 1280), (5120, 35, 1280),
+              (1280, 96, 1280), (1280, 97, 1280), (768, 64, 768), (768, 30, 384), (256, 9, 192), (128, 128, 768)]
+
+
+@pytest.mark.parametrize("impl", [5, 6, 7])
+@pytest.mark.parametrize("M,N,K", FEW_SHAPES)
+def test_few_row_split_gemm_matches_torch(built_lib, cuda, impl, M, N, K):
+    """The same kernel where few tiles leave K to be split over a cluster: the
+    bounds of the many-row shapes (fp32 sums of K bf16 products)."""
+    test_wide_gemm_matches_torch(built_lib, cuda, impl, M, N, K)
