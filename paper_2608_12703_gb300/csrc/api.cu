@@ -398,13 +398,19 @@ int gemm_rows_ln(asr_spec* h, const void* W, const CUtensorMap* mW, int M, int K
 }
 
 // The decoder layers over the rows laid out by the last plan kernel.
-// CTAs per (utterance, head) for the tensor-core attention: few utterances
-// (batch 1) split the keys over a cluster of up to 8 CTAs.
-int attn_splits_for(asr_spec* h, int t_alloc) {
+// CTAs (one cluster) per (utterance, head) for the tensor-core attention.
+// Encoder keys split while the clusters all run at once: a cluster of 8 or 4
+// is packed inside a GPC, so only part of the two-per-SM slots can be used;
+// past them the last clusters run as a second wave (large decoder, 5
+// utterances: 8.2 us with 200 CTAs, 11.6 with 400; small, 3 utterances: 5.9
+// with 144, 9.5 with 288).  Self-attention keys (a transcript: mostly one
+// 128-key chunk of the four that 448 positions have) do not pay for the merge
+// until a CTA would have more than eight chunks: 3.4 us unsplit against 5.0
+// and 8.5 in two and four at 60 keys, and each further chunk costs 0.9 us.
+int attn_splits_for(asr_spec* h, int t_alloc, bool self_attn) {
   const int nc_max = (t_alloc + 127) / 128;
   int S = 1;
-  // split until every SM has two CTAs (the ring of each keeps 96 KB in flight)
-  while (S < 8 && S * 2 <= nc_max && h->B * h->H * S < 2 * NUM_SMS_TARGET) S *= 2;
+  while (S < 8 && S * (self_attn ? 16 : 2) <= nc_max && h->B * h->H * S * 2 <= 200) S *= 2;
   return S;
 }
 
@@ -413,7 +419,7 @@ void attention(asr_spec* h, AttnArgs& a, bool self_attn, int layer) {
     launch_attention(a, h->st);
     return;
   }
-  a.splits = attn_splits_for(h, a.t_alloc);
+  a.splits = attn_splits_for(h, a.t_alloc, self_attn);
   const int ci = 0;   // 128-row boxes
   if (self_attn) {
     a.kmap = &h->m_kself[ci];
