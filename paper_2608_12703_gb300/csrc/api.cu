@@ -65,7 +65,7 @@ struct asr_spec {
   int *enc_len = nullptr, *kv_len = nullptr, *pending = nullptr, *ready = nullptr;
 
   int R_max = 0, R_pad = 0;
-  float *x = nullptr, *q = nullptr, *q_anchor = nullptr, *ml = nullptr, *part = nullptr;
+  float *x = nullptr, *q = nullptr, *q_anchor = nullptr, *ml = nullptr;
   void *xn = nullptr, *att = nullptr, *hbuf = nullptr, *xf = nullptr;
   RowPlan plan{};
   unsigned long long* row_key = nullptr;
@@ -287,8 +287,9 @@ unsigned long long* trace_slot(asr_spec* h) {
 }
 
 // One projection over the verify rows: out-features m (weights = A), rows n (activations = B).
+// ln_g / ln_b (fp32 models, f32_rows only): X holds the rows x and the operand is LayerNorm(x).
 int gemm_rows(asr_spec* h, const void* W, const CUtensorMap* mW, int M, int K, const void* X, int x_id, int N,
-              int mode, const Epi& epi_in) {
+              int mode, const Epi& epi_in, const float* ln_g = nullptr, const float* ln_b = nullptr) {
   Epi epi = epi_in;
   epi.M = M;
   epi.N = N;
@@ -302,7 +303,17 @@ int gemm_rows(asr_spec* h, const void* W, const CUtensorMap* mW, int M, int K, c
                                       : ASR_PROF_LMHEAD;
   Prof p(h, cls, 1);
   if (!h->bf16) {
-    launch_gemm_simt(W, 0, X, 0, M, N, K, mode, epi, h->st);
+    F32Gemm g{};
+    g.A = static_cast<const float*>(W);
+    g.B = static_cast<const float*>(X);
+    g.M = M;
+    g.N = N;
+    g.K = K;
+    g.ln_g = ln_g;
+    g.ln_b = ln_b;
+    g.sms = h->n_sms;
+    g.pdl = h->use_pdl;
+    launch_gemm_f32(g, mode, epi, h->st);
     return 0;
   }
   WideGemm w{};
@@ -389,6 +400,7 @@ int gemm_rows_ln(asr_spec* h, const void* W, const CUtensorMap* mW, int M, int K
     fold_consumer(h, e, c1, c2);
     return gemm_rows(h, W, mW, M, K, h->xn, BUF_XN, N, mode, e);
   }
+  if (!h->bf16 && f32_rows(N, K)) return gemm_rows(h, W, mW, M, K, h->x, 0, N, mode, e, g, b);   // normalised in the GEMM
   {
     Prof p(h, ASR_PROF_LAYERNORM, 1);
     Tl t(h, ASR_TL_LAYERNORM);
@@ -416,7 +428,8 @@ int attn_splits_for(asr_spec* h, int t_alloc, bool self_attn) {
 
 void attention(asr_spec* h, AttnArgs& a, bool self_attn, int layer) {
   if (!h->bf16) {
-    launch_attention(a, h->st);
+    a.pdl = h->use_pdl;
+    launch_attention_f32(a, h->st);
     return;
   }
   a.splits = attn_splits_for(h, a.t_alloc, self_attn);
@@ -514,16 +527,13 @@ int run_layers(asr_spec* h, int N) {
     a.H = h->H;
     a.d = d;
     a.k1 = h->kmax + 1;
-    a.chunk = attn_chunk_len(h->bf16);
-    a.n_chunks = (h->maxpos + a.chunk - 1) / a.chunk;
-    a.part = h->part;
     a.out = h->att;
     a.out_bf16 = h->bf16;
     a.ml_out = nullptr;
     a.rows_max = rows_max;
     a.tree = h->cur_tree;
     {
-      Prof p(h, ASR_PROF_SELF, h->bf16 ? 1 : 2);
+      Prof p(h, ASR_PROF_SELF, 1);
       attention(h, a, true, l);
     }
     a.tree = false;
@@ -544,10 +554,9 @@ int run_layers(asr_spec* h, int N) {
     a.vc = vx;
     a.t_alloc = h->Tmax;
     a.causal = 0;
-    a.n_chunks = (h->Tmax + a.chunk - 1) / a.chunk;
     a.ml_out = (l == h->anchor) ? h->ml : nullptr;
     {
-      Prof p(h, ASR_PROF_CROSS, h->bf16 ? 1 : 2);
+      Prof p(h, ASR_PROF_CROSS, 1);
       attention(h, a, false, l);
     }
     e = base;
@@ -962,7 +971,7 @@ int asr_spec_create(const asr_model_dims* dims, const asr_weights* weights, void
     const char* e = std::getenv("ASRSPEC_CHECK");
     const int on = e && std::atoi(e) != 0;
     set_check_gemm_tc(on);
-    set_check_gemm_simt(on);
+    set_check_gemm_f32(on);
     set_check_gemm_wide(on);
     set_check_rows(on);
     set_check_attention(on);
@@ -1154,9 +1163,6 @@ int asr_spec_create(const asr_model_dims* dims, const asr_weights* weights, void
     if ((rc = dalloc(h, &h->ln_part, (size_t)(d / 8) * R * sizeof(float2)))) return finish(rc);
     CK(cudaMemset(h->ln_part, 0, (size_t)(d / 8) * R * sizeof(float2)));
   }
-  const int chunk = h->bf16 ? 128 : attn_chunk_len(0);   // the finest split either path uses
-  const int n_chunks = (std::max(h->maxpos, h->Tmax) + chunk - 1) / chunk;
-  if ((rc = dalloc(h, &h->part, (size_t)h->Bmax * h->H * n_chunks * (h->kmax + 1) * 66 * 4))) return finish(rc);
   if ((rc = dalloc(h, &h->plan.row_b, R * 4)) || (rc = dalloc(h, &h->plan.row_i, R * 4)) ||
       (rc = dalloc(h, &h->plan.row_pos, R * 4)) || (rc = dalloc(h, &h->plan.row_tok, R * 4)) ||
       (rc = dalloc(h, &h->plan.row_epos, R * 4)) || (rc = dalloc(h, &h->plan.row_mask, R * 4)) ||
@@ -1221,7 +1227,7 @@ int asr_spec_create(const asr_model_dims* dims, const asr_weights* weights, void
     }
   }
   configure_gemm_tc();
-  configure_attention();
+  configure_attention_tc();
   CK(cudaDeviceSynchronize());
   return finish(0);
 }
@@ -1271,7 +1277,13 @@ int asr_spec_encode_cache(asr_spec_handle h, int32_t B, const void* enc_states, 
     launch_gemm_tc(g, EPI_CROSSKV, e, h->status, h->st);
   } else {
     Prof pg(h, ASR_PROF_OTHER, 1);
-    launch_gemm_simt(enc_states, 0, h->w_cross, 0, M, N, d, EPI_CROSSKV, e, h->st);
+    F32Gemm g{};
+    g.A = static_cast<const float*>(enc_states);
+    g.B = static_cast<const float*>(h->w_cross);
+    g.M = M;
+    g.N = N;
+    g.K = d;
+    launch_gemm_f32(g, EPI_CROSSKV, e, h->st);
   }
   if (h->has_draft && h->bf16) {   // the draft's own cross K/V of the same encoder states
     Epi de = e;
@@ -1809,6 +1821,9 @@ int asr_spec_debug_logits(asr_spec_handle h, float* out, int32_t max_rows) {
   if (h->ln_fold && !h->last_fused) {   // the same operand and statistics as the last verify's LM head
     fold_consumer(h, e, h->c1_lm, h->c2_lm);
     rc = gemm_rows(h, h->w_tok, &h->m_tok, h->V, h->d, h->xn, BUF_XN, R, EPI_F32, e);
+  } else if (!h->bf16) {   // the residual stream of the last verify, normalised as for its LM head
+    rc = gemm_rows_ln(h, h->w_tok, &h->m_tok, h->V, h->d, h->lnf_g, h->lnf_b, nullptr, nullptr, h->xf, BUF_XF, R,
+                      EPI_F32, e);
   } else {
     rc = gemm_rows(h, h->w_tok, &h->m_tok, h->V, h->d, h->xf, BUF_XF, R, EPI_F32, e);
   }
@@ -1863,7 +1878,7 @@ int asr_spec_test_gemm(int32_t impl, const void* A, const void* B, float* C, int
   e.out_f32 = C;
   e.ld = N;
   if (impl == 1) {
-    launch_gemm_simt(A, 1, B, 1, M, N, K, EPI_F32_MN, e, st);
+    launch_gemm_simt(A, B, M, N, K, C, st);
   } else if (impl == 3) {
     // fused argmax over m for every n: C[n] = index of the largest C[.][n]
     TcGemm g{};

@@ -1,15 +1,10 @@
-// Split-KV attention over the verify rows, and the re-anchoring readout.
+// Attention of fp32 models over the verify rows, and the re-anchoring readout.
 //
 // Self-attention (Sec. 3 "Speculative Loop": the target checks the whole
 // draft block in one pass): row i of utterance b sits at position P_b + i and
 // attends to cached keys 0 .. P_b + i, i.e. the committed cache plus rows
 // 0..i of its own block (a block-causal mask).  Cross-attention: every row
 // attends to the utterance's enc_len[b] encoder frames.
-//
-// One CTA takes one (utterance, head, key chunk): it stages the chunk's K and V
-// in shared memory once and serves every row of that utterance from it.  Each
-// chunk leaves (max, sum, unnormalised output) per row; a merge kernel
-// combines the chunks in chunk order.
 //
 // Anchor (Sec. 5 "Verification-Attention Correction"; App. "Runtime anchor
 // construction"): the head mean of the per-head softmax attention of one row
@@ -25,168 +20,202 @@ ASRSPEC_CHECK_SETTER(set_check_attention)
 
 constexpr float ATTN_SCALE = 0.125f;  // 1 / sqrt(64)
 
-// q . k over 64 dims, visiting the 32 element pairs starting at pair (j mod 32):
-// consecutive rows of a shared-memory tile then hit different banks.  The same
-// order is used by the anchor readout so both compute identical scores.
-template <typename T>
-__device__ __forceinline__ float dot64_rot(const float* q, const T* k, int j) {
-  float acc = 0.f;
-#pragma unroll 8
-  for (int t = 0; t < 32; ++t) {
-    const int w = (t + j) & 31;
-    acc = fmaf(q[2 * w], to_f<T>(k[2 * w]), acc);
-    acc = fmaf(q[2 * w + 1], to_f<T>(k[2 * w + 1]), acc);
-  }
-  return acc;
-}
+// One CTA takes one (utterance, head, key split) and up to four rows; the
+// splits of a (utterance, head, row group) form one cluster.  Bound by the
+// latency of the key and value loads (few utterances) or their bandwidth.
+// Eight lanes hold one key (two 16-byte loads each of K and V), the CTA 32 keys
+// per step and FA_U steps in flight; the encoder keys of the first steps are
+// requested before the wait on the previous kernel.  Each eight-lane group
+// keeps an online softmax, groups, warps and splits merge in a fixed order.
+// The score of a key is the sum that the anchor readout forms.
+constexpr int FA_T = 256, FA_U = 2, FA_NR = 4;
 
-constexpr int ATTN_THREADS = 256;
-constexpr int ATTN_MAX_ROWS = 32;   // rows per utterance served by one CTA (k + 1 <= 32)
-
-template <typename T, int CHUNK>
-__global__ void __launch_bounds__(ATTN_THREADS) attn_chunk_kernel(AttnArgs a) {
-  extern __shared__ __align__(16) uint8_t smem[];
-  T* Ks = reinterpret_cast<T*>(smem);
-  T* Vs = Ks + CHUNK * 64;
-  float* Qs = reinterpret_cast<float*>(Vs + CHUNK * 64);     // [rows][64]
-  float* S = Qs + ATTN_MAX_ROWS * 64;                        // [rows][CHUNK]
-  __shared__ float s_m[ATTN_MAX_ROWS], s_l[ATTN_MAX_ROWS];
-
-  const int chunk = blockIdx.x, h = blockIdx.y, b = blockIdx.z;
-  const int nr = a.plan.n_utt_rows[b];
-  if (nr == 0) return;
-  const int row0 = a.plan.row_start[b];
-  const int n_keys = a.causal ? a.kv_len[b] + nr : a.enc_len[b];
-  if (bounds_bad(a.status, n_keys > a.t_alloc || n_keys > a.n_chunks * a.chunk)) return;
-  const int key0 = chunk * CHUNK;
-  if (key0 >= n_keys) return;
-  const int nk = min(CHUNK, n_keys - key0);
-  const int tid = threadIdx.x;
-
-  // stage K, V (contiguous [nk][64] for this (b, h)) and the rows' queries
-  const size_t base = (((size_t)b * a.H + h) * a.t_alloc + key0) * 64;
-  const T* gK = static_cast<const T*>(a.kc) + base;
-  const T* gV = static_cast<const T*>(a.vc) + base;
-  constexpr int VEC = 16 / sizeof(T);
-  const int nvec = nk * 64 / VEC;
-  for (int v = tid; v < nvec; v += ATTN_THREADS) {
-    reinterpret_cast<uint4*>(Ks)[v] = __ldg(reinterpret_cast<const uint4*>(gK) + v);
-    reinterpret_cast<uint4*>(Vs)[v] = __ldg(reinterpret_cast<const uint4*>(gV) + v);
-  }
-  for (int e = tid; e < nr * 64; e += ATTN_THREADS) {
-    const int i = e >> 6, c = e & 63;
-    Qs[e] = a.q[(size_t)(row0 + i) * a.d + h * 64 + c];
-  }
-  __syncthreads();
-
-  // scores
-  for (int e = tid; e < nr * nk; e += ATTN_THREADS) {
-    const int i = e / nk, j = e - i * nk;
-    const int key = key0 + j;
-    float s = dot64_rot<T>(Qs + i * 64, Ks + j * 64, j) * ATTN_SCALE;
-    if (a.causal && key > a.plan.row_pos[row0 + i]) s = -INFINITY;
-    S[i * CHUNK + j] = s;
-  }
-  __syncthreads();
-
-  // per-row max and sum over the chunk (one warp per row)
-  const int warp = tid >> 5, lane = tid & 31;
-  for (int i = warp; i < nr; i += ATTN_THREADS / 32) {
-    float m = -INFINITY;
-    for (int j = lane; j < nk; j += 32) m = fmaxf(m, S[i * CHUNK + j]);
-    m = warp_max(m);
-    float l = 0.f;
-    for (int j = lane; j < nk; j += 32) {
-      const float s = S[i * CHUNK + j];
-      const float p = (s == -INFINITY) ? 0.f : expf(s - m);
-      S[i * CHUNK + j] = p;
-      l += p;
+__global__ void __launch_bounds__(FA_T) attn_f32_kernel(AttnArgs a) {
+  __shared__ float s_m[8][FA_NR], s_l[8][FA_NR], s_o[8][FA_NR][64];
+  __shared__ __align__(16) float p_o[FA_NR][64];   // this split's (max, sum, output) per row
+  __shared__ float p_m[FA_NR], p_l[FA_NR];
+  const int S = a.splits, split = blockIdx.x % S, h = blockIdx.y, b = blockIdx.z;
+  const int i0 = (int)(blockIdx.x / S) * FA_NR;
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, grp = tid >> 3, sub = tid & 7;
+  const size_t head = ((size_t)b * a.H + h) * a.t_alloc;
+  const float* K = static_cast<const float*>(a.kc) + head * 64 + 8 * sub;
+  const float* V = static_cast<const float*>(a.vc) + head * 64 + 8 * sub;
+  // the keys of this split: a contiguous range of whole 32-key steps
+  int jlo = 0, jhi = 0;
+  float4 kw[FA_U][2], vw[FA_U][2];
+  auto range = [&](int n_keys) {
+    const int st = (n_keys + 31) / 32;
+    jlo = st * split / S * 32;
+    jhi = min(st * (split + 1) / S * 32, n_keys);
+  };
+  auto load = [&](int j0) {
+#pragma unroll
+    for (int u = 0; u < FA_U; ++u) {
+      const int j = min(j0 + 32 * u + grp, jhi - 1);   // in range; masked below
+      const float4* kp = reinterpret_cast<const float4*>(K + (size_t)j * 64);
+      const float4* vp = reinterpret_cast<const float4*>(V + (size_t)j * 64);
+      kw[u][0] = kp[0];
+      kw[u][1] = kp[1];
+      vw[u][0] = vp[0];
+      vw[u][1] = vp[1];
     }
-    l = warp_sum(l);
-    if (lane == 0) {
-      s_m[i] = m;
-      s_l[i] = l;
+  };
+  bool loaded = false;
+  if (!a.causal) {   // constant during a verify call
+    const int n = a.enc_len[b];
+    if (n <= a.t_alloc) {
+      range(n);
+      if (jhi > jlo) {
+        load(jlo);
+        loaded = true;
+      }
     }
   }
+  pdl_wait();
+  pdl_launch();
+  const int n_rows = a.plan.n_utt_rows[b], nr = min(FA_NR, n_rows - i0);
+  const int n_keys = a.causal ? a.kv_len[b] + n_rows : a.enc_len[b];
+  if (nr <= 0 || bounds_bad(a.status, n_keys > a.t_alloc)) return;   // uniform over the cluster
+  if (!loaded) range(n_keys);
+  const int r0 = a.plan.row_start[b] + i0;
+  int hi[FA_NR];
+  float q[FA_NR][8], o[FA_NR][8], m[FA_NR], l[FA_NR];
+#pragma unroll
+  for (int i = 0; i < FA_NR; ++i) {
+    const int r = r0 + (i < nr ? i : 0);
+    hi[i] = i >= nr ? 0 : a.causal ? min(n_keys, a.plan.row_pos[r] + 1) : n_keys;
+    const float* qr = a.q + (size_t)r * a.d + h * 64 + 8 * sub;
+    const float4 q0 = *reinterpret_cast<const float4*>(qr), q1 = *reinterpret_cast<const float4*>(qr + 4);
+    q[i][0] = q0.x; q[i][1] = q0.y; q[i][2] = q0.z; q[i][3] = q0.w;
+    q[i][4] = q1.x; q[i][5] = q1.y; q[i][6] = q1.z; q[i][7] = q1.w;
+    m[i] = -INFINITY;
+    l[i] = 0.f;
+#pragma unroll
+    for (int e = 0; e < 8; ++e) o[i][e] = 0.f;
+  }
+  for (int j0 = jlo; j0 < jhi; j0 += 32 * FA_U) {   // uniform over the CTA
+    if (!loaded) load(j0);
+    loaded = false;
+    float s[FA_NR][FA_U];
+#pragma unroll
+    for (int u = 0; u < FA_U; ++u) {
+      const int j = j0 + 32 * u + grp;
+#pragma unroll
+      for (int i = 0; i < FA_NR; ++i) {
+        const float4 k0 = kw[u][0], k1 = kw[u][1];
+        float t = 0.f;
+        t = fmaf(q[i][0], k0.x, t); t = fmaf(q[i][1], k0.y, t); t = fmaf(q[i][2], k0.z, t); t = fmaf(q[i][3], k0.w, t);
+        t = fmaf(q[i][4], k1.x, t); t = fmaf(q[i][5], k1.y, t); t = fmaf(q[i][6], k1.z, t); t = fmaf(q[i][7], k1.w, t);
+        t += __shfl_xor_sync(0xffffffffu, t, 1);
+        t += __shfl_xor_sync(0xffffffffu, t, 2);
+        t += __shfl_xor_sync(0xffffffffu, t, 4);
+        s[i][u] = j < hi[i] && j < jhi ? t * ATTN_SCALE : -INFINITY;
+      }
+    }
+#pragma unroll
+    for (int i = 0; i < FA_NR; ++i) {
+      float mx = m[i];
+#pragma unroll
+      for (int u = 0; u < FA_U; ++u) mx = fmaxf(mx, s[i][u]);
+      const float c = mx == -INFINITY ? 0.f : expf(m[i] - mx);
+      m[i] = mx;
+      l[i] *= c;
+#pragma unroll
+      for (int e = 0; e < 8; ++e) o[i][e] *= c;
+#pragma unroll
+      for (int u = 0; u < FA_U; ++u) {
+        const float p = mx == -INFINITY ? 0.f : expf(s[i][u] - mx);
+        const float4 v0 = vw[u][0], v1 = vw[u][1];
+        l[i] += p;
+        o[i][0] = fmaf(p, v0.x, o[i][0]); o[i][1] = fmaf(p, v0.y, o[i][1]);
+        o[i][2] = fmaf(p, v0.z, o[i][2]); o[i][3] = fmaf(p, v0.w, o[i][3]);
+        o[i][4] = fmaf(p, v1.x, o[i][4]); o[i][5] = fmaf(p, v1.y, o[i][5]);
+        o[i][6] = fmaf(p, v1.z, o[i][6]); o[i][7] = fmaf(p, v1.w, o[i][7]);
+      }
+    }
+  }
+  // the warp's four groups, then the warps, then the splits, in a fixed order
+#pragma unroll
+  for (int i = 0; i < FA_NR; ++i) {
+#pragma unroll
+    for (int x = 8; x <= 16; x <<= 1) {
+      const float om = __shfl_xor_sync(0xffffffffu, m[i], x), ol = __shfl_xor_sync(0xffffffffu, l[i], x);
+      const float mx = fmaxf(m[i], om);
+      const float c0 = mx == -INFINITY ? 0.f : expf(m[i] - mx), c1 = mx == -INFINITY ? 0.f : expf(om - mx);
+      m[i] = mx;
+      l[i] = l[i] * c0 + ol * c1;
+#pragma unroll
+      for (int e = 0; e < 8; ++e) o[i][e] = o[i][e] * c0 + __shfl_xor_sync(0xffffffffu, o[i][e], x) * c1;
+    }
+    if (lane < 8) {
+#pragma unroll
+      for (int e = 0; e < 8; ++e) s_o[warp][i][8 * sub + e] = o[i][e];
+      if (lane == 0) {
+        s_m[warp][i] = m[i];
+        s_l[warp][i] = l[i];
+      }
+    }
+  }
   __syncthreads();
-
-  // unnormalised output of the chunk
-  float* part = a.part + (((size_t)b * a.H + h) * a.n_chunks + chunk) * a.k1 * 66;
-  for (int e = tid; e < nr * 64; e += ATTN_THREADS) {
-    const int i = e >> 6, c = e & 63;
-    float o = 0.f;
-    const float* p = S + i * CHUNK;
-    for (int j = 0; j < nk; ++j) o = fmaf(p[j], to_f<T>(Vs[j * 64 + c]), o);
-    part[i * 66 + c] = o;
+  const int i = tid >> 6, c = tid & 63;   // one output column of one row per thread
+  float M = -INFINITY, L = 0.f, ot = 0.f;
+  for (int w = 0; w < 8; ++w) M = fmaxf(M, s_m[w][i]);
+  if (M != -INFINITY)
+    for (int w = 0; w < 8; ++w) {
+      const float f = expf(s_m[w][i] - M);
+      L += s_l[w][i] * f;
+      ot += s_o[w][i][c] * f;
+    }
+  if (S > 1) {
+    p_o[i][c] = ot;
+    if (c == 0) {
+      p_m[i] = M;
+      p_l[i] = L;
+    }
+    cluster_sync();
+    // rank s writes the output columns [64 s / S, 64 (s + 1) / S)
+    const bool mine = c * S / 64 == split;
+    float om[8], ol[8], oo[8];
+#pragma unroll
+    for (int s2 = 0; s2 < 8; ++s2) {
+      om[s2] = -INFINITY;
+      ol[s2] = oo[s2] = 0.f;
+      if (mine && s2 < S) {
+        om[s2] = ld_dsmem_f32(dsmem_addr(&p_m[i], (uint32_t)s2));
+        ol[s2] = ld_dsmem_f32(dsmem_addr(&p_l[i], (uint32_t)s2));
+        oo[s2] = ld_dsmem_f32(dsmem_addr(&p_o[i][c], (uint32_t)s2));
+      }
+    }
+    M = -INFINITY;
+    L = ot = 0.f;
+#pragma unroll
+    for (int s2 = 0; s2 < 8; ++s2) M = fmaxf(M, om[s2]);
+#pragma unroll
+    for (int s2 = 0; s2 < 8; ++s2) {
+      const float f = om[s2] == -INFINITY ? 0.f : expf(om[s2] - M);
+      L += ol[s2] * f;
+      ot += oo[s2] * f;
+    }
+    cluster_sync();   // the peers have read this CTA's partials
+    if (!mine) return;
   }
-  if (tid < nr) {
-    part[tid * 66 + 64] = s_m[tid];
-    part[tid * 66 + 65] = s_l[tid];
-  }
-}
-
-// Merge the chunks of one (row, head) in chunk order.
-__global__ void attn_merge_kernel(AttnArgs a, int chunk_len) {
-  const int i = blockIdx.x, h = blockIdx.y, b = blockIdx.z;
-  const int nr = a.plan.n_utt_rows[b];
   if (i >= nr) return;
-  const int r = a.plan.row_start[b] + i;
-  const int n_keys = a.causal ? a.kv_len[b] + nr : a.enc_len[b];
-  if (bounds_bad(a.status, n_keys > a.t_alloc || n_keys > a.n_chunks * chunk_len)) return;
-  const int nc = (n_keys + chunk_len - 1) / chunk_len;
-  const float* part = a.part + ((size_t)b * a.H + h) * a.n_chunks * a.k1 * 66 + (size_t)i * 66;
-  const size_t cstride = (size_t)a.k1 * 66;
-  float M = -INFINITY;
-  for (int c = 0; c < nc; ++c) M = fmaxf(M, part[c * cstride + 64]);
-  float l = 0.f, o = 0.f;
-  const int cc = threadIdx.x;   // 64 threads, one per output dim
-  for (int c = 0; c < nc; ++c) {
-    const float m_c = part[c * cstride + 64];
-    const float w = (m_c == -INFINITY) ? 0.f : expf(m_c - M);
-    l += part[c * cstride + 65] * w;
-    o += part[c * cstride + cc] * w;
-  }
-  o = o / l;
-  const size_t oi = (size_t)r * a.d + h * 64 + cc;
-  if (a.out_bf16) reinterpret_cast<__nv_bfloat16*>(a.out)[oi] = f2bf(o);
-  else reinterpret_cast<float*>(a.out)[oi] = o;
-  if (a.ml_out && cc == 0) {
-    a.ml_out[((size_t)r * a.H + h) * 2 + 0] = M;
-    a.ml_out[((size_t)r * a.H + h) * 2 + 1] = l;
+  const size_t r = (size_t)(r0 + i);
+  static_cast<float*>(a.out)[r * a.d + h * 64 + c] = ot / L;
+  if (a.ml_out && c == 0) {
+    a.ml_out[(r * a.H + h) * 2 + 0] = M;
+    a.ml_out[(r * a.H + h) * 2 + 1] = L;
   }
 }
 
-template <typename T, int CHUNK>
-static size_t attn_smem() {
-  return (size_t)2 * CHUNK * 64 * sizeof(T) + (size_t)ATTN_MAX_ROWS * 64 * 4 + (size_t)ATTN_MAX_ROWS * CHUNK * 4;
+// Clusters of up to 8 splits while about two CTAs per SM hold them all.
+void launch_attention_f32(const AttnArgs& a0, cudaStream_t st) {
+  AttnArgs a = a0;
+  const int groups = (a.rows_max + FA_NR - 1) / FA_NR;
+  a.splits = 1;
+  while (a.splits < 8 && a.splits * 2 * 64 <= a.t_alloc && a.B * a.H * groups * a.splits * 2 <= 256) a.splits *= 2;
+  launch_ex(attn_f32_kernel, dim3(groups * a.splits, a.H, a.B), dim3(FA_T), 0, st, a.pdl, a.splits, a);
 }
-
-void configure_attention() {
-  static std::once_flag once;
-  std::call_once(once, [] {
-    cudaFuncSetAttribute(attn_chunk_kernel<__nv_bfloat16, 256>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         (int)attn_smem<__nv_bfloat16, 256>());
-    cudaFuncSetAttribute(attn_chunk_kernel<float, 128>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         (int)attn_smem<float, 128>());
-  });
-}
-
-template <typename T, int CHUNK>
-static void launch_attn_t(const AttnArgs& a, cudaStream_t st) {
-  const size_t sm = attn_smem<T, CHUNK>();
-  dim3 grid(a.n_chunks, a.H, a.B);
-  attn_chunk_kernel<T, CHUNK><<<grid, ATTN_THREADS, sm, st>>>(a);
-  dim3 mgrid(a.k1, a.H, a.B);
-  attn_merge_kernel<<<mgrid, 64, 0, st>>>(a, CHUNK);
-}
-
-void launch_attention(const AttnArgs& a, cudaStream_t st) {
-  configure_attention();
-  if (a.kv_bf16) launch_attn_t<__nv_bfloat16, 256>(a, st);
-  else launch_attn_t<float, 128>(a, st);
-}
-
-int attn_chunk_len(int kv_bf16) { return kv_bf16 ? 256 : 128; }
 
 // ---------------------------------------------------------------------------
 // Acceptance, commit and anchor readout, fused

@@ -1,0 +1,337 @@
+// fp32 projections (fp32 models: every product and sum in fp32 FFMA, no TF32).
+//
+// C[m][n] = sum_k A[m][k] B[n][k], both K-major, with the shared epilogues.
+// Two kernels:
+//   * gemm_rows_f32_kernel: the verify rows (A = weights, n = row).  A warp
+//     takes FW weight rows and eight activation rows, its lanes split K (16
+//     bytes each, coalesced), and the sums over lanes are scattered so that
+//     every lane ends with one output.  The activation rows sit in shared
+//     memory, normalised there when the input is a LayerNorm output (one
+//     launch less per projection).  Bound by latency at few rows: the first
+//     384 weights of each row are requested before the wait on the previous
+//     kernel, so what is left is the activations' trip from L2, the sums and
+//     the store; the LM head (80 MB of weights at V = 51865, d = 384) by HBM,
+//     one wave of CTAs that walk the weight rows with the next ones in flight.
+//   * gemm_tile_f32_kernel: 128 x 128 tiles, 8 x 8 outputs per thread, K in
+//     double-buffered slices of 16: the encoder K/V build (thousands of
+//     frames), bound by FFMA issue, and steps of more rows than above.
+// The 64 x 64 tiles with single-buffered 16-deep slices that these replace took
+// 50 us (K = 384) to 200 us (K = 1536) for 5 rows, on 6 to 24 CTAs.
+#include <mutex>
+
+#include "kernels.h"
+
+namespace asrspec {
+
+ASRSPEC_CHECK_SETTER(set_check_gemm_f32)
+
+namespace {
+
+constexpr int FR_NR = 8;        // activation rows per CTA
+constexpr int FR_KC = 3;        // float4 per lane and weight row in a step of 384 k
+constexpr int FR_STEP = FR_KC * 128;
+constexpr int FR_K_MAX = 5120;  // eight activation rows of this K fill 160 KB of shared memory
+
+// FW weight rows per warp; LNF: the activations are LayerNorm(x) of the rows x.
+template <int FW, int MODE, bool LNF>
+__global__ void __launch_bounds__(256)
+gemm_rows_f32_kernel(const float* __restrict__ A, const float* X, int M, int K, Epi epi,
+                     const float* __restrict__ ln_g, const float* __restrict__ ln_b) {
+  constexpr int V = FW * FR_NR;   // sums per warp: 8 (FW 1) or 32 (FW 4)
+  constexpr int SH = FW == 4 ? 0 : 2;
+  extern __shared__ __align__(16) float xs[];   // [FR_NR][K]
+  __shared__ unsigned long long s_key[8][FR_NR];
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int n0 = blockIdx.y * FR_NR;
+  const int tiles = (M + 8 * FW - 1) / (8 * FW), steps = (K + FR_STEP - 1) / FR_STEP;
+  float4 w[2][FW][FR_KC];
+  auto load = [&](int tile, int step, float4 (&d)[FW][FR_KC]) {
+#pragma unroll
+    for (int f = 0; f < FW; ++f) {
+      const int m = min((tile * 8 + warp) * FW + f, M - 1);
+      const float* row = A + (size_t)m * K;
+#pragma unroll
+      for (int c = 0; c < FR_KC; ++c) {
+        const int k = step * FR_STEP + c * 128 + 4 * lane;
+        d[f][c] = k < K ? __ldg(reinterpret_cast<const float4*>(row + k)) : make_float4(0.f, 0.f, 0.f, 0.f);
+      }
+    }
+  };
+  load(blockIdx.x, 0, w[0]);
+  pdl_wait();
+  pdl_launch();
+  const int n_valid = epi.n_valid ? min(*epi.n_valid, epi.N) : epi.N;
+  if (n0 >= n_valid) return;   // uniform over the CTA
+  const int nr = min(FR_NR, n_valid - n0), k4 = K >> 2;
+  // this lane's output: weight row f, activation row r of the warp's V sums
+  const int idx = lane >> SH, f_own = idx / FR_NR, r_own = idx % FR_NR;
+  const bool writer = (lane & ((1 << SH) - 1)) == 0;
+  int m_own = (blockIdx.x * 8 + warp) * FW + f_own;
+  const int n_own = n0 + r_own;
+  bool ok = writer && m_own < M && r_own < nr;
+  EpiPre<MODE, 1> pre;
+  if constexpr (MODE != EPI_ARGMAX) epi_load<MODE, 1>(epi, &m_own, &n_own, &ok, pre);
+  for (int e = tid; e < FR_NR * k4; e += 256) {
+    const int r = e / k4, c = e - r * k4;
+    reinterpret_cast<float4*>(xs)[e] = r < nr ? reinterpret_cast<const float4*>(X + (size_t)(n0 + r) * K)[c]
+                                              : make_float4(0.f, 0.f, 0.f, 0.f);
+  }
+  if constexpr (LNF) {   // warp r normalises row r in place
+    __syncthreads();
+    if (warp < nr) {
+      float4* xr = reinterpret_cast<float4*>(xs + warp * K);
+      float s = 0.f;
+      for (int c = lane; c < k4; c += 32) {
+        const float4 v = xr[c];
+        s += (v.x + v.y) + (v.z + v.w);
+      }
+      const float mean = warp_sum(s) / (float)K;
+      float q = 0.f;
+      for (int c = lane; c < k4; c += 32) {
+        const float4 v = xr[c];
+        const float a = v.x - mean, b = v.y - mean, g = v.z - mean, h = v.w - mean;
+        q += (a * a + b * b) + (g * g + h * h);
+      }
+      const float rstd = rsqrtf(warp_sum(q) / (float)K + 1e-5f);
+      for (int c = lane; c < k4; c += 32) {
+        const float4 v = xr[c], gg = __ldg(reinterpret_cast<const float4*>(ln_g) + c),
+                     bb = __ldg(reinterpret_cast<const float4*>(ln_b) + c);
+        xr[c] = make_float4((v.x - mean) * rstd * gg.x + bb.x, (v.y - mean) * rstd * gg.y + bb.y,
+                            (v.z - mean) * rstd * gg.z + bb.z, (v.w - mean) * rstd * gg.w + bb.w);
+      }
+    }
+  }
+  __syncthreads();
+  float acc[V];
+#pragma unroll
+  for (int i = 0; i < V; ++i) acc[i] = 0.f;
+  unsigned long long best = 0;
+  int tile = blockIdx.x, step = 0, buf = 0;
+  while (tile < tiles) {
+    int nt = tile, ns = step + 1;
+    if (ns == steps) {
+      ns = 0;
+      nt += gridDim.x;
+    }
+    auto go = [&](float4 (&cur)[FW][FR_KC], float4 (&nxt)[FW][FR_KC]) {
+      if (nt < tiles) load(nt, ns, nxt);
+#pragma unroll
+      for (int c = 0; c < FR_KC; ++c) {
+        const int k = step * FR_STEP + c * 128 + 4 * lane;
+        if (k < K) {
+#pragma unroll
+          for (int r = 0; r < FR_NR; ++r) {
+            const float4 xv = *reinterpret_cast<const float4*>(xs + r * K + k);
+#pragma unroll
+            for (int f = 0; f < FW; ++f) {
+              float& a = acc[f * FR_NR + r];
+              a = fmaf(cur[f][c].x, xv.x, a);
+              a = fmaf(cur[f][c].y, xv.y, a);
+              a = fmaf(cur[f][c].z, xv.z, a);
+              a = fmaf(cur[f][c].w, xv.w, a);
+            }
+          }
+        }
+      }
+    };
+    if (buf == 0) go(w[0], w[1]);
+    else go(w[1], w[0]);
+    buf ^= 1;
+    if (ns == 0) {   // the tile's sums are complete: scatter-reduce over the lanes
+#pragma unroll
+      for (int n = V, o = 16; n > 1; n >>= 1, o >>= 1) {
+        const bool up = lane & o;
+#pragma unroll
+        for (int i = 0; i < n / 2; ++i) {
+          const float send = up ? acc[i] : acc[i + n / 2], keep = up ? acc[i + n / 2] : acc[i];
+          acc[i] = keep + __shfl_xor_sync(0xffffffffu, send, o);
+        }
+      }
+      float val = acc[0];
+#pragma unroll
+      for (int o = (1 << SH) >> 1; o > 0; o >>= 1) val += __shfl_xor_sync(0xffffffffu, val, o);
+      m_own = (tile * 8 + warp) * FW + f_own;
+      if constexpr (MODE == EPI_ARGMAX) {
+        if (m_own < M) {
+          const unsigned long long key = argmax_key(val, (uint32_t)m_own);
+          best = key > best ? key : best;
+        }
+      } else {   // one tile per CTA (the launch), so the operands loaded above are this output's
+        epi_store<MODE, 1>(epi, &m_own, &n_own, &val, &ok, pre);
+      }
+#pragma unroll
+      for (int i = 0; i < V; ++i) acc[i] = 0.f;
+    }
+    tile = nt;
+    step = ns;
+  }
+  if constexpr (MODE == EPI_ARGMAX) {   // lanes of one activation row, then the warps
+#pragma unroll
+    for (int o = 8 << SH; o < 32; o <<= 1) {
+      const unsigned long long k = __shfl_xor_sync(0xffffffffu, best, o);
+      best = k > best ? k : best;
+    }
+    if (lane < (8 << SH) && writer) s_key[warp][r_own] = best;
+    __syncthreads();
+    if (tid < nr) {
+      unsigned long long k = s_key[0][tid];
+      for (int v = 1; v < 8; ++v) k = s_key[v][tid] > k ? s_key[v][tid] : k;
+      atomicMax(epi.row_key + n0 + tid, k);
+    }
+  }
+}
+
+constexpr int FT_B = 128, FT_K = 16, FT_LD = FT_B + 4;
+
+template <int MODE>
+__global__ void __launch_bounds__(256, 2)
+gemm_tile_f32_kernel(const float* __restrict__ A, const float* __restrict__ B, int M, int N, int K, Epi epi) {
+  __shared__ __align__(16) float As[2][FT_K][FT_LD], Bs[2][FT_K][FT_LD];
+  const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
+  const int m0 = blockIdx.y * FT_B, n0 = blockIdx.x * FT_B;
+  const int n_valid = epi.n_valid ? min(*epi.n_valid, N) : N;
+  if (n0 >= n_valid) return;
+  if constexpr (MODE == EPI_CROSSKV) {   // every frame of the tile is padding
+    bool dead = true;
+    for (int mr = m0; mr < m0 + FT_B && mr < M;) {
+      const int b = mr / epi.t_max, t = mr - b * epi.t_max;
+      if (t < epi.enc_len[b]) {
+        dead = false;
+        break;
+      }
+      mr = (b + 1) * epi.t_max;
+    }
+    if (dead) return;
+  }
+  // 128 rows x 16 k of each operand: two float4 per thread
+  float4 ra[2], rb[2];
+  auto load = [&](int k0) {
+#pragma unroll
+    for (int u = 0; u < 2; ++u) {
+      const int e = tid + 256 * u, r = e >> 2, k = k0 + 4 * (e & 3);
+      const float4 z = make_float4(0.f, 0.f, 0.f, 0.f);
+      ra[u] = m0 + r < M ? __ldg(reinterpret_cast<const float4*>(A + (size_t)(m0 + r) * K + k)) : z;
+      rb[u] = n0 + r < n_valid ? *reinterpret_cast<const float4*>(B + (size_t)(n0 + r) * K + k) : z;
+    }
+  };
+  auto stage = [&](int s) {
+#pragma unroll
+    for (int u = 0; u < 2; ++u) {
+      const int e = tid + 256 * u, r = e >> 2, k = 4 * (e & 3);
+      As[s][k][r] = ra[u].x; As[s][k + 1][r] = ra[u].y; As[s][k + 2][r] = ra[u].z; As[s][k + 3][r] = ra[u].w;
+      Bs[s][k][r] = rb[u].x; Bs[s][k + 1][r] = rb[u].y; Bs[s][k + 2][r] = rb[u].z; Bs[s][k + 3][r] = rb[u].w;
+    }
+  };
+  float acc[8][8];
+#pragma unroll
+  for (int i = 0; i < 8; ++i)
+#pragma unroll
+    for (int j = 0; j < 8; ++j) acc[i][j] = 0.f;
+  load(0);
+  stage(0);
+  __syncthreads();
+  const int nk = K / FT_K;
+  for (int it = 0; it < nk; ++it) {
+    const int s = it & 1;
+    if (it + 1 < nk) load((it + 1) * FT_K);
+#pragma unroll
+    for (int k = 0; k < FT_K; ++k) {
+      float a[8], b[8];   // m: ty 4 + {0..3}, 64 + ..; n: tx 4 + {0..3}, 64 + ..
+      *reinterpret_cast<float4*>(a) = *reinterpret_cast<const float4*>(&As[s][k][4 * ty]);
+      *reinterpret_cast<float4*>(a + 4) = *reinterpret_cast<const float4*>(&As[s][k][64 + 4 * ty]);
+      *reinterpret_cast<float4*>(b) = *reinterpret_cast<const float4*>(&Bs[s][k][4 * tx]);
+      *reinterpret_cast<float4*>(b + 4) = *reinterpret_cast<const float4*>(&Bs[s][k][64 + 4 * tx]);
+#pragma unroll
+      for (int i = 0; i < 8; ++i)
+#pragma unroll
+        for (int j = 0; j < 8; ++j) acc[i][j] = fmaf(a[i], b[j], acc[i][j]);
+    }
+    if (it + 1 < nk) stage(s ^ 1);
+    __syncthreads();
+  }
+#pragma unroll
+  for (int i = 0; i < 8; ++i) {
+    const int m = m0 + (i >> 2) * 64 + 4 * ty + (i & 3);
+    if constexpr (MODE == EPI_CROSSKV) {
+      if (m >= M) continue;
+      const int b = m / epi.t_max, t = m - b * epi.t_max;
+      if (bounds_bad(epi.status, b >= epi.b_max || t >= epi.max_enc) || t >= epi.enc_len[b]) continue;
+#pragma unroll
+      for (int q = 0; q < 2; ++q) {   // four consecutive features lie in one head: one 16-byte store
+        const int n = n0 + 64 * q + 4 * tx;
+        if (n >= n_valid) continue;
+        const int two_d = 2 * epi.d, l = n / two_d, r = n - l * two_d, which = r / epi.d, f = r - which * epi.d;
+        const size_t o = (((((size_t)l * 2 + which) * epi.b_max + b) * epi.n_heads + (f >> 6)) * epi.max_enc + t) * 64 +
+                         (f & 63);
+        const float4 bi = __ldg(reinterpret_cast<const float4*>(epi.bias + n));
+        *reinterpret_cast<float4*>(static_cast<float*>(epi.kcache) + o) =
+            make_float4(acc[i][4 * q] + bi.x, acc[i][4 * q + 1] + bi.y, acc[i][4 * q + 2] + bi.z,
+                        acc[i][4 * q + 3] + bi.w);
+      }
+    } else {
+#pragma unroll
+      for (int j = 0; j < 8; ++j) {
+        const int n = n0 + (j >> 2) * 64 + 4 * tx + (j & 3);
+        if (m >= M || n >= n_valid) continue;
+        if constexpr (MODE == EPI_ARGMAX) atomicMax(epi.row_key + n, argmax_key(acc[i][j], (uint32_t)m));
+        else epi_apply<MODE>(epi, m, n, acc[i][j]);
+      }
+    }
+  }
+}
+
+template <int FW, int MODE, bool LNF>
+void launch_rows_t(const F32Gemm& g, const Epi& epi, cudaStream_t st) {
+  static std::once_flag once;
+  std::call_once(once, [] {
+    cudaFuncSetAttribute(gemm_rows_f32_kernel<FW, MODE, LNF>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                         FR_NR * FR_K_MAX * 4);
+  });
+  int gx = (g.M + 8 * FW - 1) / (8 * FW);
+  if (MODE == EPI_ARGMAX) gx = gx < 2 * g.sms ? gx : 2 * g.sms;   // a wave; each CTA walks the weight rows
+  launch_ex(gemm_rows_f32_kernel<FW, MODE, LNF>, dim3(gx, (g.N + FR_NR - 1) / FR_NR), dim3(256),
+            (size_t)FR_NR * g.K * 4, st, g.pdl, 1, g.A, g.B, g.M, g.K, epi, g.ln_g, g.ln_b);
+}
+
+template <int MODE>
+void launch_mode(const F32Gemm& g, const Epi& epi, cudaStream_t st) {
+  if constexpr (MODE != EPI_CROSSKV) {
+    if (f32_rows(g.N, g.K)) {
+      // four weight rows per warp where that still gives every SM a CTA (each
+      // activation read from shared memory then serves four)
+      const bool wide = (g.M / 32) * ((g.N + FR_NR - 1) / FR_NR) >= g.sms;
+      if (g.ln_g) {
+        if (wide) launch_rows_t<4, MODE, true>(g, epi, st);
+        else launch_rows_t<1, MODE, true>(g, epi, st);
+      } else {
+        if (wide) launch_rows_t<4, MODE, false>(g, epi, st);
+        else launch_rows_t<1, MODE, false>(g, epi, st);
+      }
+      return;
+    }
+  }
+  gemm_tile_f32_kernel<MODE><<<dim3((g.N + FT_B - 1) / FT_B, (g.M + FT_B - 1) / FT_B), 256, 0, st>>>(
+      g.A, g.B, g.M, g.N, g.K, epi);
+}
+
+}  // namespace
+
+// Up to 512 rows the row kernel (34 groups of eight rows re-read the weights
+// from L2 at 272 rows); past that, or for K that does not fit shared memory,
+// tiles.
+bool f32_rows(int N, int K) { return N <= 512 && K <= FR_K_MAX; }
+
+void launch_gemm_f32(const F32Gemm& g, int mode, const Epi& epi, cudaStream_t st) {
+  switch (mode) {
+    case EPI_F32: launch_mode<EPI_F32>(g, epi, st); break;
+    case EPI_QKV: launch_mode<EPI_QKV>(g, epi, st); break;
+    case EPI_RESID: launch_mode<EPI_RESID>(g, epi, st); break;
+    case EPI_Q: launch_mode<EPI_Q>(g, epi, st); break;
+    case EPI_GELU: launch_mode<EPI_GELU>(g, epi, st); break;
+    case EPI_CROSSKV: launch_mode<EPI_CROSSKV>(g, epi, st); break;
+    case EPI_ARGMAX: launch_mode<EPI_ARGMAX>(g, epi, st); break;
+    default: break;
+  }
+}
+
+}  // namespace asrspec

@@ -47,12 +47,23 @@ struct WideGemm {
 bool wide_pick(int M, int N, int K, int mode, int sms, int* bn, int* split);
 void launch_gemm_wide(const WideGemm& g, int mode, const Epi& epi, int* status, cudaStream_t st);
 void configure_gemm_tc();
-void configure_attention();
+void configure_attention_tc();
 
-// SIMT path (fp32 models, and a cross-check of the tensor-core path).
-// A: [M][K] of type a_bf16 ? bf16 : fp32; B: [N][K] likewise.
-void launch_gemm_simt(const void* A, int a_bf16, const void* B, int b_bf16, int M, int N, int K, int mode,
-                      const Epi& epi, cudaStream_t st);
+// fp32 models (csrc/gemm_f32.cu): A [M][K], B [N][K] fp32, K % 64 == 0.  With
+// ln_g set (row kernel only, f32_rows) B holds the rows x and the operand is
+// LayerNorm(x).
+struct F32Gemm {
+  const float *A, *B;
+  int M, N, K;
+  const float *ln_g = nullptr, *ln_b = nullptr;
+  int sms = 0;
+  bool pdl = false;
+};
+bool f32_rows(int N, int K);
+void launch_gemm_f32(const F32Gemm& g, int mode, const Epi& epi, cudaStream_t st);
+
+// SIMT cross-check of the tensor-core GEMM (tests): C [M][N] fp32 of bf16 A, B.
+void launch_gemm_simt(const void* A, const void* B, int M, int N, int K, float* C, cudaStream_t st);
 
 // ---- Row bookkeeping, embedding, LayerNorm ---------------------------------
 struct RowPlan {
@@ -110,9 +121,6 @@ struct AttnArgs {
   const int* kv_len;       // [B_max] committed lengths (self; keys up to kv_len + i)
   RowPlan plan;
   int B, H, d, k1;         // utterances, heads, d_model, rows per utterance slot (k + 1)
-  int chunk;               // keys per split
-  int n_chunks;            // splits per (b, h)
-  float* part;             // [B][H][n_chunks][k1] x (64 + 2) partials
   void* out;               // [R][d] attention output (bf16 or fp32)
   int out_bf16;
   float* ml_out;           // optional [R][H][2] (max, sum) of the full softmax
@@ -130,7 +138,7 @@ struct AttnArgs {
   unsigned long long* tl = nullptr;   // launch timeline slot (tl_mark), or null
   int* status = nullptr;   // device status word (bounds-check mode)
 };
-void launch_attention(const AttnArgs& a, cudaStream_t st);
+void launch_attention_f32(const AttnArgs& a, cudaStream_t st);   // fp32 caches
 void launch_attention_tc(const AttnArgs& a, int* status, cudaStream_t st);
 // Tensor map over a [rows][64] bf16 cache with `box_rows`-row boxes.
 bool make_tmap_cache(CUtensorMap* map, const void* base, uint64_t rows, uint32_t box_rows);
@@ -298,11 +306,10 @@ void launch_synth_drafts(const int* truth, const int* total_len, const int* repl
                          int B, int max_pos, const int* kv_len, int* draft_out, int* lens_out, cudaStream_t st);
 void launch_mark_ready(const int* enc_len, int B, int t_max, int* ready, int* kv_len, int* pending, int* status,
                        cudaStream_t st);
-int attn_chunk_len(int kv_bf16);
 
 // Bounds-check mode switches, one per translation unit (see bounds_bad).
 void set_check_gemm_tc(int on);
-void set_check_gemm_simt(int on);
+void set_check_gemm_f32(int on);
 void set_check_gemm_wide(int on);
 void set_check_rows(int on);
 void set_check_attention(int on);

@@ -110,6 +110,29 @@ def test_edge_cases_fp32(built_lib, cuda):
     assert st.near_ties == 0
 
 
+@pytest.mark.parametrize("d,heads,ffn,vocab,batch,k,t_max", [
+    (192, 3, 576, 301, 2, 8, 129),     # nine rows: a second group of one; K below one 384-wide step, F above it
+    (448, 7, 1792, 1001, 3, 16, 300),  # 51 rows; K not a multiple of the step
+    (64, 1, 64, 97, 33, 15, 70),       # 528 rows: the tile kernel, LayerNorm as its own launch
+])
+def test_fp32_projection_and_attention_sizes(built_lib, cuda, d, heads, ffn, vocab, batch, k, t_max):
+    """fp32 row kernel (groups of eight rows, K steps of 384, one or four
+    weight rows per warp), tile kernel and split attention at their edges."""
+    dims = W.ModelDims(n_layers=2, d_model=d, n_heads=heads, d_ffn=ffn, vocab=vocab, dtype="fp32",
+                       max_pos=40, max_enc=t_max, anchor_layer=1)
+    blob = _blob(dims, 0.1)
+    enc_lens = [t_max if b == 0 else 1 + (b * 37) % t_max for b in range(batch)]
+    enc = W.make_encoder_states(dims, enc_lens, t_max)
+    prompt = W.make_prompt(dims, batch)
+    total = [W.PROMPT_LEN + 6 + b % 9 for b in range(batch)]
+    wl = W.Workload("f", dims, batch, k, tuple(t - W.PROMPT_LEN for t in total), tuple(enc_lens), (0.2,) * batch, "half")
+    st, _ = run_decode(dims, blob, enc, enc_lens, prompt, total, k, W.make_corruption(wl),
+                       _session(dims, blob, batch, k))
+    _report(f"fp32 d{d} b{batch} k{k}", st)
+    assert st.emitted == sum(wl.n_out)
+    assert_bounded(st)
+
+
 @pytest.mark.slow
 def test_large_bf16_batch1_full_decode(built_lib, cuda):
     """Full-size large decoder, batch 1, k = 8 with a slip every round: the
