@@ -14,7 +14,12 @@ using namespace asrspec;
 
 namespace {
 
-constexpr int NUM_SMS_TARGET = 152;
+// Rows that one prefill step may lay out (prompt tokens of all utterances):
+// the work buffers hold at least as many.  A step costs what its launches and
+// one pass over the weights cost, whatever its rows, up to a few hundred: four
+// utterances of 202 tokens (small decoder) took 26 steps of k + 1 = 8 tokens,
+// 0.5 ms each.
+constexpr int PREFILL_ROWS = 1024;
 
 struct LayerW {
   void *wqkv, *wo, *wcq, *wco, *w1, *w2;
@@ -159,7 +164,7 @@ struct asr_spec {
   unsigned long long* d_row_key = nullptr;
   bool d_after_verify = false;
   float d_threshold = 0.f;            // confidence threshold of the proposals (0 = off)
-  float* d_logits = nullptr;          // threshold on: the pass's logits [R_pad][V]
+  float* d_logits = nullptr;          // threshold on: the pass's logits [R_max][V]
   float* d_row_p = nullptr;           // threshold on: [R_pad] probability of each row's argmax
   int last_k = 0;   // k of the last linear verification (stride of its drafts)
 };
@@ -419,10 +424,11 @@ int gemm_rows_ln(asr_spec* h, const void* W, const CUtensorMap* mW, int M, int K
 // 128-key chunk of the four that 448 positions have) do not pay for the merge
 // until a CTA would have more than eight chunks: 3.4 us unsplit against 5.0
 // and 8.5 in two and four at 60 keys, and each further chunk costs 0.9 us.
-int attn_splits_for(asr_spec* h, int t_alloc, bool self_attn) {
+// utts: utterances, or segments of their rows.
+int attn_splits_for(asr_spec* h, int utts, int t_alloc, bool self_attn) {
   const int nc_max = (t_alloc + 127) / 128;
   int S = 1;
-  while (S < 8 && S * (self_attn ? 16 : 2) <= nc_max && h->B * h->H * S * 2 <= 200) S *= 2;
+  while (S < 8 && S * (self_attn ? 16 : 2) <= nc_max && utts * h->H * S * 2 <= 200) S *= 2;
   return S;
 }
 
@@ -432,7 +438,8 @@ void attention(asr_spec* h, AttnArgs& a, bool self_attn, int layer) {
     launch_attention_f32(a, h->st);
     return;
   }
-  a.splits = attn_splits_for(h, a.t_alloc, self_attn);
+  a.segs = (a.rows_max + 31) / 32;
+  a.splits = attn_splits_for(h, h->B * a.segs, a.t_alloc, self_attn);
   const int ci = 0;   // 128-row boxes
   if (self_attn) {
     a.kmap = &h->m_kself[ci];
@@ -462,7 +469,10 @@ int tap_copy(asr_spec* h, int l, int rows) {
   return 0;
 }
 
-int run_layers(asr_spec* h, int N) {
+// prefill: only the K/V of the rows are wanted, so the last layer ends with
+// its QKV projection (with a draft, which reads the last layer's output, it
+// runs whole).
+int run_layers(asr_spec* h, int N, bool prefill = false) {
   const int rows_max = N / std::max(h->B, 1);
   const int d = h->d;
   Epi base{};
@@ -512,6 +522,7 @@ int run_layers(asr_spec* h, int N) {
     if (int rc = gemm_rows_ln(h, w.wqkv, &w.m_wqkv, 3 * d, d, w.ln1g, w.ln1b, w.c1_qkv, w.c2_qkv, h->xn, BUF_XN, N,
                               EPI_QKV, e))
       return rc;
+    if (prefill && l + 1 == h->L && !h->has_draft) return 0;
     AttnArgs a{};
     a.status = h->status;
     a.q = h->q;
@@ -526,7 +537,6 @@ int run_layers(asr_spec* h, int N) {
     a.B = h->B;
     a.H = h->H;
     a.d = d;
-    a.k1 = h->kmax + 1;
     a.out = h->att;
     a.out_bf16 = h->bf16;
     a.ml_out = nullptr;
@@ -1148,7 +1158,7 @@ int asr_spec_create(const asr_model_dims* dims, const asr_weights* weights, void
 
   // work buffers
   h->R_max = h->Bmax * (h->kmax + 1);
-  h->R_pad = ((h->R_max + 255) / 256) * 256;
+  h->R_pad = ((std::max(h->R_max, PREFILL_ROWS) + 255) / 256) * 256;
   const size_t R = h->R_pad;
   if ((rc = dalloc(h, &h->x, R * d * 4)) || (rc = dalloc(h, &h->q, R * d * 4)) ||
       (rc = dalloc(h, &h->q_anchor, R * d * 4)) || (rc = dalloc(h, &h->ml, R * h->H * 2 * 4)) ||
@@ -1321,14 +1331,14 @@ int asr_spec_prefill(asr_spec_handle h, const int32_t* prompt, int32_t P0) {
     CK(cudaMemsetAsync(h->d_last_tap, 0, (size_t)h->Bmax * 4 * h->d * 4, h->st));
     h->d_after_verify = false;
   }
-  const int c_max = h->kmax + 1;
+  const int c_max = h->R_pad / h->B;   // tokens per utterance and step
   for (int p0 = 0; p0 < P0 - 1; p0 += c_max) {
     const int c = std::min(c_max, P0 - 1 - p0);
     {
       Prof p(h, ASR_PROF_OTHER, 1);
       launch_plan_prefill_chunk(h->prompt_buf, P0, p0, c, h->B, h->V, h->ready, h->plan, h->status, h->st);
     }
-    if (int rc = run_layers(h, h->B * c)) return rc;
+    if (int rc = run_layers(h, h->B * c, true)) return rc;
     if (h->has_draft) {   // the draft's cache of the same prompt rows (their taps as its inputs)
       DraftArgs A{};
       A.B = h->B;
@@ -1659,7 +1669,7 @@ int asr_spec_draft_set_threshold(asr_spec_handle h, float threshold) {
   if (!h->has_draft) return fail(h, ASR_E_STATE, "no draft (asr_spec_draft_create)");
   if (!(threshold >= 0.f && threshold <= 1.f)) return fail(h, ASR_E_INVAL, "threshold outside [0, 1]");
   if (threshold > 0.f && !h->d_logits) {
-    if (int rc = dalloc(h, &h->d_logits, (size_t)h->R_pad * h->V * 4)) return rc;
+    if (int rc = dalloc(h, &h->d_logits, (size_t)h->R_max * h->V * 4)) return rc;
     if (int rc = dalloc(h, &h->d_row_p, (size_t)h->R_pad * 4)) return rc;
   }
   h->d_threshold = threshold;

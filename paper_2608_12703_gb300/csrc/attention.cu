@@ -74,7 +74,7 @@ __global__ void __launch_bounds__(FA_T) attn_f32_kernel(AttnArgs a) {
   pdl_wait();
   pdl_launch();
   const int n_rows = a.plan.n_utt_rows[b], nr = min(FA_NR, n_rows - i0);
-  const int n_keys = a.causal ? a.kv_len[b] + n_rows : a.enc_len[b];
+  const int n_keys = a.causal ? a.kv_len[b] + i0 + nr : a.enc_len[b];   // up to the group's last row
   if (nr <= 0 || bounds_bad(a.status, n_keys > a.t_alloc)) return;   // uniform over the cluster
   if (!loaded) range(n_keys);
   const int r0 = a.plan.row_start[b] + i0;

@@ -96,16 +96,18 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap kmap, const __grid_constant__
   __shared__ __align__(8) uint64_t bar[TCA_STAGES];
   __shared__ __align__(8) uint64_t rbar;   // PUSH: the other splits' partials have landed
 
-  const int S = gridDim.x, split = blockIdx.x, h = blockIdx.y, b = blockIdx.z;
+  // utterance and, where a prefill step gives one more rows than the m-tiles hold, segment of its rows
+  const int S = gridDim.x, split = blockIdx.x, h = blockIdx.y, b = blockIdx.z / a.segs;
+  const int s0 = (int)(blockIdx.z % a.segs) * MT * 16;
   tl_mark(a.tl, TL_ENTRY);
-  const int nr = a.plan.n_utt_rows[b];
-  if (nr == 0) {                             // uniform over the cluster
+  const int nr_all = a.plan.n_utt_rows[b], nr = min(nr_all - s0, MT * 16);
+  if (nr <= 0) {                             // uniform over the cluster
     pdl_wait();
     return;
   }
-  const int row0 = a.plan.row_start[b];
-  const int n_keys = a.causal ? a.kv_len[b] + nr : a.enc_len[b];
-  if (bounds_bad(status, n_keys > a.t_alloc || nr > a.rows_max)) {   // uniform over the cluster
+  const int row0 = a.plan.row_start[b] + s0;
+  const int n_keys = a.causal ? a.kv_len[b] + s0 + nr : a.enc_len[b];
+  if (bounds_bad(status, n_keys > a.t_alloc || nr_all > a.rows_max)) {   // uniform over the cluster
     pdl_wait();
     return;
   }
@@ -409,7 +411,7 @@ void configure_attention_tc() {
 
 template <int MT, int ST, bool PUSH, bool TREE = false>
 static void launch_one(const AttnArgs& a, int splits, int* status, cudaStream_t st) {
-  launch_ex(attn_tc_kernel<MT, ST, PUSH, TREE>, dim3(splits, a.H, a.B), dim3(TCA_THREADS), TcaCfg<MT, ST, PUSH>::SMEM,
+  launch_ex(attn_tc_kernel<MT, ST, PUSH, TREE>, dim3(splits, a.H, a.B * a.segs), dim3(TCA_THREADS), TcaCfg<MT, ST, PUSH>::SMEM,
             st, a.pdl, splits, *a.kmap, *a.vmap, a, status);
 }
 

@@ -120,7 +120,7 @@ struct AttnArgs {
   const int* enc_len;      // [B_max] (cross)
   const int* kv_len;       // [B_max] committed lengths (self; keys up to kv_len + i)
   RowPlan plan;
-  int B, H, d, k1;         // utterances, heads, d_model, rows per utterance slot (k + 1)
+  int B, H, d;             // utterances, heads, d_model
   void* out;               // [R][d] attention output (bf16 or fp32)
   int out_bf16;
   float* ml_out;           // optional [R][H][2] (max, sum) of the full softmax
@@ -132,6 +132,7 @@ struct AttnArgs {
   long long k_row0 = 0, v_row0 = 0;
   int* tickets = nullptr;
   int rows_max = 0;        // most rows of one utterance in this call
+  int segs = 1;            // tensor-core path: segments of 32 rows per utterance (1 up to 32 rows)
   int splits = 1;          // CTAs (one cluster) per (utterance, head)
   bool pdl = false;        // programmatic dependent launch
   bool tree = false;       // self-attention of a tree verify: slots past kv_len visible by plan.row_mask

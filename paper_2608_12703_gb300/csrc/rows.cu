@@ -136,34 +136,30 @@ plan_prefill_kernel(const int* __restrict__ prompt, int P0, int p0, int c, int B
   __syncthreads();
   const int b = threadIdx.x;
   int err = 0;
-  if (b < B) {
-    if (!ready[b]) err |= ST_NOT_READY;
-    for (int i = 0; i < P0; ++i) {
-      const int t = prompt[(size_t)b * P0 + i];
-      if (t < 0 || t >= vocab) err |= ST_BAD_TOKEN;
-    }
+  if (b < B && !ready[b]) err |= ST_NOT_READY;
+  for (int e = threadIdx.x; e < B * P0; e += PLAN_THREADS) {   // a prompt has up to max_pos tokens
+    const int t = prompt[e];
+    if (t < 0 || t >= vocab) err |= ST_BAD_TOKEN;
   }
   if (err) atomicOr(&s_err, err);
   __syncthreads();
-  const int n_b = (b < B && !s_err) ? c : 0;
+  const int n_b = s_err ? 0 : c;
   if (s_err && threadIdx.x == 0) set_status(status, s_err);
-  int total;
-  const int start = block_excl_scan(n_b, &total);
   if (b < B) {
-    plan.row_start[b] = start;
+    plan.row_start[b] = b * n_b;
     plan.n_utt_rows[b] = n_b;
-    for (int i = 0; i < n_b; ++i) {
-      const int r = start + i;
-      plan.row_b[r] = b;
-      plan.row_i[r] = i;
-      plan.row_pos[r] = p0 + i;
-      plan.row_epos[r] = p0 + i;
-      plan.row_tok[r] = prompt[(size_t)b * P0 + p0 + i];
-    }
+  }
+  for (int r = threadIdx.x; r < B * n_b; r += PLAN_THREADS) {
+    const int u = r / c, i = r - u * c;
+    plan.row_b[r] = u;
+    plan.row_i[r] = i;
+    plan.row_pos[r] = p0 + i;
+    plan.row_epos[r] = p0 + i;
+    plan.row_tok[r] = prompt[(size_t)u * P0 + p0 + i];
   }
   if (threadIdx.x == 0) {
-    plan.row_start[B] = total;
-    *plan.n_rows = total;
+    plan.row_start[B] = B * n_b;
+    *plan.n_rows = B * n_b;
   }
 }
 

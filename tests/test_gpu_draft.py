@@ -217,6 +217,13 @@ def test_draft_attention_edges(built_lib, cuda, k):
     _check(f"attention edges k{k}", st, ds, seqs, truth, total)
 
 
+def test_draft_long_prompt(built_lib, cuda):
+    """A prompt of 41 tokens: its 40 rows in one prefill step, ten groups of the draft's attention."""
+    total = [41 + n for n in (12, 9)]
+    st, ds, seqs, truth, _ = run_lockstep([90, 200], total, 4, "anchor", prompt_len=41)
+    _check("long prompt", st, ds, seqs, truth, total)
+
+
 def test_draft_edges(built_lib, cuda):
     """A one-token prompt (zero representations for the first restart), k = 0
     rounds between full ones, an utterance whose only round offers no draft

@@ -133,6 +133,27 @@ def test_fp32_projection_and_attention_sizes(built_lib, cuda, d, heads, ffn, voc
     assert_bounded(st)
 
 
+@pytest.mark.parametrize("dtype,batch,prompt_len", [
+    ("bf16", 2, 33), ("bf16", 2, 34), ("bf16", 1, 66), ("bf16", 40, 28), ("fp32", 2, 35), ("fp32", 30, 40)])
+def test_prompt_lengths(built_lib, cuda, dtype, batch, prompt_len):
+    """Prompts in one prefill step or several (1024 rows a step), with one
+    segment of 32 rows per utterance in the attention or more, and a segment
+    of a single row; the last layer of a prefill stops at its K/V."""
+    dims = W.ModelDims(n_layers=2, d_model=128, n_heads=2, d_ffn=512, vocab=500, dtype=dtype,
+                       max_pos=90, max_enc=150, anchor_layer=1)
+    blob = _blob(dims, 0.1)
+    enc_lens = [150 - (b * 41) % 149 for b in range(batch)]
+    enc = W.make_encoder_states(dims, enc_lens, 150)
+    prompt = W.make_prompt(dims, batch, length=prompt_len)
+    total = [prompt_len + 5 + b % 4 for b in range(batch)]
+    wl = W.Workload("p", dims, batch, 3, tuple(t - prompt_len for t in total), tuple(enc_lens), (0.3,) * batch, "half")
+    st, _ = run_decode(dims, blob, enc, enc_lens, prompt, total, 3, W.make_corruption(wl),
+                       _session(dims, blob, batch, 3), scale=scale_for(dims, 0.1))
+    _report(f"{dtype} b{batch} prompt {prompt_len}", st)
+    assert st.emitted == sum(wl.n_out)
+    assert_bounded(st)
+
+
 @pytest.mark.slow
 def test_large_bf16_batch1_full_decode(built_lib, cuda):
     """Full-size large decoder, batch 1, k = 8 with a slip every round: the
