@@ -132,7 +132,8 @@ struct asr_spec {
   int wide_bn = 64;      // N tile for many rows (ASRSPEC_WIDE_BN: 64, 128, 192, 224, 256)
   int wide_target = 2 * 152;   // CTAs a many-row GEMM may fill by splitting K (ASRSPEC_WIDE_TARGET)
   int few_target = 2 * 152;    // the same for few rows (ASRSPEC_FEW_TARGET)
-  // encoder-cache GEMM: N tile (ASRSPEC_ENC_BN) and M tiles per band of the
+  bool enc_pair = true;   // encoder-cache GEMM on CTA pairs (ASRSPEC_ENC_PAIR=0: one CTA per tile)
+  // encoder cache, one CTA per tile: N tile (ASRSPEC_ENC_BN) and M tiles per band of the
   // grouped order (ASRSPEC_ENC_GROUP, 0 = plain); measured at 64 utterances x
   // 1500 frames: 14.5 ms (128, 64) against 16.7 (256, 32) and 23.6 (256, plain)
   int enc_bn = 128;
@@ -983,6 +984,7 @@ int asr_spec_create(const asr_model_dims* dims, const asr_weights* weights, void
     set_check_gemm_tc(on);
     set_check_gemm_f32(on);
     set_check_gemm_wide(on);
+    set_check_gemm_pair(on);
     set_check_rows(on);
     set_check_attention(on);
     set_check_attention_tc(on);
@@ -1000,6 +1002,7 @@ int asr_spec_create(const asr_model_dims* dims, const asr_weights* weights, void
     const int v = std::atoi(e);
     if (v == 64 || v == 128 || v == 256) h->enc_bn = v;
   }
+  if (const char* e = std::getenv("ASRSPEC_ENC_PAIR")) h->enc_pair = std::atoi(e) != 0;
   if (const char* e = std::getenv("ASRSPEC_ENC_GROUP")) h->enc_group = std::max(0, std::atoi(e));
   h->es = h->bf16 ? 2 : 4;
   h->ln_fold = h->bf16 && h->d % 128 == 0 && h->wide_bn <= 64;
@@ -1237,6 +1240,7 @@ int asr_spec_create(const asr_model_dims* dims, const asr_weights* weights, void
     }
   }
   configure_gemm_tc();
+  configure_gemm_pair(h->n_sms);
   configure_attention_tc();
   CK(cudaDeviceSynchronize());
   return finish(0);
@@ -1247,6 +1251,44 @@ int asr_spec_set_host_io(asr_spec_handle h, int host_io) {
   h->host_io = host_io ? 1 : 0;
   return ASR_OK;
 }
+
+}  // extern "C"
+
+namespace {
+
+// Encoder states [M][d] times the stacked cross projections W [N][d] into the
+// cross cache (bf16).  The pair kernel from three waves of its 256 x 256 tiles
+// on (one utterance of 1500 frames, 8 layers: 72 us against 113; 64 utterances
+// 1869 against 3582); below, the 128 x 128 tiles spread better (100 tiles: 25
+// us against 30).
+int encode_gemm(asr_spec* h, const void* enc_states, const void* W, int M, int N, const Epi& e) {
+  const int d = h->d;
+  TcGemm g{};
+  g.bn = h->enc_bn;
+  if (!make_tmap_bf16(&g.mapA, enc_states, M, d, 128))
+    return fail(h, ASR_E_INVAL, "encoder states must be 16-byte aligned");
+  const long long tiles = (long long)(M / e.t_max) * ((e.t_max + 255) / 256) * ((N + 255) / 256);
+  Prof pg(h, ASR_PROF_OTHER, 1);
+  if (h->enc_pair && tiles >= 3 * (h->n_sms / 2)) {
+    if (!make_tmap_bf16(&g.mapB, W, N, d, 128)) return fail(h, ASR_E_CUDA, "tensor map encode failed");
+    if (launch_encode_pair(g.mapA, g.mapB, M / e.t_max, d, e, h->status, h->st)) return 0;
+  }
+  if (!make_tmap_bf16(&g.mapB, W, N, d, g.bn)) return fail(h, ASR_E_CUDA, "tensor map encode failed");
+  Epi et = e;
+  et.group_m = h->enc_group;   // both operands exceed L2: bands of frame tiles sweep the weight tiles
+  g.M = M;
+  g.N = N;
+  g.K = d;
+  g.splits = 1;
+  g.ws = h->ws;
+  g.tickets = h->tickets;
+  launch_gemm_tc(g, EPI_CROSSKV, et, h->status, h->st);
+  return 0;
+}
+
+}  // namespace
+
+extern "C" {
 
 int asr_spec_encode_cache(asr_spec_handle h, int32_t B, const void* enc_states, int32_t t_max,
                           const int32_t* enc_lens) {
@@ -1272,19 +1314,7 @@ int asr_spec_encode_cache(asr_spec_handle h, int32_t B, const void* enc_states, 
   e.M = M;
   e.N = N;
   if (h->bf16) {
-    TcGemm g{};
-    g.bn = h->enc_bn;
-    if (!make_tmap_bf16(&g.mapA, enc_states, M, d, 128) || !make_tmap_bf16(&g.mapB, h->w_cross, N, d, g.bn))
-      return fail(h, ASR_E_INVAL, "encoder states must be 16-byte aligned");
-    g.M = M;
-    g.N = N;
-    g.K = d;
-    e.group_m = h->enc_group;   // both operands exceed L2: bands of frame tiles sweep the weight tiles
-    g.splits = 1;
-    g.ws = h->ws;
-    g.tickets = h->tickets;
-    Prof pg(h, ASR_PROF_OTHER, 1);
-    launch_gemm_tc(g, EPI_CROSSKV, e, h->status, h->st);
+    if (int rc = encode_gemm(h, enc_states, h->w_cross, M, N, e)) return rc;
   } else {
     Prof pg(h, ASR_PROF_OTHER, 1);
     F32Gemm g{};
@@ -1300,18 +1330,7 @@ int asr_spec_encode_cache(asr_spec_handle h, int32_t B, const void* enc_states, 
     de.bias = h->dw.b_cross;
     de.kcache = h->d_xkv;
     de.N = 2 * d;
-    TcGemm g{};
-    g.bn = h->enc_bn;
-    if (!make_tmap_bf16(&g.mapA, enc_states, M, d, 128) || !make_tmap_bf16(&g.mapB, h->dw.w_cross, 2 * d, d, g.bn))
-      return fail(h, ASR_E_INVAL, "encoder states must be 16-byte aligned");
-    g.M = M;
-    g.N = 2 * d;
-    g.K = d;
-    g.splits = 1;
-    g.ws = h->ws;
-    g.tickets = h->tickets;
-    Prof pg(h, ASR_PROF_OTHER, 1);
-    launch_gemm_tc(g, EPI_CROSSKV, de, h->status, h->st);
+    if (int rc = encode_gemm(h, enc_states, h->dw.w_cross, M, 2 * d, de)) return rc;
   }
   CK(cudaGetLastError());
   h->B = B;

@@ -1,0 +1,375 @@
+// Encoder-cache GEMM on CTA pairs: every layer's cross K/V projections of the encoder states, Kx = E Wck^T, Vx = E Wcv^T + bcv (C[m][n], m = frame, n =
+// (layer, k | v, head, c)), written straight into the cross cache.
+//
+// tcgen05.mma with cta_group::2: a pair of CTAs multiplies a 256 x 256 tile,
+// each CTA holding 128 frames of A, half of the 256 weight rows of B and its
+// 128 rows of the accumulator.  A single CTA's 128 x 128 tile takes 32 KB from
+// L2 per 128 x 128 x 64 products, more than the 64 bytes per clock that an SM
+// gets (the 128 x 128 tiles before this kernel ran at 660 TFLOP/s); a pair's
+// 256 x 256 tile takes 32 KB per CTA for four times the products per pair, half
+// of that rate.  Persistent: 76 pairs walk the tiles,
+//   warp 0      : TMA producer of its CTA's halves, PG_STAGES-deep ring; the
+//                 copies of both CTAs count on the leader's barrier
+//   warp 1      : the leader's MMA issuer; commits release both CTAs' stages
+//   warps 4 - 7 : epilogue of the previous tile (two accumulators of 256
+//                 columns in tensor memory), so that the cache writes overlap
+//                 the next tile's products
+// The frames are taken in blocks of 128 that start at an utterance's first
+// frame: only blocks that hold real frames are visited, found through a prefix
+// sum over the utterances' block counts, and the two CTAs of a pair may hold
+// blocks of different utterances.  Blocks advance in bands of PG_BAND pairs
+// that sweep the weight tiles, so that a band's states stay in L2.  64 utterances of 875 frames on average, d =
+// 1280, 8 layers: 1869 us, 1625 TFLOP/s, against 3582 us.
+#include <mutex>
+
+#include "kernels.h"
+
+namespace asrspec {
+
+ASRSPEC_CHECK_SETTER(set_check_gemm_pair)
+
+namespace {
+
+constexpr int PG_THREADS = 256;
+constexpr int PG_STAGES = 6;
+constexpr int PG_TILE = 128 * 64 * 2;              // one operand half of a k-block
+constexpr int PG_STAGE_BYTES = 2 * PG_TILE;        // per CTA
+constexpr int PG_BAND = 32;
+constexpr int PG_B_MAX = 1024;                     // utterances of a handle
+constexpr int PG_SMEM = 1024 + PG_STAGES * PG_STAGE_BYTES + 256;
+
+__device__ __forceinline__ void tma_load_2d_pair(void* smem_dst, const CUtensorMap* map, uint32_t bar, int x, int y) {
+  asm volatile(
+      "cp.async.bulk.tensor.2d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4}], "
+      "[%2];" ::"r"(smem_u32(smem_dst)),
+      "l"(reinterpret_cast<uint64_t>(map)), "r"(bar), "r"(x), "r"(y)
+      : "memory");
+}
+__device__ __forceinline__ void umma_bf16_pair(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc,
+                                               uint32_t accumulate) {
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t"
+      "setp.ne.b32 p, %4, 0;\n\t"
+      "tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(d_tmem),
+      "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate)
+      : "memory");
+}
+// Arrive on the same barrier of both CTAs once the issued MMAs complete.
+__device__ __forceinline__ void umma_commit_pair(uint64_t* bar) {
+  asm volatile(
+      "tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;" ::"r"(
+          smem_u32(bar)),
+      "h"((uint16_t)3)
+      : "memory");
+}
+__device__ __forceinline__ void mbar_arrive_remote(uint32_t bar) {
+  asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(bar) : "memory");
+}
+__device__ __forceinline__ void tmem_ld32(uint32_t taddr, float* v) {
+  uint32_t r[32];
+  asm volatile(
+      "tcgen05.ld.sync.aligned.32x32b.x32.b32 "
+      "{%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,"
+      "%29,%30,%31}, [%32];"
+      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),
+        "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]), "=r"(r[16]),
+        "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]), "=r"(r[24]),
+        "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
+      : "r"(taddr));
+  asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+  for (int i = 0; i < 32; ++i) v[i] = __uint_as_float(r[i]);
+}
+
+// Shared-memory layout of both kernels: A ring, B ring, barriers.
+struct PairSmem {
+  uint8_t *a, *b;
+  uint64_t *full, *empty, *acc_full, *acc_empty;   // full, acc_empty: the leader's count
+  uint32_t* tmem_slot;
+  __device__ explicit PairSmem(uint8_t* raw) {
+    uint8_t* base = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(raw) + 1023) & ~uintptr_t(1023));
+    a = base;
+    b = base + PG_STAGES * PG_TILE;
+    full = reinterpret_cast<uint64_t*>(base + PG_STAGES * PG_STAGE_BYTES);
+    empty = full + PG_STAGES;
+    acc_full = empty + PG_STAGES;   // [2]
+    acc_empty = acc_full + 2;       // [2] four warps of both CTAs
+    tmem_slot = reinterpret_cast<uint32_t*>(acc_empty + 2);
+  }
+};
+
+// Warp 2 takes the pair's tensor memory, thread 0 the barriers.
+__device__ __forceinline__ void pair_setup(const PairSmem& sm, int warp) {
+  if (warp == 2) {
+    __syncwarp();
+    asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(sm.tmem_slot)),
+                 "r"(512u)
+                 : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
+  }
+  if (threadIdx.x == 0) {
+    for (int s = 0; s < PG_STAGES; ++s) {
+      mbar_init(&sm.full[s], 1);
+      mbar_init(&sm.empty[s], 1);
+    }
+    for (int a = 0; a < 2; ++a) {
+      mbar_init(&sm.acc_full[a], 1);
+      mbar_init(&sm.acc_empty[a], 8);
+    }
+    fence_mbar_init();
+  }
+}
+
+__device__ __forceinline__ void pair_teardown(uint32_t tmem, int warp) {
+  __syncwarp();
+  tc_fence_before();
+  __syncthreads();
+  cluster_sync();   // no MMA of the pair, no copy and no arrival is outstanding
+  if (warp == 2) {
+    tc_fence_after();
+    asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512u) : "memory");
+  }
+}
+
+// One thread per CTA: the k-blocks of tiles first, first + step, ... into the
+// ring.  rows(t, ra, rb): the tile's rows of this CTA's halves of A and B.
+// With PDL the first stages' B (constant weights) is requested before the wait
+// on the previous kernel.
+template <bool PDL, class Rows>
+__device__ __forceinline__ void pair_produce(const PairSmem& sm, const CUtensorMap* mapA, const CUtensorMap* mapB,
+                                             uint32_t rank, int first, int step, int tiles, int nkb, int* status,
+                                             Rows rows) {
+  tma_prefetch_desc(mapA);
+  tma_prefetch_desc(mapB);
+  auto load_b = [&](int s, int kb, int rb) {
+    if (rank == 0) mbar_arrive_expect_tx(&sm.full[s], 2 * PG_STAGE_BYTES);   // both CTAs' halves of A and B
+    tma_load_2d_pair(sm.b + s * PG_TILE, mapB, dsmem_addr(&sm.full[s], 0), kb * 64, rb);
+  };
+  auto load_a = [&](int s, int kb, int ra) {
+    tma_load_2d_pair(sm.a + s * PG_TILE, mapA, dsmem_addr(&sm.full[s], 0), kb * 64, ra);
+  };
+  int it = 0, ahead = 0;   // k-blocks issued; of them with B only, so far
+  if constexpr (PDL) {
+    if (first < tiles) {
+      int ra, rb;
+      rows(first, ra, rb);
+      ahead = nkb < PG_STAGES ? nkb : PG_STAGES;
+      for (int kb = 0; kb < ahead; ++kb) load_b(kb, kb, rb);
+    }
+    pdl_wait();
+  }
+  bool ok = true;
+  for (int t = first; t < tiles && ok; t += step) {
+    int ra, rb;
+    rows(t, ra, rb);
+    for (int kb = 0; kb < nkb; ++kb, ++it) {
+      const int s = it % PG_STAGES;
+      if (it >= ahead) {
+        if (!mbar_wait(&sm.empty[s], ((it / PG_STAGES) & 1) ^ 1, status)) {
+          ok = false;
+          break;
+        }
+        load_b(s, kb, rb);
+      }
+      load_a(s, kb, ra);
+    }
+  }
+  if (rank == 0)   // drain: both CTAs' copies have landed
+    for (int i = it - PG_STAGES > 0 ? it - PG_STAGES : 0; i < it; ++i)
+      mbar_wait(&sm.full[i % PG_STAGES], (i / PG_STAGES) & 1, status);
+}
+
+// One thread of the leader: the tiles' products, alternating accumulators.
+__device__ __forceinline__ void pair_mma(const PairSmem& sm, uint32_t tmem, uint32_t idesc, int first, int step,
+                                         int tiles, int nkb, int* status) {
+  int it = 0, n = 0;
+  bool ok = true;
+  for (int t = first; t < tiles && ok; t += step, ++n) {
+    const int a = n & 1;
+    if (!mbar_wait(&sm.acc_empty[a], ((n >> 1) & 1) ^ 1, status)) break;
+    tc_fence_after();
+    const uint32_t acc = tmem + (uint32_t)(a * 256);
+    for (int kb = 0; kb < nkb; ++kb, ++it) {
+      const int s = it % PG_STAGES;
+      if (!mbar_wait(&sm.full[s], (it / PG_STAGES) & 1, status)) {
+        ok = false;
+        break;
+      }
+      tc_fence_after();
+      const uint32_t a_addr = smem_u32(sm.a + s * PG_TILE), b_addr = smem_u32(sm.b + s * PG_TILE);
+#pragma unroll
+      for (int kk = 0; kk < 4; ++kk)
+        umma_bf16_pair(acc, umma_desc_sw128(a_addr + kk * 32), umma_desc_sw128(b_addr + kk * 32), idesc,
+                       (kb | kk) != 0);
+      umma_commit_pair(&sm.empty[s]);
+    }
+    umma_commit_pair(&sm.acc_full[a]);
+  }
+}
+
+__global__ void __launch_bounds__(PG_THREADS, 1)
+encode_pair_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUtensorMap mapB, int B, int K,
+                   Epi epi, int* status) {
+  extern __shared__ uint8_t smem_raw[];
+  const PairSmem sm(smem_raw);
+  __shared__ int s_pre[PG_B_MAX + 1];        // blocks before utterance b
+  __shared__ int s_warp[PG_THREADS / 32];
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const uint32_t rank = cluster_ctarank();
+
+  pair_setup(sm, warp);
+  // inclusive prefix sum of the block counts, four utterances per thread
+  int c[4], sum = 0;
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    const int b = 4 * tid + i;
+    const int T = b < B ? min(max(epi.enc_len[b], 0), epi.t_max) : 0;
+    sum += (T + 127) / 128;
+    c[i] = sum;
+  }
+  int x = sum;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const int y = __shfl_up_sync(0xffffffffu, x, o);
+    if (lane >= o) x += y;
+  }
+  if (lane == 31) s_warp[warp] = x;
+  __syncthreads();
+  int base = x - sum;
+  for (int w = 0; w < warp; ++w) base += s_warp[w];
+  if (tid == 0) s_pre[0] = 0;
+#pragma unroll
+  for (int i = 0; i < 4; ++i)
+    if (4 * tid + i < B) s_pre[4 * tid + i + 1] = base + c[i];
+  tc_fence_before();
+  __syncthreads();
+  cluster_sync();   // the peer's barriers are initialised
+  tc_fence_after();
+  const uint32_t tmem = *sm.tmem_slot;
+
+  const int n_blocks = s_pre[B], n_pairs = (n_blocks + 1) / 2;
+  const int nt = (epi.N + 255) / 256, nkb = K / 64;
+  const int tiles = n_pairs * nt;
+  // tile -> (pair of blocks, weight tile): bands of PG_BAND pairs sweep the weight tiles
+  auto tile_of = [&](int t, int& pair, int& n0) {
+    const int band = t / (PG_BAND * nt), r = t - band * PG_BAND * nt;
+    const int gm = min(PG_BAND, n_pairs - band * PG_BAND);
+    pair = band * PG_BAND + r % gm;
+    n0 = r / gm * 256;
+  };
+  // block of this CTA -> utterance and its first frame (t_max: none)
+  auto block_of = [&](int pair, int& b, int& t0) {
+    const int blk = 2 * pair + (int)rank;
+    if (blk >= n_blocks) {
+      b = 0;
+      t0 = epi.t_max;
+      return;
+    }
+    int lo = 0, hi = B;   // s_pre[lo] <= blk < s_pre[hi]
+    while (hi - lo > 1) {
+      const int mid = (lo + hi) >> 1;
+      if (s_pre[mid] <= blk) lo = mid;
+      else hi = mid;
+    }
+    b = lo;
+    t0 = (blk - s_pre[lo]) * 128;
+  };
+  const int first = blockIdx.x / 2, step = gridDim.x / 2;
+
+  if (warp == 0 && lane == 0) {
+    pair_produce<false>(sm, &mapA, &mapB, rank, first, step, tiles, nkb, status, [&](int t, int& ra, int& rb) {
+      int pair, b, t0;
+      tile_of(t, pair, rb);
+      block_of(pair, b, t0);
+      ra = t0 < epi.t_max ? b * epi.t_max + t0 : 0;   // no block: any rows, not stored
+      rb += (int)rank * 128;
+    });
+  } else if (warp == 1 && lane == 0 && rank == 0) {
+    pair_mma(sm, tmem, umma_idesc_bf16(256, 256), first, step, tiles, nkb, status);
+  } else if (warp >= 4) {
+    const int wq = warp - 4;
+    int n = 0;
+    for (int t = first; t < tiles; t += step, ++n) {
+      const int a = n & 1;
+      int pair, n0, b, t0;
+      tile_of(t, pair, n0);
+      block_of(pair, b, t0);
+      const int ft = t0 + wq * 32 + lane;
+      const bool frame_ok = t0 < epi.t_max && ft < min(epi.enc_len[b], epi.t_max);
+      __syncwarp();
+      const bool ok = mbar_wait(&sm.acc_full[a], (n >> 1) & 1, status);
+      if (__any_sync(0xffffffffu, !ok)) break;
+      tc_fence_after();
+      const uint32_t t_lane = tmem + ((uint32_t)(wq * 32) << 16) + (uint32_t)(a * 256);
+#pragma unroll 1
+      for (int c0 = 0; c0 < 256; c0 += 32) {
+        __syncwarp();   // tcgen05.ld is warp-aligned; only the stores branch
+        float v[32];
+        tmem_ld32(t_lane + c0, v);
+        const int f0 = n0 + c0;
+        if (frame_ok && f0 < epi.N && !bounds_bad(epi.status, b >= epi.b_max || ft >= epi.max_enc)) {
+          // 32 features of one frame lie in one head (N and d are multiples of 64): four 16-byte stores
+          const int two_d = 2 * epi.d, l = f0 / two_d, r = f0 - l * two_d, which = r / epi.d, f = r - which * epi.d;
+          const size_t idx =
+              (((((size_t)l * 2 + which) * epi.b_max + b) * epi.n_heads + (f >> 6)) * epi.max_enc + ft) * 64 + (f & 63);
+          uint4* dst = reinterpret_cast<uint4*>(static_cast<__nv_bfloat16*>(epi.kcache) + idx);
+#pragma unroll
+          for (int q = 0; q < 4; ++q) {
+            const float4 b0 = __ldg(reinterpret_cast<const float4*>(epi.bias + f0) + 2 * q);
+            const float4 b1 = __ldg(reinterpret_cast<const float4*>(epi.bias + f0) + 2 * q + 1);
+            const float* w = v + 8 * q;
+            __nv_bfloat162 p0 = __floats2bfloat162_rn(w[0] + b0.x, w[1] + b0.y),
+                           p1 = __floats2bfloat162_rn(w[2] + b0.z, w[3] + b0.w),
+                           p2 = __floats2bfloat162_rn(w[4] + b1.x, w[5] + b1.y),
+                           p3 = __floats2bfloat162_rn(w[6] + b1.z, w[7] + b1.w);
+            dst[q] = make_uint4(*reinterpret_cast<uint32_t*>(&p0), *reinterpret_cast<uint32_t*>(&p1),
+                                *reinterpret_cast<uint32_t*>(&p2), *reinterpret_cast<uint32_t*>(&p3));
+          }
+        }
+        __syncwarp();
+      }
+      tc_fence_before();
+      __syncwarp();
+      if (lane == 0) mbar_arrive_remote(dsmem_addr(&sm.acc_empty[a], 0));
+    }
+  }
+  pair_teardown(tmem, warp);
+}
+
+}  // namespace
+
+// CTA pairs of a kernel that run at once on this device (0: it cannot run).
+template <class Kern>
+static int pair_count(Kern kern, int sms) {
+  if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, PG_SMEM) != cudaSuccess) return 0;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(2 * (sms / 2));
+  cfg.blockDim = dim3(PG_THREADS);
+  cfg.dynamicSmemBytes = PG_SMEM;
+  cudaLaunchAttribute at;
+  at.id = cudaLaunchAttributeClusterDimension;
+  at.val.clusterDim.x = 2;
+  at.val.clusterDim.y = at.val.clusterDim.z = 1;
+  cfg.attrs = &at;
+  cfg.numAttrs = 1;
+  int n = 0;
+  if (cudaOccupancyMaxActiveClusters(&n, kern, &cfg) != cudaSuccess) return 0;
+  return n < sms / 2 ? n : sms / 2;
+}
+
+static int g_encode_pairs = 0;
+void configure_gemm_pair(int sms) {
+  static std::once_flag once;
+  std::call_once(once, [&] {
+    g_encode_pairs = pair_count(encode_pair_kernel, sms);
+  });
+}
+
+bool launch_encode_pair(const CUtensorMap& mapA, const CUtensorMap& mapB, int B, int K, const Epi& epi, int* status,
+                        cudaStream_t st) {
+  if (g_encode_pairs < 1 || B > PG_B_MAX || epi.N % 64 || epi.d % 64) return false;
+  return launch_ex(encode_pair_kernel, dim3(2 * g_encode_pairs), dim3(PG_THREADS), (size_t)PG_SMEM, st, false, 2, mapA,
+                   mapB, B, K, epi, status) == cudaSuccess;
+}
+
+}  // namespace asrspec

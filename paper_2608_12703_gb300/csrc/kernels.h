@@ -29,6 +29,13 @@ int tc_pick_bn(int n_max);
 int tc_pick_bn_wide(int n);
 void launch_gemm_tc(const TcGemm& g, int mode, const Epi& epi, int* status, cudaStream_t st);
 size_t tc_smem_bytes(int bn);
+// CTA-pair kernels (csrc/gemm_pair.cu).  Encoder-cache build: mapA over the
+// encoder states [B * t_max][K], mapB over the stacked weights [N][K] (boxes
+// 64 x 128), epi as for EPI_CROSSKV.  False
+// when it cannot run here.
+void configure_gemm_pair(int sms);
+bool launch_encode_pair(const CUtensorMap& mapA, const CUtensorMap& mapB, int B, int K, const Epi& epi, int* status,
+                        cudaStream_t st);
 // 2-D fp32 tensor map over [rows][cols], no swizzle, box {box_cols, box_rows}.
 bool make_tmap_f32(CUtensorMap* map, const void* base, uint64_t rows, uint64_t cols, uint32_t box_cols,
                    uint32_t box_rows);
@@ -312,6 +319,7 @@ void launch_mark_ready(const int* enc_len, int B, int t_max, int* ready, int* kv
 void set_check_gemm_tc(int on);
 void set_check_gemm_f32(int on);
 void set_check_gemm_wide(int on);
+void set_check_gemm_pair(int on);
 void set_check_rows(int on);
 void set_check_attention(int on);
 void set_check_attention_tc(int on);

@@ -133,6 +133,36 @@ def test_fp32_projection_and_attention_sizes(built_lib, cuda, d, heads, ffn, voc
     assert_bounded(st)
 
 
+@pytest.mark.parametrize("d,n_layers", [(128, 2), (192, 2)])
+def test_encoder_cache_on_pairs(built_lib, cuda, d, n_layers):
+    """Enough frames for the CTA-pair encoder GEMM: blocks of 128 frames that
+    end inside, at and just past an utterance, an odd number of blocks (the
+    last pair half empty), weight tiles that straddle a layer and end short
+    (d = 192); bit for bit the one-CTA kernel's cache, seen through a verification."""
+    dims = W.ModelDims(n_layers=n_layers, d_model=d, n_heads=d // 64, d_ffn=4 * d, vocab=500, dtype="bf16",
+                       max_pos=40, max_enc=600, anchor_layer=1)
+    blob = _blob(dims, 0.1)
+    enc_lens = [600, 1, 127, 128, 129, 255, 256, 257, 512, 384] * 4 + [385]
+    B = len(enc_lens)
+    enc = W.make_encoder_states(dims, enc_lens, 600)
+    prompt = W.make_prompt(dims, B)
+    outs = []
+    for pair in ("1", "0"):
+        with pytest.MonkeyPatch.context() as mp:
+            mp.setenv("ASRSPEC_ENC_PAIR", pair)
+            sess = _session(dims, blob, B, 3)()
+        sess.encode_cache(enc, enc_lens)
+        sess.prefill(prompt)
+        o = sess.verify(np.tile(prompt[:, -1:], (1, 3)), [3] * B)
+        outs.append((o, sess.anchor_profile()))
+        assert sess.status() == 0
+        sess.close()
+    for a, b in zip(outs[0][0].__dict__.values(), outs[1][0].__dict__.values()):
+        np.testing.assert_array_equal(a, b)
+    for b in range(B):
+        np.testing.assert_array_equal(outs[0][1][b, :enc_lens[b]], outs[1][1][b, :enc_lens[b]])
+
+
 @pytest.mark.parametrize("dtype,batch,prompt_len", [
     ("bf16", 2, 33), ("bf16", 2, 34), ("bf16", 1, 66), ("bf16", 40, 28), ("fp32", 2, 35), ("fp32", 30, 40)])
 def test_prompt_lengths(built_lib, cuda, dtype, batch, prompt_len):
