@@ -133,6 +133,7 @@ struct asr_spec {
   int wide_target = 2 * 152;   // CTAs a many-row GEMM may fill by splitting K (ASRSPEC_WIDE_TARGET)
   int few_target = 2 * 152;    // the same for few rows (ASRSPEC_FEW_TARGET)
   bool enc_pair = true;   // encoder-cache GEMM on CTA pairs (ASRSPEC_ENC_PAIR=0: one CTA per tile)
+  bool lm_pair = true;    // LM head of more than 64 rows on CTA pairs (ASRSPEC_LM_PAIR=0: one CTA per tile)
   // encoder cache, one CTA per tile: N tile (ASRSPEC_ENC_BN) and M tiles per band of the
   // grouped order (ASRSPEC_ENC_GROUP, 0 = plain); measured at 64 utterances x
   // 1500 frames: 14.5 ms (128, 64) against 16.7 (256, 32) and 23.6 (256, plain)
@@ -343,6 +344,13 @@ int gemm_rows(asr_spec* h, const void* W, const CUtensorMap* mW, int M, int K, c
       h->ln_S = M / 128;
     }
     return 0;
+  }
+  if (mode == EPI_ARGMAX && h->lm_pair && N > 64) {   // up to 64 rows the weights' HBM time bounds one CTA per tile too
+    const CUtensorMap* mb = bmap(h, x_id, X, h->R_pad, K, 128);
+    if (!mb) return fail(h, ASR_E_CUDA, "tensor map encode failed");
+    Tl t(h, ASR_TL_GEMM + mode + (epi.ln_part ? ASR_TL_LN_FUSED : 0));
+    epi.tl = h->tl_cur;
+    if (launch_lmhead_pair(*mb, *mW, K, epi, h->use_pdl, h->status, h->st)) return 0;
   }
   TcGemm g{};
   g.mapA = *mW;
@@ -1003,6 +1011,7 @@ int asr_spec_create(const asr_model_dims* dims, const asr_weights* weights, void
     if (v == 64 || v == 128 || v == 256) h->enc_bn = v;
   }
   if (const char* e = std::getenv("ASRSPEC_ENC_PAIR")) h->enc_pair = std::atoi(e) != 0;
+  if (const char* e = std::getenv("ASRSPEC_LM_PAIR")) h->lm_pair = std::atoi(e) != 0;
   if (const char* e = std::getenv("ASRSPEC_ENC_GROUP")) h->enc_group = std::max(0, std::atoi(e));
   h->es = h->bf16 ? 2 : 4;
   h->ln_fold = h->bf16 && h->d % 128 == 0 && h->wide_bn <= 64;

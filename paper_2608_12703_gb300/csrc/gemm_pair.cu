@@ -1,4 +1,5 @@
-// Encoder-cache GEMM on CTA pairs: every layer's cross K/V projections of the encoder states, Kx = E Wck^T, Vx = E Wcv^T + bcv (C[m][n], m = frame, n =
+// GEMMs on CTA pairs: the LM head with argmax for many rows (below), and the
+// encoder cache: every layer's cross K/V projections of the encoder states, Kx = E Wck^T, Vx = E Wcv^T + bcv (C[m][n], m = frame, n =
 // (layer, k | v, head, c)), written straight into the cross cache.
 //
 // tcgen05.mma with cta_group::2: a pair of CTAs multiplies a 256 x 256 tile,
@@ -336,6 +337,145 @@ encode_pair_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_consta
   pair_teardown(tmem, warp);
 }
 
+// LM head with argmax on the same pipeline: A = the verify rows (256 per tile,
+// 128 per CTA), B = token embeddings (256 ids per tile).  Rows on the lane side
+// of the accumulator: a thread of the epilogue holds one row and scans its 256
+// logits without any exchange (y = rstd (acc - mu c1) + c2 where the LayerNorm
+// is folded), keeps the row's best in shared memory over the tiles of the CTA,
+// and one atomicMax per row and CTA ends it.  448 rows, V = 51866, d = 1280: 48
+// us (84 with ids on the lanes and one CTA per tile, 56 on pairs with the keys
+// of 32 lanes reduced by shuffles); 544 rows at d = 768 36 us (85), 96 rows at d
+// = 1280 30 us (42).
+constexpr int PL_ROWS = 1024;   // rows whose statistics and best keys fit beside the ring
+
+__global__ void __launch_bounds__(PG_THREADS, 1)
+lmhead_pair_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_constant__ CUtensorMap mapW, int K, Epi epi,
+                   int* status) {
+  extern __shared__ uint8_t smem_raw[];
+  const PairSmem sm(smem_raw);
+  __shared__ unsigned long long s_best[PL_ROWS];
+  __shared__ float s_mu[PL_ROWS], s_rs[PL_ROWS];
+  __shared__ __align__(16) float s_c[4][2][256];   // per epilogue warp: the tile's folded-LayerNorm c1, c2
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const uint32_t rank = cluster_ctarank();
+  tl_mark(epi.tl, TL_ENTRY);
+  const int n_valid = epi.n_valid ? min(*epi.n_valid, epi.N) : epi.N;
+  pair_setup(sm, warp);
+  for (int r = tid; r < n_valid; r += PG_THREADS) s_best[r] = 0ull;
+  tc_fence_before();
+  __syncthreads();
+  cluster_sync();   // the peer's barriers are initialised
+  tc_fence_after();
+  const uint32_t tmem = *sm.tmem_slot;
+  const int rt = (n_valid + 255) / 256, nkb = K / 64;
+  const int tiles = (epi.M + 255) / 256 * rt;   // the row tiles of one weight tile follow one another
+  const int first = blockIdx.x / 2, step = gridDim.x / 2;
+
+  if (warp == 0 && lane == 0) {
+    pair_produce<true>(sm, &mapX, &mapW, rank, first, step, tiles, nkb, status, [&](int t, int& ra, int& rb) {
+      ra = t % rt * 256 + (int)rank * 128;
+      rb = t / rt * 256 + (int)rank * 128;
+    });
+  } else if (warp == 1 && lane == 0 && rank == 0) {
+    pair_mma(sm, tmem, umma_idesc_bf16(256, 256), first, step, tiles, nkb, status);
+  } else if (warp >= 4) {
+    pdl_wait();
+    tl_mark(epi.tl, TL_WORK);
+    pdl_launch();
+    const int et = tid - 128;
+    const bool fold = epi.ln_part != nullptr;
+    if (fold) {   // row statistics from the producer's equal slices, shifted by the first one's mean
+      const int S = epi.ln_S;
+      for (int r = et; r < n_valid; r += 128) {
+        const float2* pr = epi.ln_part + r;
+        const float shift = pr[0].x;
+        float e1 = 0.f, e2 = 0.f, m2 = 0.f;
+        for (int j0 = 0; j0 < S; j0 += 8) {
+          float2 p[8];
+#pragma unroll
+          for (int u = 0; u < 8; ++u)
+            p[u] = j0 + u < S ? pr[(size_t)(j0 + u) * epi.ln_stride] : make_float2(shift, 0.f);
+#pragma unroll
+          for (int u = 0; u < 8; ++u) {
+            const float es = p[u].x - shift;
+            e1 += es;
+            e2 += es * es;
+            m2 += p[u].y;
+          }
+        }
+        const float q = m2 + (float)epi.ln_c * fmaxf(e2 - e1 * e1 / (float)S, 0.f);
+        s_mu[r] = shift + e1 / (float)S;
+        s_rs[r] = rsqrtf(q / (float)(S * epi.ln_c) + 1e-5f);
+      }
+      asm volatile("bar.sync 1, 128;" ::: "memory");   // the epilogue warps
+    }
+    const int wq = warp - 4;
+    int n = 0;
+    for (int t = first; t < tiles; t += step, ++n) {
+      const int a = n & 1, v0 = t / rt * 256;
+      const int r = t % rt * 256 + (int)rank * 128 + wq * 32 + lane;
+      const bool row_ok = r < n_valid;
+      const float mu = fold && row_ok ? s_mu[r] : 0.f, rs = fold && row_ok ? s_rs[r] : 1.f;
+      if (fold) {   // while the products run
+        __syncwarp();   // the previous tile's reads
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+          const int id = v0 + 32 * i + lane;
+          s_c[wq][0][32 * i + lane] = id < epi.M ? __ldg(epi.ln_c1 + id) : 0.f;
+          s_c[wq][1][32 * i + lane] = id < epi.M ? __ldg(epi.ln_c2 + id) : 0.f;
+        }
+      }
+      __syncwarp();
+      const bool ok = mbar_wait(&sm.acc_full[a], (n >> 1) & 1, status);
+      if (__any_sync(0xffffffffu, !ok)) break;
+      tc_fence_after();
+      const uint32_t t_lane = tmem + ((uint32_t)(wq * 32) << 16) + (uint32_t)(a * 256);
+      unsigned long long best = 0ull;
+#pragma unroll 1
+      for (int c0 = 0; c0 < 256; c0 += 32) {   // uniform over the warp
+        const int id0 = v0 + c0;
+        if (id0 >= epi.M) break;
+        float v[32];
+        tmem_ld32(t_lane + c0, v);
+        uint32_t m = 0u;   // the logits' order codes, as in argmax_key
+        int mi = 0;
+        if (fold) {
+#pragma unroll
+          for (int i = 0; i < 32; i += 4) {
+            const float4 c1 = *reinterpret_cast<const float4*>(&s_c[wq][0][c0 + i]);
+            const float4 c2 = *reinterpret_cast<const float4*>(&s_c[wq][1][c0 + i]);
+            v[i] = rs * (v[i] - mu * c1.x) + c2.x;
+            v[i + 1] = rs * (v[i + 1] - mu * c1.y) + c2.y;
+            v[i + 2] = rs * (v[i + 2] - mu * c1.z) + c2.z;
+            v[i + 3] = rs * (v[i + 3] - mu * c1.w) + c2.w;
+          }
+        }
+#pragma unroll
+        for (int i = 0; i < 32; ++i) {   // increasing ids: the first maximum is kept
+          const uint32_t u = ordered_bits(v[i]);
+          if (id0 + i < epi.M && u > m) {
+            m = u;
+            mi = i;
+          }
+        }
+        const unsigned long long key = ((unsigned long long)m << 32) | (0xFFFFFFFFu - (uint32_t)(id0 + mi));
+        best = key > best ? key : best;
+        __syncwarp();
+      }
+      tc_fence_before();
+      __syncwarp();
+      if (lane == 0) mbar_arrive_remote(dsmem_addr(&sm.acc_empty[a], 0));
+      if (row_ok && best > s_best[r]) s_best[r] = best;   // this thread's row until the next tile
+    }
+    asm volatile("bar.sync 1, 128;" ::: "memory");
+    for (int r = et; r < n_valid; r += 128)
+      if (s_best[r]) atomicMax(epi.row_key + r, s_best[r]);
+  }
+  tl_mark(epi.tl, TL_MID);
+  pair_teardown(tmem, warp);
+  tl_mark(epi.tl, TL_EXIT);
+}
+
 }  // namespace
 
 // CTA pairs of a kernel that run at once on this device (0: it cannot run).
@@ -357,11 +497,12 @@ static int pair_count(Kern kern, int sms) {
   return n < sms / 2 ? n : sms / 2;
 }
 
-static int g_encode_pairs = 0;
+static int g_encode_pairs = 0, g_lmhead_pairs = 0;
 void configure_gemm_pair(int sms) {
   static std::once_flag once;
   std::call_once(once, [&] {
     g_encode_pairs = pair_count(encode_pair_kernel, sms);
+    g_lmhead_pairs = pair_count(lmhead_pair_kernel, sms);
   });
 }
 
@@ -370,6 +511,13 @@ bool launch_encode_pair(const CUtensorMap& mapA, const CUtensorMap& mapB, int B,
   if (g_encode_pairs < 1 || B > PG_B_MAX || epi.N % 64 || epi.d % 64) return false;
   return launch_ex(encode_pair_kernel, dim3(2 * g_encode_pairs), dim3(PG_THREADS), (size_t)PG_SMEM, st, false, 2, mapA,
                    mapB, B, K, epi, status) == cudaSuccess;
+}
+
+bool launch_lmhead_pair(const CUtensorMap& mapX, const CUtensorMap& mapW, int K, const Epi& epi, bool pdl, int* status,
+                        cudaStream_t st) {
+  if (g_lmhead_pairs < 1 || epi.N > PL_ROWS) return false;
+  return launch_ex(lmhead_pair_kernel, dim3(2 * g_lmhead_pairs), dim3(PG_THREADS), (size_t)PG_SMEM, st, pdl, 2, mapX,
+                   mapW, K, epi, status) == cudaSuccess;
 }
 
 }  // namespace asrspec

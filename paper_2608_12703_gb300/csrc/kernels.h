@@ -31,10 +31,13 @@ void launch_gemm_tc(const TcGemm& g, int mode, const Epi& epi, int* status, cuda
 size_t tc_smem_bytes(int bn);
 // CTA-pair kernels (csrc/gemm_pair.cu).  Encoder-cache build: mapA over the
 // encoder states [B * t_max][K], mapB over the stacked weights [N][K] (boxes
-// 64 x 128), epi as for EPI_CROSSKV.  False
-// when it cannot run here.
+// 64 x 128), epi as for EPI_CROSSKV.  LM head with argmax: mapX over the rows,
+// mapW over the embeddings (boxes 64 x 128), epi as for EPI_ARGMAX; at most
+// 1024 rows.  False when they cannot run here.
 void configure_gemm_pair(int sms);
 bool launch_encode_pair(const CUtensorMap& mapA, const CUtensorMap& mapB, int B, int K, const Epi& epi, int* status,
+                        cudaStream_t st);
+bool launch_lmhead_pair(const CUtensorMap& mapX, const CUtensorMap& mapW, int K, const Epi& epi, bool pdl, int* status,
                         cudaStream_t st);
 // 2-D fp32 tensor map over [rows][cols], no swizzle, box {box_cols, box_rows}.
 bool make_tmap_f32(CUtensorMap* map, const void* base, uint64_t rows, uint64_t cols, uint32_t box_cols,

@@ -163,6 +163,44 @@ def test_encoder_cache_on_pairs(built_lib, cuda, d, n_layers):
         np.testing.assert_array_equal(outs[0][1][b, :enc_lens[b]], outs[1][1][b, :enc_lens[b]])
 
 
+@pytest.mark.parametrize("batch,k,vocab,ln_fold", [(11, 5, 255, "1"), (9, 14, 257, "1"), (33, 7, 1001, "0"),
+                                                   (86, 5, 513, "1"), (64, 15, 40, "1")])
+def test_lm_head_on_pairs(built_lib, cuda, batch, k, vocab, ln_fold):
+    """The CTA-pair LM head at 66 to 1024 rows (one to four row tiles, the last
+    one ragged; vocabularies around and below a 256-id tile) gives the tokens
+    of the one-CTA kernel."""
+    dims = W.ModelDims(n_layers=1, d_model=128, n_heads=2, d_ffn=512, vocab=vocab, dtype="bf16",
+                       max_pos=40, max_enc=20, anchor_layer=0)
+    blob = _blob(dims, 0.1)
+    enc_lens = [1 + b % 20 for b in range(batch)]
+    enc = W.make_encoder_states(dims, enc_lens, 20)
+    prompt = W.make_prompt(dims, batch)
+    rng = np.random.default_rng(batch)
+    outs = []
+    for pair in ("1", "0"):
+        with pytest.MonkeyPatch.context() as mp:
+            mp.setenv("ASRSPEC_LM_PAIR", pair)
+            mp.setenv("ASRSPEC_LN_FOLD", ln_fold)
+            sess = _session(dims, blob, batch, k)()
+        sess.encode_cache(enc, enc_lens)
+        sess.prefill(prompt)
+        rng = np.random.default_rng(batch)
+        for _ in range(2):   # whole blocks, then ragged ones
+            lens = np.where(rng.random(batch) < 0.2, rng.integers(-1, k + 1, batch), k).astype(np.int32)
+            o = sess.verify(rng.integers(0, vocab, (batch, k)).astype(np.int32), lens)
+            outs.append(np.stack([o.accepted, o.bonus, o.kv_len, o.anchor]))
+        lg = sess.debug_logits(batch * (k + 1)).cpu().numpy()
+        r0 = 0
+        for b in range(batch):   # the bonus row's own argmax (no draft was accepted unless it matched)
+            if lens[b] >= 0:
+                assert int(lg[r0 + o.accepted[b]].argmax()) == o.bonus[b]
+                r0 += int(lens[b]) + 1
+        assert sess.status() == 0
+        sess.close()
+    np.testing.assert_array_equal(outs[0], outs[2])
+    np.testing.assert_array_equal(outs[1], outs[3])
+
+
 @pytest.mark.parametrize("dtype,batch,prompt_len", [
     ("bf16", 2, 33), ("bf16", 2, 34), ("bf16", 1, 66), ("bf16", 40, 28), ("fp32", 2, 35), ("fp32", 30, 40)])
 def test_prompt_lengths(built_lib, cuda, dtype, batch, prompt_len):
