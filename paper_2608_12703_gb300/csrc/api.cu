@@ -85,7 +85,7 @@ struct asr_spec {
   int* tickets = nullptr;
   int n_tickets = 0;
   int* attn_tickets = nullptr;                       // [B_max * H], tensor-core attention merge
-  CUtensorMap m_kself[2], m_vself[2], m_xkv[2];      // boxes of 128 and 256 rows
+  CUtensorMap m_kself[2], m_vself[2], m_xkv[2];      // boxes of 128 and 32 rows
   std::map<std::pair<int, int>, CUtensorMap> bmaps;  // (buffer id, BN) -> map
   std::map<std::pair<int, int>, CUtensorMap> xmaps;   // (target 0 / draft 1, BN) -> map of its residual stream (fp32, box 128 x BN)
   int n_sms = 0;
@@ -449,13 +449,15 @@ void attention(asr_spec* h, AttnArgs& a, bool self_attn, int layer) {
   }
   a.segs = (a.rows_max + 31) / 32;
   a.splits = attn_splits_for(h, h->B * a.segs, a.t_alloc, self_attn);
-  const int ci = 0;   // 128-row boxes
   if (self_attn) {
-    a.kmap = &h->m_kself[ci];
-    a.vmap = &h->m_vself[ci];
+    a.kmap = &h->m_kself[0];
+    a.vmap = &h->m_vself[0];
+    a.kmap32 = &h->m_kself[1];
+    a.vmap32 = &h->m_vself[1];
     a.k_row0 = a.v_row0 = (long long)layer * h->Bmax * h->H * h->maxpos;
   } else {
-    a.kmap = a.vmap = &h->m_xkv[ci];
+    a.kmap = a.vmap = &h->m_xkv[0];
+    a.kmap32 = a.vmap32 = &h->m_xkv[1];
     a.k_row0 = (long long)layer * 2 * h->Bmax * h->H * h->Tmax;
     a.v_row0 = a.k_row0 + (long long)h->Bmax * h->H * h->Tmax;
   }
@@ -1216,7 +1218,7 @@ int asr_spec_create(const asr_model_dims* dims, const asr_weights* weights, void
     const uint64_t self_rows = (uint64_t)L * h->Bmax * h->H * h->maxpos;
     const uint64_t cross_rows = (uint64_t)L * 2 * h->Bmax * h->H * h->Tmax;
     for (int i = 0; i < 2; ++i) {
-      const uint32_t box = i ? 256 : 128;
+      const uint32_t box = i ? 32 : 128;
       if (!make_tmap_cache(&h->m_kself[i], h->kself, self_rows, box) ||
           !make_tmap_cache(&h->m_vself[i], h->vself, self_rows, box) ||
           !make_tmap_cache(&h->m_xkv[i], h->xkv, cross_rows, box))

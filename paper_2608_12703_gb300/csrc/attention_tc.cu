@@ -13,6 +13,10 @@
 //     mma.sync m16n8k16 (bf16 in, fp32 accumulate): S = Q K^T, then an online
 //     softmax on the accumulator fragments (quad shuffles), then O = P V with
 //     P re-used from the S fragments and V fragments from ldmatrix.trans;
+//   * a last chunk of fewer than 97 keys is loaded as 32-key boxes, only those
+//     that hold keys (a transcript of 38 keys: 16 KB instead of 32; ragged
+//     encoder lengths: 16 keys too many on average instead of 64), and the
+//     warps without a block skip it;
 //   * each of the 4 warps takes a quarter of every chunk's keys; the CTA
 //     combines its warps, and the S splits of one (utterance, head) form a
 //     thread-block cluster: CTA q owns output columns [64q/S, 64(q+1)/S), every
@@ -83,7 +87,8 @@ struct TcaCfg {
 // results by pushing them to the CTA that owns each output column (PUSH).
 template <int MT, int TCA_STAGES, bool PUSH, bool TREE>
 __global__ void __launch_bounds__(TCA_THREADS)
-attn_tc_kernel(const __grid_constant__ CUtensorMap kmap, const __grid_constant__ CUtensorMap vmap, AttnArgs a,
+attn_tc_kernel(const __grid_constant__ CUtensorMap kmap, const __grid_constant__ CUtensorMap vmap,
+               const __grid_constant__ CUtensorMap kmap32, const __grid_constant__ CUtensorMap vmap32, AttnArgs a,
                int* status) {
   using C = TcaCfg<MT, TCA_STAGES, PUSH>;
   extern __shared__ uint8_t smem_raw[];
@@ -133,9 +138,19 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap kmap, const __grid_constant__
     const int st = i % TCA_STAGES;
     const int key0 = (split + i * S) * TCA_CH;
     uint8_t* ks = smem + st * 2 * TCA_TILE;
-    mbar_arrive_expect_tx(&bar[st], 2 * TCA_TILE);
-    tma_load_2d(ks, &kmap, &bar[st], 0, (int)(a.k_row0 + rb + key0));
-    tma_load_2d(ks + TCA_TILE, &vmap, &bar[st], 0, (int)(a.v_row0 + rb + key0));
+    const int kr = (int)(a.k_row0 + rb + key0), vr = (int)(a.v_row0 + rb + key0);
+    const int blocks = (n_keys - key0 + 31) / 32;   // 32-key blocks that hold keys (one per warp)
+    if (blocks >= 4) {
+      mbar_arrive_expect_tx(&bar[st], 2 * TCA_TILE);
+      tma_load_2d(ks, &kmap, &bar[st], 0, kr);
+      tma_load_2d(ks + TCA_TILE, &vmap, &bar[st], 0, vr);
+    } else {
+      mbar_arrive_expect_tx(&bar[st], blocks * (TCA_TILE / 2));
+      for (int j = 0; j < blocks; ++j) {
+        tma_load_2d(ks + j * (TCA_TILE / 4), &kmap32, &bar[st], 0, kr + 32 * j);
+        tma_load_2d(ks + TCA_TILE + j * (TCA_TILE / 4), &vmap32, &bar[st], 0, vr + 32 * j);
+      }
+    }
   };
   // The encoder K/V cache is constant during a verify call: its first chunks
   // load while the previous kernel finishes.  Self-attention keys include rows
@@ -203,6 +218,7 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap kmap, const __grid_constant__
     const uint32_t vs_base = ks_base + TCA_TILE;
     const int kbase = (split + i * S) * TCA_CH + warp * C::KW;
 
+    if (kbase < n_keys) {   // this warp's block was loaded (uniform over the warp)
     float Sf[MT][C::NT][4];
 #pragma unroll
     for (int nt = 0; nt < C::NT; ++nt) {
@@ -281,6 +297,7 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap kmap, const __grid_constant__
           mma_bf16_16816(O[mt][2 * nd2 + 1], pa[mt], r2, r3);
         }
       }
+    }
     }
     __syncthreads();   // every warp is done with stage st
     if (tid == 0 && i + TCA_STAGES < n_iter) issue(i + TCA_STAGES);
@@ -412,7 +429,7 @@ void configure_attention_tc() {
 template <int MT, int ST, bool PUSH, bool TREE = false>
 static void launch_one(const AttnArgs& a, int splits, int* status, cudaStream_t st) {
   launch_ex(attn_tc_kernel<MT, ST, PUSH, TREE>, dim3(splits, a.H, a.B * a.segs), dim3(TCA_THREADS), TcaCfg<MT, ST, PUSH>::SMEM,
-            st, a.pdl, splits, *a.kmap, *a.vmap, a, status);
+            st, a.pdl, splits, *a.kmap, *a.vmap, *a.kmap32, *a.vmap32, a, status);
 }
 
 // a.splits CTAs (1, 2, 4 or 8; one cluster) per (utterance, head);

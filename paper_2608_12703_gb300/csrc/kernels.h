@@ -139,6 +139,7 @@ struct AttnArgs {
   // of this layer in each; per-(b, h) tickets for the in-kernel chunk merge
   const CUtensorMap* kmap = nullptr;
   const CUtensorMap* vmap = nullptr;
+  const CUtensorMap *kmap32 = nullptr, *vmap32 = nullptr;   // the same with boxes of 32 keys
   long long k_row0 = 0, v_row0 = 0;
   int* tickets = nullptr;
   int rows_max = 0;        // most rows of one utterance in this call

@@ -133,6 +133,26 @@ def test_fp32_projection_and_attention_sizes(built_lib, cuda, d, heads, ffn, voc
     assert_bounded(st)
 
 
+@pytest.mark.parametrize("k", [3, 17])
+def test_attention_key_blocks(built_lib, cuda, k):
+    """Encoder memories and transcripts whose last 128-key chunk holds one to
+    four 32-key blocks, full or by one key more or less; one and two m-tiles."""
+    dims = W.ModelDims(n_layers=2, d_model=128, n_heads=2, d_ffn=512, vocab=500, dtype="bf16",
+                       max_pos=150, max_enc=225, anchor_layer=1)
+    blob = _blob(dims, 0.05)
+    enc_lens = [225, 31, 32, 33, 96, 97, 129, 160]
+    B = len(enc_lens)
+    enc = W.make_encoder_states(dims, enc_lens, 225)
+    prompt = W.make_prompt(dims, B, length=120)
+    total = [120 + (12 if b < 2 else 3 + b % 3) for b in range(B)]   # two transcripts run past key 128
+    wl = W.Workload("a", dims, B, k, tuple(t - 120 for t in total), tuple(enc_lens), (0.1,) * B, "none")
+    st, _ = run_decode(dims, blob, enc, enc_lens, prompt, total, k, W.make_corruption(wl), _session(dims, blob, B, k),
+                       scale=scale_for(dims, 0.05))
+    _report(f"key blocks k{k}", st)
+    assert st.emitted == sum(wl.n_out)
+    assert_bounded(st)
+
+
 @pytest.mark.parametrize("d,n_layers", [(128, 2), (192, 2)])
 def test_encoder_cache_on_pairs(built_lib, cuda, d, n_layers):
     """Enough frames for the CTA-pair encoder GEMM: blocks of 128 frames that
