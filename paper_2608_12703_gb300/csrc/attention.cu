@@ -220,9 +220,15 @@ void launch_attention_f32(const AttnArgs& a0, cudaStream_t st) {
 // ---------------------------------------------------------------------------
 // Acceptance, commit and anchor readout, fused
 // ---------------------------------------------------------------------------
-// One CTA per (FB encoder frames, utterance).  The anchor layer's encoder keys
-// do not change during a verify call, so each CTA starts copying its frames'
-// keys (all heads) into shared memory before it waits for the LM head.  Then
+// One CTA per (FB encoder frames, utterance), walking the heads through a ring
+// of key blocks ([FB][64], contiguous in the cache).  The anchor layer's encoder
+// keys do not change during a verify call, so the first heads' blocks are
+// requested before the wait on the LM head.  FB = 128 where that still gives
+// every SM a CTA: 64 utterances then read 16 KB per copy from about one wave of
+// CTAs (16 frames of all heads per CTA, 2 KB per copy and 3500 CTAs that each
+// paid the latency of the acceptance and of the queries, took 70 us for 130 MB
+// of keys; 31 us now); FB = 32 with every head's block in flight for few
+// utterances.  After the wait
 // one warp recomputes the accepted length n from the per-row argmax keys (one
 // ballot); the first CTA commits: accepted, bonus, kv_len += 1 + n, pending =
 // bonus (Sec. 3 "Speculative Loop"; a round advances 1 + L tokens, App.
@@ -238,24 +244,17 @@ void launch_attention_f32(const AttnArgs& a0, cudaStream_t st) {
 // row is the path's last node.
 constexpr int ANCHOR_HMAX = 32;   // heads (d_model <= 2048)
 
-template <typename T>
-struct AnchorCfg {
-  static constexpr int FB = sizeof(T) == 2 ? 16 : 8;   // frames per CTA (40 KB of keys for 20 heads)
-  static constexpr int ROW_BYTES = 64 * (int)sizeof(T);
-  static constexpr int SMEM = ANCHOR_HMAX * FB * ROW_BYTES;   // keys [H][FB][64]; <= 64 KB
-};
-
-template <typename T>
+// ST: key blocks in flight per CTA
+template <typename T, int FB>
 __global__ void __launch_bounds__(256)
-accept_anchor_kernel(AcceptAnchorArgs A) {
-  using C = AnchorCfg<T>;
-  constexpr int FB = C::FB;
-  extern __shared__ __align__(128) uint8_t anchor_keys[];
-  __shared__ float qs[ANCHOR_HMAX][64];
-  __shared__ float ph[ANCHOR_HMAX][FB + 1];
+accept_anchor_kernel(AcceptAnchorArgs A, int ST) {
+  constexpr int ROW_BYTES = 64 * (int)sizeof(T), STAGE = FB * ROW_BYTES;
+  extern __shared__ __align__(128) uint8_t anchor_keys[];   // [ST][FB][64]
+  __shared__ __align__(16) float qs[ANCHOR_HMAX][64];
   __shared__ float sM[ANCHOR_HMAX], sL[ANCHOR_HMAX];
-  __shared__ __align__(8) uint64_t bar;
-  __shared__ int s_n, s_node, s_last;
+  __shared__ __align__(8) uint64_t bar[ANCHOR_HMAX];
+  __shared__ unsigned long long s_key[8];
+  __shared__ int s_n, s_node;
   tl_mark(A.tl, TL_ENTRY);
   const int b = blockIdx.y, f0 = blockIdx.x * FB, tid = threadIdx.x;
   const int warp = tid >> 5, lane = tid & 31;
@@ -265,17 +264,18 @@ accept_anchor_kernel(AcceptAnchorArgs A) {
     pdl_wait();
     return;
   }
-  const int rows = min(FB, n_frames - f0) > 0 ? min(FB, n_frames - f0) : 0;
+  const int rows = max(0, min(FB, n_frames - f0));
+  auto issue = [&](int h) {   // thread 0: head h's keys of this CTA's frames
+    mbar_arrive_expect_tx(&bar[h % ST], (uint32_t)(rows * ROW_BYTES));
+    bulk_load(anchor_keys + (h % ST) * STAGE,
+              static_cast<const char*>(A.kc) + (((size_t)b * H + h) * A.t_alloc + f0) * ROW_BYTES,
+              (uint32_t)(rows * ROW_BYTES), &bar[h % ST]);
+  };
   if (tid == 0) {
-    mbar_init(&bar, 1);
+    for (int i = 0; i < ST; ++i) mbar_init(&bar[i], 1);
     fence_mbar_init();
-    if (rows > 0) {
-      mbar_arrive_expect_tx(&bar, (uint32_t)(H * rows * C::ROW_BYTES));
-      const char* kc = static_cast<const char*>(A.kc);
-      for (int h = 0; h < H; ++h)
-        bulk_load(anchor_keys + h * FB * C::ROW_BYTES,
-                  kc + (((size_t)b * H + h) * A.t_alloc + f0) * C::ROW_BYTES, (uint32_t)(rows * C::ROW_BYTES), &bar);
-    }
+    if (rows > 0)
+      for (int h = 0; h < ST && h < H; ++h) issue(h);
   }
   pdl_wait();
   tl_mark(A.tl, TL_WORK);
@@ -292,7 +292,8 @@ accept_anchor_kernel(AcceptAnchorArgs A) {
       A.restart[b] = 0;
     }
     __syncthreads();
-    if (rows > 0) mbar_wait(&bar, 0, A.status);       // no CTA leaves with copies in flight
+    if (rows > 0)
+      for (int i = 0; i < ST && i < H; ++i) mbar_wait(&bar[i], 0, A.status);   // no CTA leaves with copies in flight
     return;
   }
   const int r0 = A.plan.row_start[b];
@@ -366,83 +367,119 @@ accept_anchor_kernel(AcceptAnchorArgs A) {
     sL[tid] = A.ml[((size_t)r * H + tid) * 2 + 1];
   }
   __syncthreads();
-  if (rows > 0) mbar_wait(&bar, 0, A.status);
-  // scores: 8 lanes per (head, frame), each over 8 of the 64 dimensions, so
-  // that a warp reads four consecutive key rows of shared memory at once
+  // scores: 8 lanes per frame, each over 8 of the 64 dimensions
   const int g = lane >> 3, c = lane & 7;
   const float scale = A.kv_bf16 ? 1.f : ATTN_SCALE;
-  for (int base = warp * 4; base < H * FB; base += 32) {   // uniform over the warp
-    const int p = base + g;
-    const int h = p / FB, fr = p - h * FB;
-    const bool ok = p < H * FB && fr < rows;
+  auto prob = [&](const uint8_t* kr, const float4& q0, const float4& q1, float mh, float lh) {
     float s = 0.f;
-    if (ok) {
-      const uint8_t* kr = anchor_keys + (h * FB + fr) * C::ROW_BYTES;
-      const float* qh = qs[h] + 8 * c;
-      if constexpr (sizeof(T) == 2) {
-        const uint4 kv = *reinterpret_cast<const uint4*>(kr + 16 * c);
-        const __nv_bfloat162* k2 = reinterpret_cast<const __nv_bfloat162*>(&kv);
-#pragma unroll
-        for (int w = 0; w < 4; ++w) {
-          const float2 kf = __bfloat1622float2(k2[w]);
-          s = fmaf(qh[2 * w], kf.x, s);
-          s = fmaf(qh[2 * w + 1], kf.y, s);
-        }
-      } else {
-        const float4 k0 = *reinterpret_cast<const float4*>(kr + 32 * c);
-        const float4 k1 = *reinterpret_cast<const float4*>(kr + 32 * c + 16);
-        s = fmaf(qh[0], k0.x, s); s = fmaf(qh[1], k0.y, s); s = fmaf(qh[2], k0.z, s); s = fmaf(qh[3], k0.w, s);
-        s = fmaf(qh[4], k1.x, s); s = fmaf(qh[5], k1.y, s); s = fmaf(qh[6], k1.z, s); s = fmaf(qh[7], k1.w, s);
-      }
+    if constexpr (sizeof(T) == 2) {
+      const uint4 kv = *reinterpret_cast<const uint4*>(kr + 16 * c);
+      const float2 k0 = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&kv.x));
+      const float2 k1 = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&kv.y));
+      const float2 k2 = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&kv.z));
+      const float2 k3 = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&kv.w));
+      s = fmaf(q0.x, k0.x, s); s = fmaf(q0.y, k0.y, s); s = fmaf(q0.z, k1.x, s); s = fmaf(q0.w, k1.y, s);
+      s = fmaf(q1.x, k2.x, s); s = fmaf(q1.y, k2.y, s); s = fmaf(q1.z, k3.x, s); s = fmaf(q1.w, k3.y, s);
+    } else {
+      const float4 k0 = *reinterpret_cast<const float4*>(kr + 32 * c);
+      const float4 k1 = *reinterpret_cast<const float4*>(kr + 32 * c + 16);
+      s = fmaf(q0.x, k0.x, s); s = fmaf(q0.y, k0.y, s); s = fmaf(q0.z, k0.z, s); s = fmaf(q0.w, k0.w, s);
+      s = fmaf(q1.x, k1.x, s); s = fmaf(q1.y, k1.y, s); s = fmaf(q1.z, k1.z, s); s = fmaf(q1.w, k1.w, s);
     }
     s += __shfl_xor_sync(0xffffffffu, s, 1);
     s += __shfl_xor_sync(0xffffffffu, s, 2);
     s += __shfl_xor_sync(0xffffffffu, s, 4);
-    if (c == 0 && p < H * FB) ph[h][fr] = ok ? expf(s * scale - sM[h]) / sL[h] : 0.f;
-  }
-  __syncthreads();
-  if (warp == 0) {
-    float pbar = 0.f;
-    const int fr = lane < FB ? lane : 0;
-    for (int h = 0; h < H; ++h) pbar += ph[h][fr];
-    pbar /= (float)H;
-    if (lane < rows) A.profile[(size_t)b * A.t_alloc + f0 + lane] = pbar;
-    unsigned long long key = lane < rows ? argmax_key(pbar, (uint32_t)(f0 + lane)) : 0ull;
-    key = warp_max_u64(key);
-    if (lane == 0) {
-      const int n_cta = n_frames > FB ? (n_frames + FB - 1) / FB : 1;   // CTAs of this utterance that take part
-      atomicMax(A.frame_key + b, key);
-      __threadfence();
-      s_last = (atomicAdd(A.tickets + b, 1) == n_cta - 1);
-      if (s_last) {
-        __threadfence();
-        const unsigned long long fk = atomicExch(A.frame_key + b, 0ull);
-        A.anchor_out[b] = (int)argmax_index(fk);
-        A.tickets[b] = 0;
+    return expf(s * scale - mh) / lh;   // past the frames: stale keys, not used
+  };
+  unsigned long long best = 0ull;
+  auto keep = [&](int fr, float sum) {   // one frame's head mean
+    const float pm = sum / (float)H;
+    A.profile[(size_t)b * A.t_alloc + f0 + fr] = pm;
+    const unsigned long long key = argmax_key(pm, (uint32_t)(f0 + fr));
+    best = key > best ? key : best;
+  };
+  // NP passes of 4 frames per warp and head.  FB = 128: the warps share each
+  // head's frames, heads summed in order.  FB = 32: a warp takes every eighth
+  // head over all frames (short serial chains), the warps summed in order.
+  constexpr bool BY_HEAD = FB == 32;
+  constexpr int NP = BY_HEAD ? FB / 4 : FB / 32;
+  __shared__ float s_p[BY_HEAD ? 8 : 1][BY_HEAD ? FB : 1];
+  float pbar[NP];
+#pragma unroll
+  for (int i = 0; i < NP; ++i) pbar[i] = 0.f;
+  for (int h0 = 0; h0 < H && rows > 0; h0 += BY_HEAD ? 8 : 1) {
+    const int h = BY_HEAD ? h0 + warp : h0;
+    if (h < H) {
+      const uint8_t* keys = anchor_keys + (h % ST) * STAGE;
+      const float4 q0 = *reinterpret_cast<const float4*>(&qs[h][8 * c]);
+      const float4 q1 = *reinterpret_cast<const float4*>(&qs[h][8 * c + 4]);
+      const float mh = sM[h], lh = sL[h];
+      mbar_wait(&bar[h % ST], (h / ST) & 1, A.status);
+      __syncwarp();
+#pragma unroll
+      for (int i = 0; i < NP; ++i) {
+        const int fr = BY_HEAD ? i * 4 + g : i * 32 + warp * 4 + g;
+        pbar[i] += prob(keys + fr * ROW_BYTES, q0, q1, mh, lh);
       }
+    }
+    if (h0 + ST < H) {   // ST is a multiple of 8 where it is less than H (FB = 32)
+      __syncthreads();   // the blocks are free
+      if (tid == 0)
+        for (int i = h0 + ST; i < H && i < h0 + ST + (BY_HEAD ? 8 : 1); ++i) issue(i);
+    }
+  }
+  if constexpr (BY_HEAD) {
+    if (c == 0)
+#pragma unroll
+      for (int i = 0; i < NP; ++i) s_p[warp][i * 4 + g] = pbar[i];
+    __syncthreads();
+    if (tid < rows) {
+      float sum = 0.f;
+      for (int w = 0; w < 8; ++w) sum += s_p[w][tid];
+      keep(tid, sum);
+    }
+  } else {
+#pragma unroll
+    for (int i = 0; i < NP; ++i) {
+      const int fr = i * 32 + warp * 4 + g;
+      if (fr < rows && c == 0) keep(fr, pbar[i]);
+    }
+  }
+  best = warp_max_u64(best);
+  if (lane == 0) s_key[warp] = best;
+  __syncthreads();
+  if (tid == 0) {
+    for (int w = 1; w < 8; ++w) best = s_key[w] > best ? s_key[w] : best;
+    const int n_cta = n_frames > FB ? (n_frames + FB - 1) / FB : 1;   // CTAs of this utterance that take part
+    atomicMax(A.frame_key + b, best);
+    __threadfence();
+    if (atomicAdd(A.tickets + b, 1) == n_cta - 1) {
+      __threadfence();
+      const unsigned long long fk = atomicExch(A.frame_key + b, 0ull);
+      A.anchor_out[b] = (int)argmax_index(fk);
+      A.tickets[b] = 0;
     }
   }
   tl_mark(A.tl, TL_EXIT);
 }
 
-void launch_accept_anchor(const AcceptAnchorArgs& A, cudaStream_t st) {
+template <typename T, int FB>
+static void launch_accept_t(const AcceptAnchorArgs& A, cudaStream_t st) {
+  // FB = 128: four blocks, three CTAs per SM (bf16).  FB = 32: up to every head's block at once.
+  constexpr int STAGE = FB * 64 * (int)sizeof(T), ST_MAX = FB == 128 ? 4 : 128 * 1024 / STAGE;
   static std::once_flag once;
   std::call_once(once, [] {
-    cudaFuncSetAttribute(accept_anchor_kernel<__nv_bfloat16>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         AnchorCfg<__nv_bfloat16>::SMEM);
-    cudaFuncSetAttribute(accept_anchor_kernel<float>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         AnchorCfg<float>::SMEM);
+    cudaFuncSetAttribute(accept_anchor_kernel<T, FB>, cudaFuncAttributeMaxDynamicSharedMemorySize, ST_MAX * STAGE);
   });
-  if (A.kv_bf16) {
-    using C = AnchorCfg<__nv_bfloat16>;
-    dim3 grid((A.t_alloc + C::FB - 1) / C::FB, A.B);
-    launch_ex(accept_anchor_kernel<__nv_bfloat16>, grid, dim3(256), (size_t)A.H * C::FB * C::ROW_BYTES, st, A.pdl, 1,
-              A);
-  } else {
-    using C = AnchorCfg<float>;
-    dim3 grid((A.t_alloc + C::FB - 1) / C::FB, A.B);
-    launch_ex(accept_anchor_kernel<float>, grid, dim3(256), (size_t)A.H * C::FB * C::ROW_BYTES, st, A.pdl, 1, A);
-  }
+  const int ST = A.H < ST_MAX ? A.H : ST_MAX;
+  launch_ex(accept_anchor_kernel<T, FB>, dim3((A.t_alloc + FB - 1) / FB, A.B), dim3(256), (size_t)(ST * STAGE), st,
+            A.pdl, 1, A, ST);
+}
+
+void launch_accept_anchor(const AcceptAnchorArgs& A, cudaStream_t st) {
+  const bool wide = (long long)A.B * ((A.t_alloc + 127) / 128) >= 152;
+  if (A.kv_bf16) wide ? launch_accept_t<__nv_bfloat16, 128>(A, st) : launch_accept_t<__nv_bfloat16, 32>(A, st);
+  else wide ? launch_accept_t<float, 128>(A, st) : launch_accept_t<float, 32>(A, st);
 }
 
 // Tree verify commit: one warp per (utterance, layer, head) moves the accepted

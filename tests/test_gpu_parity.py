@@ -153,6 +153,25 @@ def test_attention_key_blocks(built_lib, cuda, k):
     assert_bounded(st)
 
 
+@pytest.mark.parametrize("batch,t_max", [(39, 400), (1, 33), (2, 32)])
+@pytest.mark.parametrize("dtype", ["bf16", "fp32"])
+def test_anchor_readout_sizes(built_lib, cuda, dtype, batch, t_max):
+    """The anchor readout over 128 frames per CTA (from 152 CTAs on) and over
+    32, frames that end inside and at a block; every anchor and profile."""
+    dims = W.ModelDims(n_layers=1, d_model=128, n_heads=2, d_ffn=512, vocab=300, dtype=dtype,
+                       max_pos=24, max_enc=t_max, anchor_layer=0)
+    blob = _blob(dims, 0.1)
+    enc_lens = [max(1, t_max - 31 * b) for b in range(batch)]
+    enc = W.make_encoder_states(dims, enc_lens, t_max)
+    prompt = W.make_prompt(dims, batch)
+    total = [W.PROMPT_LEN + 2] * batch
+    wl = W.Workload("r", dims, batch, 2, (2,) * batch, tuple(enc_lens), (0.2,) * batch, "half")
+    st, _ = run_decode(dims, blob, enc, enc_lens, prompt, total, 2, W.make_corruption(wl),
+                       _session(dims, blob, batch, 2), scale=scale_for(dims, 0.1))
+    _report(f"anchor readout {dtype} b{batch} t{t_max}", st)
+    assert_bounded(st)
+
+
 @pytest.mark.parametrize("d,n_layers", [(128, 2), (192, 2)])
 def test_encoder_cache_on_pairs(built_lib, cuda, d, n_layers):
     """Enough frames for the CTA-pair encoder GEMM: blocks of 128 frames that
