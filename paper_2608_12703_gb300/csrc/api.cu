@@ -77,7 +77,7 @@ struct asr_spec {
   unsigned long long* frame_key = nullptr;  // [Bmax] keys + [Bmax] int tickets
   int* anchor_row = nullptr;
   // out4: accepted, bonus, kv_len, anchor and restart of the last verify, [Bmax] each
-  int *draft_buf = nullptr, *lens_buf = nullptr, *prompt_buf = nullptr, *out4 = nullptr, *misc = nullptr;
+  int *draft_buf = nullptr, *lens_buf = nullptr, *prompt_buf = nullptr, *out4 = nullptr;
   float* anchor_prof = nullptr;   // [Bmax][Tmax] head-mean profile of the last verify's anchor rows
   int* status = nullptr;
   float* ws = nullptr;
@@ -1203,7 +1203,7 @@ int asr_spec_create(const asr_model_dims* dims, const asr_weights* weights, void
     return finish(rc);
   if ((rc = dalloc(h, &h->draft_buf, (size_t)h->Bmax * std::max(h->kmax, 1) * 4)) ||
       (rc = dalloc(h, &h->lens_buf, h->Bmax * 4)) || (rc = dalloc(h, &h->prompt_buf, (size_t)h->Bmax * h->maxpos * 4)) ||
-      (rc = dalloc(h, &h->out4, 5 * h->Bmax * 4)) || (rc = dalloc(h, &h->misc, 64 * 4)) ||
+      (rc = dalloc(h, &h->out4, 5 * h->Bmax * 4)) ||
       (rc = dalloc(h, &h->anchor_prof, (size_t)h->Bmax * h->Tmax * 4)) ||
       (rc = dalloc(h, &h->status, 4)))
     return finish(rc);
@@ -1400,18 +1400,28 @@ int asr_spec_prefill(asr_spec_handle h, const int32_t* prompt, int32_t P0) {
 
 namespace {
 
+// Aligned for int32 loads and stores by a kernel.
+bool words(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 3) == 0; }
+
 // The verify call: inputs into the internal buffers, the body (a CUDA graph per
 // (B, k, linear or tree), captured on first use), outputs out.
 int verify_call(asr_spec* h, const int32_t* draft, const int32_t* parent, const int32_t* lens, int32_t k,
                 int32_t* accepted, int32_t* bonus, int32_t* kv_len, int32_t* anchor, int32_t* path) {
   const bool tree = parent != nullptr;
   const int B = h->B;
-  if (k > 0) {
-    if (int rc = copy_in(h, h->draft_buf, draft, (size_t)B * k)) return rc;
-    if (tree)
-      if (int rc = copy_in(h, h->parent_buf, parent, (size_t)B * k)) return rc;
+  // device arrays: one launch each way (a copy each took 2 to 3 us of the stream); host ones: copies
+  const bool by_kernel = !h->host_io && words(draft) && words(parent) && words(lens) && words(accepted) &&
+                         words(bonus) && words(kv_len) && words(anchor) && words(path);
+  if (by_kernel) {
+    launch_copy_in(draft, parent, B * k, lens, B, h->draft_buf, h->parent_buf, h->lens_buf, h->st);
+  } else {
+    if (k > 0) {
+      if (int rc = copy_in(h, h->draft_buf, draft, (size_t)B * k)) return rc;
+      if (tree)
+        if (int rc = copy_in(h, h->parent_buf, parent, (size_t)B * k)) return rc;
+    }
+    if (int rc = copy_in(h, h->lens_buf, lens, B)) return rc;
   }
-  if (int rc = copy_in(h, h->lens_buf, lens, B)) return rc;
   for (int c = 0; c < ASR_PROF_N; ++c) h->cur[c] = 0;
   struct TreeScope {   // the enqueued layers read cur_tree; cleared on every way out
     asr_spec* h;
@@ -1450,12 +1460,19 @@ int verify_call(asr_spec* h, const int32_t* draft, const int32_t* parent, const 
   }
   CK(cudaGetLastError());
   int* o = h->out4;
-  if (int rc = copy_out(h, accepted, o, B)) return rc;
-  if (int rc = copy_out(h, bonus, o + h->Bmax, B)) return rc;
-  if (int rc = copy_out(h, kv_len, o + 2 * h->Bmax, B)) return rc;
-  if (int rc = copy_out(h, anchor, o + 3 * h->Bmax, B)) return rc;
-  if (tree && path && k > 0)
-    if (int rc = copy_out(h, path, h->path_buf, (size_t)B * k)) return rc;
+  const bool with_path = tree && path && k > 0;
+  if (by_kernel) {
+    launch_copy_out(o, h->Bmax, h->path_buf, B * k, B, accepted, bonus, kv_len, anchor, with_path ? path : nullptr,
+                    h->st);
+    CK(cudaGetLastError());
+  } else {
+    if (int rc = copy_out(h, accepted, o, B)) return rc;
+    if (int rc = copy_out(h, bonus, o + h->Bmax, B)) return rc;
+    if (int rc = copy_out(h, kv_len, o + 2 * h->Bmax, B)) return rc;
+    if (int rc = copy_out(h, anchor, o + 3 * h->Bmax, B)) return rc;
+    if (with_path)
+      if (int rc = copy_out(h, path, h->path_buf, (size_t)B * k)) return rc;
+  }
   h->d_after_verify = h->has_draft && !tree;
   if (!tree) h->last_k = k;
   if (h->host_io) CK(cudaStreamSynchronize(h->st));
@@ -1822,10 +1839,15 @@ int asr_spec_rollback(asr_spec_handle h, const int32_t* new_len, const int32_t* 
   if (!h) return ASR_E_INVAL;
   if (h->state < 2) return fail(h, ASR_E_STATE, "rollback before prefill");
   if (!new_len || !new_pending) return fail(h, ASR_E_INVAL, "null pointer");
-  if (int rc = copy_in(h, h->misc, new_len, h->B)) return rc;
-  if (int rc = copy_in(h, h->lens_buf, new_pending, h->B)) return rc;
+  const int *nl = new_len, *np = new_pending;
+  if (h->host_io || !words(new_len) || !words(new_pending)) {
+    if (int rc = copy_in(h, h->prompt_buf, new_len, h->B)) return rc;
+    if (int rc = copy_in(h, h->lens_buf, new_pending, h->B)) return rc;
+    nl = h->prompt_buf;
+    np = h->lens_buf;
+  }
   Prof p(h, ASR_PROF_OTHER, 1);
-  launch_rollback(h->misc, h->lens_buf, h->B, h->V, h->kv_len, h->pending, h->status, h->st);
+  launch_rollback(nl, np, h->B, h->V, h->kv_len, h->pending, h->status, h->st);
   CK(cudaGetLastError());
   h->d_after_verify = false;   // the draft has no verification rows of the rewound state
   if (h->host_io) CK(cudaStreamSynchronize(h->st));

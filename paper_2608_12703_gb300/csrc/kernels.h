@@ -105,6 +105,13 @@ void launch_plan_verify(const int* draft, const int* lens, int k, int B, int voc
                         const int* pending, const int* ready, RowPlan plan, unsigned long long* row_key,
                         int* status, const TrafficArgs& tr, cudaStream_t st, unsigned long long* tl = nullptr,
                         const int* parent = nullptr);
+// The call's inputs into the handle's buffers (draft and parent [n], lens [B];
+// parent may be null), and its outputs ([B] each, stride out_stride in out4;
+// path [n] or null) to the caller's, one launch each.
+void launch_copy_in(const int* draft, const int* parent, int n, const int* lens, int B, int* draft_buf, int* parent_buf,
+                    int* lens_buf, cudaStream_t st);
+void launch_copy_out(const int* out4, int out_stride, const int* path_buf, int n, int B, int* accepted, int* bonus,
+                     int* kv_len, int* anchor, int* path, cudaStream_t st);
 void launch_plan_prefill_chunk(const int* prompt, int P0, int p0, int c, int B, int vocab, const int* ready,
                                RowPlan plan, int* status, cudaStream_t st);
 // xg / gain / st_part: the folded first LayerNorm's operand bf16(gain * x) [R][d]

@@ -1,6 +1,8 @@
 // Row bookkeeping of the verify step: input validation and row layout,
 // embeddings, LayerNorm, greedy longest-prefix acceptance with the KV-length
 // commit, rollback, and the synthetic draft source used by benchmarks.
+#include <algorithm>
+
 #include "kernels.h"
 
 namespace asrspec {
@@ -49,28 +51,36 @@ plan_verify_kernel(const int* __restrict__ draft, const int* __restrict__ lens, 
                    unsigned long long* tl, const int* __restrict__ parent) {
   __shared__ int s_err;
   __shared__ unsigned long long s_cnt[4];
+  __shared__ int s_n[PLAN_THREADS], s_start[PLAN_THREADS], s_kv[PLAN_THREADS];   // per utterance
   tl_mark(tl, TL_ENTRY);
   tl_mark(tl, TL_WORK);
   if (threadIdx.x == 0) s_err = 0;
   if (threadIdx.x < 4) s_cnt[threadIdx.x] = 0;
   __syncthreads();
   const int b = threadIdx.x;
-  int n_b = 0, err = 0;
+  int n_b = 0, err = 0, kv = 0;
   if (b < B) {
     const int l = lens[b];
+    kv = kv_len[b];
     if (l < -1 || l > k) err |= ST_BAD_LENS;
     else if (l >= 0) {
       if (!ready[b]) err |= ST_NOT_READY;
-      if (kv_len[b] + l + 1 > max_pos) err |= ST_CAPACITY;
-      for (int i = 0; i < l; ++i) {
-        const int t = draft[(size_t)b * k + i];
-        if (t < 0 || t >= vocab) err |= ST_BAD_TOKEN;
-        if (parent != nullptr) {
-          const int p = parent[(size_t)b * k + i];
-          if (p < 0 || p > i) err |= ST_BAD_TREE;
-        }
-      }
+      if (kv + l + 1 > max_pos) err |= ST_CAPACITY;
       n_b = l + 1;
+    }
+    s_n[b] = n_b;
+    s_kv[b] = kv;
+  }
+  __syncthreads();
+  // the drafts, one per thread and step (a thread per utterance took 14 us for 64 x 6)
+  for (int e = threadIdx.x; e < B * k; e += PLAN_THREADS) {
+    const int u = e / k, i = e - u * k;
+    if (i + 1 >= s_n[u]) continue;
+    const int t = draft[e];
+    if (t < 0 || t >= vocab) err |= ST_BAD_TOKEN;
+    if (parent != nullptr) {
+      const int p = parent[e];
+      if (p < 0 || p > i) err |= ST_BAD_TREE;
     }
   }
   if (err) atomicOr(&s_err, err);
@@ -81,41 +91,55 @@ plan_verify_kernel(const int* __restrict__ draft, const int* __restrict__ lens, 
   }
   int total;
   const int start = block_excl_scan(n_b, &total);
+  unsigned long long cnt[4] = {0, 0, 0, 0};
   if (b < B) {
     plan.row_start[b] = start;
     plan.n_utt_rows[b] = n_b;
-    int depth[32];
-    unsigned anc[32];
-    for (int i = 0; i < n_b; ++i) {
-      const int r = start + i;
-      plan.row_b[r] = b;
-      plan.row_i[r] = i;
-      plan.row_pos[r] = kv_len[b] + i;
-      plan.row_tok[r] = i == 0 ? pending[b] : draft[(size_t)b * k + i - 1];
-      if (parent != nullptr) {   // n_b <= 32 (k <= 31)
-        const int p = i == 0 ? 0 : parent[(size_t)b * k + i - 1];
-        depth[i] = i == 0 ? 0 : depth[p] + 1;
-        anc[i] = (i == 0 ? 0u : anc[p]) | (1u << i);
-        plan.row_epos[r] = kv_len[b] + depth[i];
-        plan.row_mask[r] = anc[i];
-      } else {
-        plan.row_epos[r] = kv_len[b] + i;
-      }
-      row_key[r] = 0ull;
-    }
+    s_start[b] = start;
+    s_n[b] = n_b;
     if (n_b > 0 && tr.counters) {
       // algorithmic bytes of this utterance: self K/V read over the visible
       // keys of all layers, encoder K/V read by cross-attention, and one
       // anchor-layer key pass
       const unsigned long long es = (unsigned long long)tr.elem_bytes, d = tr.d, L = tr.n_layers;
       const unsigned long long T = (unsigned long long)tr.enc_len[b];
-      atomicAdd(&s_cnt[0], 2ull * L * (unsigned long long)(kv_len[b] + n_b) * d * es);
-      atomicAdd(&s_cnt[1], 2ull * L * T * d * es);
-      atomicAdd(&s_cnt[2], T * d * es);
-      atomicAdd(&s_cnt[3], (unsigned long long)n_b);
+      cnt[0] = 2ull * L * (unsigned long long)(kv + n_b) * d * es;
+      cnt[1] = 2ull * L * T * d * es;
+      cnt[2] = T * d * es;
+      cnt[3] = (unsigned long long)n_b;
     }
   }
+  // a warp's sums first: 64-bit shared atomics from every utterance serialise
+  if (tr.counters && (threadIdx.x & ~31) < B)   // uniform over the warp
+#pragma unroll
+    for (int c = 0; c < 4; ++c) {
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) cnt[c] += __shfl_xor_sync(0xffffffffu, cnt[c], o);
+      if ((threadIdx.x & 31) == 0 && cnt[c]) atomicAdd(&s_cnt[c], cnt[c]);
+    }
   __syncthreads();
+  for (int e = threadIdx.x; e < B * (k + 1); e += PLAN_THREADS) {
+    const int u = e / (k + 1), i = e - u * (k + 1);
+    if (i >= s_n[u]) continue;
+    const int r = s_start[u] + i, P = s_kv[u];
+    plan.row_b[r] = u;
+    plan.row_i[r] = i;
+    plan.row_pos[r] = P + i;
+    plan.row_tok[r] = i == 0 ? pending[u] : draft[(size_t)u * k + i - 1];
+    if (parent != nullptr) {   // at most 32 nodes; the checked parents lead to the root
+      int depth = 0;
+      unsigned anc = 1u << i;
+      for (int j = i; j > 0; ++depth) {
+        j = parent[(size_t)u * k + j - 1];
+        anc |= 1u << j;
+      }
+      plan.row_epos[r] = P + depth;
+      plan.row_mask[r] = anc;
+    } else {
+      plan.row_epos[r] = P + i;
+    }
+    row_key[r] = 0ull;
+  }
   if (threadIdx.x == 0) {
     plan.row_start[B] = total;
     *plan.n_rows = total;
@@ -125,6 +149,37 @@ plan_verify_kernel(const int* __restrict__ draft, const int* __restrict__ lens, 
     }
   }
   tl_mark(tl, TL_EXIT);
+}
+
+__global__ void copy_in_kernel(const int* __restrict__ draft, const int* __restrict__ parent, int n,
+                               const int* __restrict__ lens, int B, int* draft_buf, int* parent_buf, int* lens_buf) {
+  const int e = blockIdx.x * blockDim.x + threadIdx.x;
+  if (e < n) {
+    draft_buf[e] = draft[e];
+    if (parent) parent_buf[e] = parent[e];
+  }
+  if (e < B) lens_buf[e] = lens[e];
+}
+void launch_copy_in(const int* draft, const int* parent, int n, const int* lens, int B, int* draft_buf, int* parent_buf,
+                    int* lens_buf, cudaStream_t st) {
+  copy_in_kernel<<<(std::max(n, B) + 255) / 256, 256, 0, st>>>(draft, parent, n, lens, B, draft_buf, parent_buf,
+                                                               lens_buf);
+}
+__global__ void copy_out_kernel(const int* __restrict__ out4, int stride, const int* __restrict__ path_buf, int n, int B,
+                                int* accepted, int* bonus, int* kv_len, int* anchor, int* path) {
+  const int e = blockIdx.x * blockDim.x + threadIdx.x;
+  if (e < B) {
+    accepted[e] = out4[e];
+    bonus[e] = out4[stride + e];
+    kv_len[e] = out4[2 * stride + e];
+    anchor[e] = out4[3 * stride + e];
+  }
+  if (path && e < n) path[e] = path_buf[e];
+}
+void launch_copy_out(const int* out4, int out_stride, const int* path_buf, int n, int B, int* accepted, int* bonus,
+                     int* kv_len, int* anchor, int* path, cudaStream_t st) {
+  copy_out_kernel<<<(std::max(path ? n : 0, B) + 255) / 256, 256, 0, st>>>(out4, out_stride, path_buf, n, B, accepted,
+                                                                         bonus, kv_len, anchor, path);
 }
 
 // Prefill rows: prompt tokens p0 .. p0+c-1 of every utterance at positions p0 + i.

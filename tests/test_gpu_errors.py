@@ -180,3 +180,29 @@ def test_timeline_records_every_launch_in_order(built_lib, cuda):
     assert np.all(mid[has_mid] <= end[has_mid])
     slack = 2000   # ns: the timer is global, CTAs on different SMs read it
     assert np.all(work[1:] >= end[:-1] - slack)
+
+
+def test_rollback_of_many_utterances(built_lib, cuda):
+    """Every utterance of a large batch is rewound (the call's arrays are as long as the batch)."""
+    from paper_2608_12703_gb300.session import Session
+    dims = W.ModelDims(n_layers=1, d_model=128, n_heads=2, d_ffn=256, vocab=200, dtype="bf16",
+                       max_pos=32, max_enc=20, anchor_layer=0)
+    B = 300
+    sess = Session(dims, W.make_weights(dims, std=0.1), max_batch=B, max_draft=2)
+    sess.encode_cache(W.make_encoder_states(dims, [20] * B, 20), [20] * B)
+    sess.prefill(W.make_prompt(dims, B, length=9))
+    new_len = np.arange(B, dtype=np.int32) % 9
+    new_len[7] = -1
+    pending = (np.arange(B, dtype=np.int32) * 3) % 200
+    kv0, pe0 = sess.state()
+    for host_io in (False, True):
+        sess.set_host_io(host_io)
+        sess.rollback(new_len, pending)
+        kv, pe = sess.state()
+        want_kv, want_pe = new_len.copy(), pending.copy()
+        want_kv[7], want_pe[7] = kv0[7], pe0[7]
+        np.testing.assert_array_equal(kv, want_kv)
+        np.testing.assert_array_equal(pe, want_pe)
+    sess.set_host_io(False)
+    assert sess.status() == 0
+    sess.close()
