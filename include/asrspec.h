@@ -294,8 +294,8 @@ void asr_spec_destroy(asr_spec_handle h);
 #define ASR_PROF_LMHEAD 6     /* LM head with fused argmax */
 #define ASR_PROF_LAYERNORM 7  /* stand-alone LayerNorm */
 #define ASR_PROF_OTHER 8      /* row plan, embedding, accept + anchor, encoder cache build, prefill steps */
-#define ASR_PROF_QKV_SELF 9   /* few rows: LayerNorm + QKV projection + self-attention, one cluster per head */
-#define ASR_PROF_QUERY_CROSS 10  /* few rows: LayerNorm + cross query + cross-attention, one cluster per head */
+#define ASR_PROF_QKV_SELF 9   /* few rows: LayerNorm + QKV projection + self-attention (one stage, two launches) */
+#define ASR_PROF_QUERY_CROSS 10  /* few rows: LayerNorm + cross query + cross-attention (one stage, two launches) */
 #define ASR_PROF_N 11
 int asr_spec_set_graphs(asr_spec_handle h, int enable);
 int asr_spec_profile(asr_spec_handle h, int enable);
@@ -323,8 +323,8 @@ int asr_spec_profile_read(asr_spec_handle h, double* ms, int64_t* launches, uint
 #define ASR_TL_ATTN_SELF 4     /* self-attention */
 #define ASR_TL_ATTN_CROSS 5    /* cross-attention */
 #define ASR_TL_ACCEPT 6        /* acceptance, commit and anchor readout */
-#define ASR_TL_QKV_SELF 8      /* few rows: LayerNorm + QKV + self-attention, one cluster per head */
-#define ASR_TL_QUERY_CROSS 9   /* few rows: LayerNorm + cross query + cross-attention, one cluster per head */
+#define ASR_TL_QKV_SELF 8      /* few rows: LayerNorm + QKV + self-attention (two launches, one record) */
+#define ASR_TL_QUERY_CROSS 9   /* few rows: LayerNorm + cross query + cross-attention (two launches, one record) */
 #define ASR_TL_GEMM 16         /* + epilogue: 0 plain, 1 QKV + cache append, 2 residual, 3 query, 4 GELU, 6 argmax */
 #define ASR_TL_LN_FUSED 32     /* added to a GEMM kind whose input LayerNorm is folded into it (no LayerNorm launch) */
 int asr_spec_timeline(asr_spec_handle h, int32_t enable);
@@ -332,22 +332,21 @@ int asr_spec_timeline_read(asr_spec_handle h, uint64_t* ns, int32_t* kind, int32
 
 
 /* ---- Diagnostics of the few-row layers (not part of the paper's method) ---
- * asr_spec_fewrow_trace: when enabled, every verify that runs the few-row
- * layers (bf16 models, batch x (k + 1) <= 9 rows) records, per CTA of each of
- * its 6 L layer launches, the GPU global timer (ns) at 12 phases: entry, past
- * the wait on the previous launch, input rows ready, weights landed,
- * projection reduced, exchange landed, attention done, exit, first K/V chunk
- * landed, first chunk combined, merge inputs landed, bf16 input rows landed
- * (GEMVs without a LayerNorm) (0 where a launch has no such phase); verify
- * then launches directly (no graph).  A
- * verify of more rows records its 6 L tensor-core projections instead (in
- * layer order: QKV, self out, cross query, cross out, MLP up, MLP down), for
- * their first 320 CTAs: 0 entry, 1 set-up done, 2 first k-block landed,
+ * asr_spec_fewrow_trace: when enabled, every verify of a bf16 model records, per
+ * CTA of the projections of each layer (in layer order: QKV, self out, cross
+ * query, cross out, MLP up, MLP down; their first 320 CTAs), the GPU global
+ * timer (ns) at 12 phases (0 where a launch has no such phase); verify then
+ * launches directly (no graph).  Tensor-core projections (all of them, or with
+ * the few-row layers, batch x (k + 1) <= 9 rows, QKV and the cross query):
+ * 0 entry, 1 set-up done, 2 first k-block landed,
  * 3 MMAs done, 4 exit, 5 K-split partial staged (one CTA per tile: tile
  * staged in shared memory), 6 partials landed (staging barrier passed),
  * 7 reduction done (rows written), 8 past the wait on the previous launch,
- * 9 last k-block issued, 10 epilogue operands loaded, 11 first rows written
- * (many-row kernel).  ASR_E_INVAL for an fp32 model.
+ * 9 last k-block issued, 10 epilogue operands loaded, 11 first rows written.
+ * GEMVs of the few-row layers: 0 entry, 1 past the wait on the previous
+ * launch, 2 input rows ready, 3 weights landed, 4 projection reduced,
+ * 5 exchange landed, 7 exit, 11 bf16 input rows landed.  ASR_E_INVAL for an
+ * fp32 model.
  * asr_spec_fewrow_trace_read: synchronise and copy the last traced call's
  * stamps, [n_launches][320 CTAs][12] words in launch order, up to `cap` words. */
 int asr_spec_fewrow_trace(asr_spec_handle h, int32_t enable);

@@ -30,7 +30,7 @@ struct LayerW {
   float *c1_qkv = nullptr, *c2_qkv = nullptr, *c1_cq = nullptr, *c2_cq = nullptr, *c1_fc1 = nullptr, *c2_fc1 = nullptr;
   CUtensorMap m_wqkv, m_wo, m_wcq, m_wco, m_w1, m_w2;
   // the same weights packed for the few-row kernels (launch_fr_pack), or null
-  void *p_qkv = nullptr, *p_wo = nullptr, *p_wcq = nullptr, *p_wco = nullptr, *p_w1 = nullptr, *p_w2 = nullptr;
+  void *p_wo = nullptr, *p_wco = nullptr, *p_w1 = nullptr, *p_w2 = nullptr;
 };
 
 }  // namespace
@@ -90,7 +90,7 @@ struct asr_spec {
   std::map<std::pair<int, int>, CUtensorMap> xmaps;   // (target 0 / draft 1, BN) -> map of its residual stream (fp32, box 128 x BN)
   int n_sms = 0;
   bool use_wide = true;   // many-row projections on the one-tile-per-SM kernel (ASRSPEC_WIDE=0: the split-K chain)
-  int fr_prefetch = 3;    // few-row launches prefetch the weights of the launch this many ahead into L2 (0: none)
+  int fr_prefetch = 6;    // few-row launches prefetch the weights of the launch this many ahead into L2 (0: none)
   int wide_stages = 0;    // its stages per pipeline (ASRSPEC_WIDE_STAGES; 0 = as deep as shared memory allows)
 
   // profiling: CUDA events around each kernel class (direct launches only)
@@ -112,12 +112,10 @@ struct asr_spec {
   bool ln_fold = false;
   float2* ln_part = nullptr;
   int ln_S = 0, ln_c = 0;
-  // few-row verify layers (csrc/fewrow.cu) for steps of at most VF_ROWS rows:
-  // the cluster size per head (0 = unavailable for this model or device);
+  // few-row verify layers (csrc/fewrow.cu) for steps of at most VF_ROWS rows;
   // ASRSPEC_FEWROW=0 keeps the tensor-core chain for every step
   bool use_fewrow = true;
-  int fr_C = 0;
-  int fr_sms = 0;   // SMs of the device: the GEMVs run one CTA (group) per SM
+  int fr_sms = 0;   // SMs of the device: the GEMVs run one CTA (group) per SM (0: not for this model or device)
   int fr_gd = 0;    // groups of the MLP down-projection (clusters resident at once)
   bool last_fused = false;    // the last verify ran the few-row layers (LM-head input in xf)
   // per-CTA phase stamps of the few-row launches of the last traced call
@@ -294,6 +292,33 @@ unsigned long long* trace_slot(asr_spec* h) {
 }
 
 // One projection over the verify rows: out-features m (weights = A), rows n (activations = B).
+// One projection over the verify rows on the many-row kernel (the caller records profile and timeline).
+int wide_rows(asr_spec* h, const CUtensorMap* mW, int M, int K, const void* X, int x_id, int N, int mode, Epi epi) {
+  WideGemm w{};
+  if (!wide_pick(M, N, K, mode, h->n_sms, &w.bn, &w.split)) return fail(h, ASR_E_CUDA, "no tile for this projection");
+  const CUtensorMap* mb = bmap(h, x_id, X, h->R_pad, K, w.bn);
+  const CUtensorMap* mx = mode == EPI_RESID ? xmap(h, epi.x, w.bn) : mW;
+  if (!mb || !mx) return fail(h, ASR_E_CUDA, "tensor map encode failed");
+  epi.M = M;
+  epi.N = N;
+  epi.status = h->status;
+  if (mode == EPI_QKV) epi.b_max = h->Bmax;
+  if (!epi.trace) epi.trace = trace_slot(h);
+  w.mapA = *mW;
+  w.mapB = *mb;
+  w.mapX = *mx;
+  w.M = M;
+  w.N = N;
+  w.K = K;
+  w.pdl = h->use_pdl;
+  w.stages = h->wide_stages;
+  launch_gemm_wide(w, mode, epi, h->status, h->st);
+  return 0;
+}
+
+// A launch inside a stage whose Prof counts one.
+void count_launch(asr_spec* h) { (h->capturing ? h->cur : h->launches)[ASR_PROF_OTHER] += 1; }
+
 // ln_g / ln_b (fp32 models, f32_rows only): X holds the rows x and the operand is LayerNorm(x).
 int gemm_rows(asr_spec* h, const void* W, const CUtensorMap* mW, int M, int K, const void* X, int x_id, int N,
               int mode, const Epi& epi_in, const float* ln_g = nullptr, const float* ln_b = nullptr) {
@@ -302,7 +327,6 @@ int gemm_rows(asr_spec* h, const void* W, const CUtensorMap* mW, int M, int K, c
   epi.N = N;
   epi.status = h->status;
   if (mode == EPI_QKV) epi.b_max = h->Bmax;
-  if (mode != EPI_ARGMAX && !epi.trace) epi.trace = trace_slot(h);
   const int cls = mode == EPI_QKV     ? ASR_PROF_QKV
                   : mode == EPI_RESID ? ASR_PROF_RESID
                   : mode == EPI_Q     ? ASR_PROF_QUERY
@@ -323,22 +347,11 @@ int gemm_rows(asr_spec* h, const void* W, const CUtensorMap* mW, int M, int K, c
     launch_gemm_f32(g, mode, epi, h->st);
     return 0;
   }
-  WideGemm w{};
-  if (h->use_wide && wide_pick(M, N, K, mode, h->n_sms, &w.bn, &w.split)) {
-    const CUtensorMap* mb = bmap(h, x_id, X, h->R_pad, K, w.bn);
-    const CUtensorMap* mx = mode == EPI_RESID ? xmap(h, epi.x, w.bn) : mW;
-    if (!mb || !mx) return fail(h, ASR_E_CUDA, "tensor map encode failed");
-    w.mapA = *mW;
-    w.mapB = *mb;
-    w.mapX = *mx;
-    w.M = M;
-    w.N = N;
-    w.K = K;
-    w.pdl = h->use_pdl;
-    w.stages = h->wide_stages;
+  int bn, split;
+  if (h->use_wide && wide_pick(M, N, K, mode, h->n_sms, &bn, &split)) {
     Tl t(h, ASR_TL_GEMM + mode + (epi.ln_part ? ASR_TL_LN_FUSED : 0));
     epi.tl = h->tl_cur;
-    launch_gemm_wide(w, mode, epi, h->status, h->st);
+    if (int rc = wide_rows(h, mW, M, K, X, x_id, N, mode, epi)) return rc;
     if (epi.xg) {   // every tile wrote the statistics of its 128-feature slice
       h->ln_c = 128;
       h->ln_S = M / 128;
@@ -380,6 +393,7 @@ int gemm_rows(asr_spec* h, const void* W, const CUtensorMap* mW, int M, int K, c
   g.pdl = h->use_pdl;
   g.ws = h->ws;
   g.tickets = h->tickets;
+  if (mode != EPI_ARGMAX && mode != EPI_F32) epi.trace = trace_slot(h);
   Tl t(h, ASR_TL_GEMM + mode + (epi.ln_part ? ASR_TL_LN_FUSED : 0));
   epi.tl = h->tl_cur;
   launch_gemm_tc(g, mode, epi, h->status, h->st);
@@ -441,12 +455,8 @@ int attn_splits_for(asr_spec* h, int utts, int t_alloc, bool self_attn) {
   return S;
 }
 
-void attention(asr_spec* h, AttnArgs& a, bool self_attn, int layer) {
-  if (!h->bf16) {
-    a.pdl = h->use_pdl;
-    launch_attention_f32(a, h->st);
-    return;
-  }
+// The tensor-core attention of one layer (the caller records the timeline).
+void attention_launch(asr_spec* h, AttnArgs& a, bool self_attn, int layer) {
   a.segs = (a.rows_max + 31) / 32;
   a.splits = attn_splits_for(h, h->B * a.segs, a.t_alloc, self_attn);
   if (self_attn) {
@@ -463,10 +473,19 @@ void attention(asr_spec* h, AttnArgs& a, bool self_attn, int layer) {
   }
   a.tickets = h->attn_tickets;
   a.pdl = h->use_pdl;
-  Tl t(h, self_attn ? ASR_TL_ATTN_SELF : ASR_TL_ATTN_CROSS);
   a.tl = h->tl_cur;
   launch_attention_tc(a, h->status, h->st);
   a.tl = nullptr;
+}
+
+void attention(asr_spec* h, AttnArgs& a, bool self_attn, int layer) {
+  if (!h->bf16) {
+    a.pdl = h->use_pdl;
+    launch_attention_f32(a, h->st);
+    return;
+  }
+  Tl t(h, self_attn ? ASR_TL_ATTN_SELF : ASR_TL_ATTN_CROSS);
+  attention_launch(h, a, self_attn, layer);
 }
 
 // With a draft: the residual stream after a tapped layer into its column of
@@ -603,81 +622,108 @@ int run_layers(asr_spec* h, int N, bool prefill = false) {
 }
 
 // The decoder layers of a step with at most VF_ROWS rows (csrc/fewrow.cu):
-// six launches per layer.
-int run_layers_few(asr_spec* h) {
-  const int d = h->d, F = h->F, H = h->H, C = h->fr_C, N = h->B * (h->kmax + 1);
+// eight launches per layer.  The timeline and the class profile see the two
+// launches of QKV + self-attention, and of cross query + cross-attention, as
+// one stage each.
+int run_layers_few(asr_spec* h, int N) {
+  const int d = h->d, F = h->F, H = h->H;
+  const int rows_max = N / std::max(h->B, 1);
   const int nt_o = d / 8, nt_f = F / 8, KS = F / d;
   const int g_o = std::min(nt_o, h->fr_sms), g_f = std::min(nt_f, h->fr_sms), g_d = h->fr_gd;
   const size_t self_layer = (size_t)h->Bmax * H * h->maxpos * 64;
   {
     Prof p(h, ASR_PROF_OTHER, 1);
     Tl t(h, ASR_TL_EMBED);
-    launch_embed(h->w_tok, h->w_pos, h->bf16, h->plan, std::min(N, VF_ROWS), d, h->x, h->st, h->use_pdl, h->tl_cur,
-                 nullptr, nullptr, nullptr, h->V, h->maxpos, h->status);
+    launch_embed(h->w_tok, h->w_pos, h->bf16, h->plan, N, d, h->x, h->st, h->use_pdl, h->tl_cur,
+                 static_cast<__nv_bfloat16*>(h->xn), h->lw[0].ln1g, h->ln_part, h->V, h->maxpos, h->status);
   }
-  auto bf = [](void* p) { return static_cast<const __nv_bfloat16*>(p); };
-  // the packed weights of the layers' six launches in launch order, for the
-  // L2 prefetch of a later launch's weights
+  // The weights of the launch fr_prefetch ahead, for its L2 prefetch (six: the
+  // large MLP matrices ride on QKV and self-attention; 1272 us per round of
+  // the full large decoder against 1305 without and 1277 to 1339 at 1 to 5, 7
+  // and 8); launch slots of a layer: QKV, self, out, query, cross, out, up, down.
   auto later = [&](int l, int slot, const void** pf, uint32_t* bytes) {
-    const int g = 6 * l + slot + h->fr_prefetch;
+    const int g = 8 * l + slot + h->fr_prefetch;
     *pf = nullptr;
     *bytes = 0;
-    if (h->fr_prefetch <= 0 || g >= 6 * h->L) return;
-    const LayerW& n = h->lw[g / 6];
+    if (h->fr_prefetch <= 0 || g >= 8 * h->L) return;
+    const LayerW& n = h->lw[g / 8];
     const uint32_t dd = (uint32_t)d * d * 2, fd = (uint32_t)F * d * 2;
-    const void* p[6] = {n.p_qkv, n.p_wo, n.p_wcq, n.p_wco, n.p_w1, n.p_w2};
-    const uint32_t b[6] = {3 * dd, dd, dd, dd, fd, fd};
-    *pf = p[g % 6];
-    *bytes = b[g % 6];
+    const void* p[8] = {n.wqkv, nullptr, n.p_wo, n.wcq, nullptr, n.p_wco, n.p_w1, n.p_w2};
+    const uint32_t b[8] = {3 * dd, 0, dd, dd, 0, dd, fd, fd};
+    *pf = p[g % 8];
+    *bytes = b[g % 8];
   };
+  Epi base{};
+  base.n_valid = h->plan.n_rows;
+  base.d = d;
+  base.row_b = h->plan.row_b;
+  base.row_pos = h->plan.row_pos;
+  base.kv_bf16 = 1;
+  base.act_bf16 = 1;
+  base.max_pos = h->maxpos;
+  base.n_heads = H;
+  base.ln_part = h->ln_part;   // one slice of d features from the embedding, then slices of 8 from the GEMVs
+  base.ln_S = 1;
+  base.ln_c = d;
+  base.ln_stride = h->R_pad;
+  AttnArgs a{};
+  a.status = h->status;
+  a.kv_bf16 = 1;
+  a.enc_len = h->enc_len;
+  a.kv_len = h->kv_len;
+  a.plan = h->plan;
+  a.B = h->B;
+  a.H = H;
+  a.d = d;
+  a.out = h->att;
+  a.out_bf16 = 1;
+  a.rows_max = rows_max;
+  FrGemv g{};
+  g.n_rows = h->plan.n_rows;
+  g.status = h->status;
+  g.x = h->x;
+  g.x_out = h->x;
   for (int l = 0; l < h->L; ++l) {
     LayerW& w = h->lw[l];
-    FrHead hd{};
-    hd.x = h->x;
-    hd.d = d;
-    hd.H = H;
-    hd.C = C;
-    hd.B = h->B;
-    hd.max_pos = h->maxpos;
-    hd.plan = h->plan;
-    hd.kv_len = h->kv_len;
-    hd.enc_len = h->enc_len;
-    hd.att = static_cast<__nv_bfloat16*>(h->att);
-    hd.status = h->status;
-    // LayerNorm 1 -> QKV -> self-attention
-    FrHead hs = hd;
-    hs.W = bf(w.p_qkv);
-    hs.bias = w.bqkv;
-    hs.ln_g = w.ln1g;
-    hs.ln_b = w.ln1b;
-    hs.tiles_max = (24 + C - 1) / C;
-    hs.mrg_slots = (h->maxpos + 127) / 128;
-    hs.ks = static_cast<__nv_bfloat16*>(h->kself) + l * self_layer;
-    hs.vs = static_cast<__nv_bfloat16*>(h->vself) + l * self_layer;
-    hs.row0 = (long long)l * h->Bmax * H * h->maxpos;
-    hs.t_alloc = h->maxpos;
-    later(l, 0, &hs.pf, &hs.pf_bytes);
+    // QKV (LayerNorm 1 folded) and self-attention
     {
       Prof p(h, ASR_PROF_QKV_SELF, 1);
       Tl t(h, ASR_TL_QKV_SELF);
-      hs.tl = h->tl_cur;
-      hs.trace = trace_slot(h);
-      CK(launch_fr_self(&h->m_kself[0], &h->m_vself[0], hs, h->st, h->use_pdl));
+      Epi e = base;
+      e.bias = w.bqkv;
+      e.out_f32 = h->q;
+      e.kcache = static_cast<__nv_bfloat16*>(h->kself) + l * self_layer;
+      e.vcache = static_cast<__nv_bfloat16*>(h->vself) + l * self_layer;
+      e.ln_c1 = w.c1_qkv;
+      e.ln_c2 = w.c2_qkv;
+      later(l, 0, &e.pf, &e.pf_bytes);
+      e.tl = h->tl_cur;
+      if (int rc = wide_rows(h, &w.m_wqkv, 3 * d, d, h->xn, BUF_XN, N, EPI_QKV, e)) return rc;
+      count_launch(h);
+      a.q = h->q;
+      a.causal = 1;
+      a.t_alloc = h->maxpos;
+      a.ml_out = nullptr;
+      a.tree = h->cur_tree;
+      later(l, 1, &a.pf, &a.pf_bytes);
+      attention_launch(h, a, true, l);
+      a.tree = false;
     }
-    FrGemv g{};
-    g.n_rows = h->plan.n_rows;
-    g.status = h->status;
-    g.x = h->x;
-    g.x_out = h->x;
     // self-attention output projection + residual
     FrGemv go = g;
-    go.W = bf(w.p_wo);
+    go.W = static_cast<const __nv_bfloat16*>(w.p_wo);
     go.bias = w.bo;
     go.N = d;
     go.K = d;
     go.tiles_max = (nt_o + g_o - 1) / g_o;
     go.a = static_cast<const __nv_bfloat16*>(h->att);
-    later(l, 1, &go.pf, &go.pf_bytes);
+    go.xg = static_cast<__nv_bfloat16*>(h->xn);
+    go.xg_gain = w.ln2g;
+    go.st_part = h->ln_part;
+    go.st_stride = h->R_pad;
+    base.ln_S = nt_o;
+    base.ln_c = 8;
+    later(l, 2, &go.pf, &go.pf_bytes);
     {
       Prof p(h, ASR_PROF_RESID, 1);
       Tl t(h, ASR_TL_GEMM + EPI_RESID);
@@ -685,32 +731,32 @@ int run_layers_few(asr_spec* h) {
       go.trace = trace_slot(h);
       CK(launch_fr_gemv(go, FR_RESID, 1, g_o, d, h->st, h->use_pdl));
     }
-    // LayerNorm 2 -> cross query -> cross-attention
-    FrHead hc = hd;
-    hc.W = bf(w.p_wcq);
-    hc.bias = w.bcq;
-    hc.ln_g = w.ln2g;
-    hc.ln_b = w.ln2b;
-    hc.tiles_max = (8 + C - 1) / C;
-    hc.mrg_slots = C;
-    hc.row0 = (long long)l * 2 * h->Bmax * H * h->Tmax;
-    hc.vofs = (long long)h->Bmax * H * h->Tmax;
-    hc.t_alloc = h->Tmax;
-    hc.q_anchor = l == h->anchor ? h->q_anchor : nullptr;
-    hc.ml = l == h->anchor ? h->ml : nullptr;
-    later(l, 2, &hc.pf, &hc.pf_bytes);
+    // cross query (LayerNorm 2 folded) and cross-attention
     {
       Prof p(h, ASR_PROF_QUERY_CROSS, 1);
       Tl t(h, ASR_TL_QUERY_CROSS);
-      hc.tl = h->tl_cur;
-      hc.trace = trace_slot(h);
-      CK(launch_fr_cross(&h->m_xkv[0], hc, h->st, h->use_pdl));
+      Epi e = base;
+      e.bias = w.bcq;
+      e.out_f32 = l == h->anchor ? h->q_anchor : h->q;
+      e.ln_c1 = w.c1_cq;
+      e.ln_c2 = w.c2_cq;
+      later(l, 3, &e.pf, &e.pf_bytes);
+      e.tl = h->tl_cur;
+      if (int rc = wide_rows(h, &w.m_wcq, d, d, h->xn, BUF_XN, N, EPI_Q, e)) return rc;
+      count_launch(h);
+      a.q = e.out_f32;
+      a.causal = 0;
+      a.t_alloc = h->Tmax;
+      a.ml_out = l == h->anchor ? h->ml : nullptr;
+      later(l, 4, &a.pf, &a.pf_bytes);
+      attention_launch(h, a, false, l);
     }
     // cross-attention output projection + residual
     FrGemv gc = go;
-    gc.W = bf(w.p_wco);
+    gc.W = static_cast<const __nv_bfloat16*>(w.p_wco);
     gc.bias = w.bco;
-    later(l, 3, &gc.pf, &gc.pf_bytes);
+    gc.xg = nullptr;
+    later(l, 5, &gc.pf, &gc.pf_bytes);
     {
       Prof p(h, ASR_PROF_RESID, 1);
       Tl t(h, ASR_TL_GEMM + EPI_RESID);
@@ -720,7 +766,7 @@ int run_layers_few(asr_spec* h) {
     }
     // LayerNorm 3 -> MLP up + GELU
     FrGemv gu = g;
-    gu.W = bf(w.p_w1);
+    gu.W = static_cast<const __nv_bfloat16*>(w.p_w1);
     gu.bias = w.b1;
     gu.N = F;
     gu.K = d;
@@ -728,7 +774,7 @@ int run_layers_few(asr_spec* h) {
     gu.ln_g = w.ln3g;
     gu.ln_b = w.ln3b;
     gu.h_out = static_cast<__nv_bfloat16*>(h->hbuf);
-    later(l, 4, &gu.pf, &gu.pf_bytes);
+    later(l, 6, &gu.pf, &gu.pf_bytes);
     {
       Prof p(h, ASR_PROF_UP, 1);
       Tl t(h, ASR_TL_GEMM + EPI_GELU);
@@ -738,13 +784,19 @@ int run_layers_few(asr_spec* h) {
     }
     // MLP down + residual (K split over a cluster of F / d CTAs)
     FrGemv gd = g;
-    gd.W = bf(w.p_w2);
+    gd.W = static_cast<const __nv_bfloat16*>(w.p_w2);
     gd.bias = w.b2;
     gd.N = d;
     gd.K = F;
     gd.tiles_max = (nt_o + g_d - 1) / g_d;
     gd.a = static_cast<const __nv_bfloat16*>(h->hbuf);
-    later(l, 5, &gd.pf, &gd.pf_bytes);
+    if (l + 1 < h->L) {
+      gd.xg = static_cast<__nv_bfloat16*>(h->xn);
+      gd.xg_gain = h->lw[l + 1].ln1g;
+      gd.st_part = h->ln_part;
+      gd.st_stride = h->R_pad;
+    }
+    later(l, 7, &gd.pf, &gd.pf_bytes);
     {
       Prof p(h, ASR_PROF_RESID, 1);
       Tl t(h, ASR_TL_GEMM + EPI_RESID);
@@ -752,7 +804,7 @@ int run_layers_few(asr_spec* h) {
       gd.trace = trace_slot(h);
       CK(launch_fr_gemv(gd, FR_RESID, KS, g_d, d, h->st, h->use_pdl));
     }
-    if (int rc = tap_copy(h, l, VF_ROWS)) return rc;
+    if (int rc = tap_copy(h, l, N)) return rc;
   }
   return 0;
 }
@@ -861,6 +913,9 @@ int draft_block(asr_spec* h, const RowPlan& plan, int rows, bool lm) {
   return 0;
 }
 
+// Steps of at most VF_ROWS rows take the few-row layers.
+bool few_rows(const asr_spec* h, int N) { return h->fr_sms > 0 && h->use_fewrow && h->ln_fold && h->use_wide && N <= VF_ROWS; }
+
 bool dims_ok(const asr_model_dims& m) {
   return m.n_layers >= 1 && m.d_model >= 64 && m.d_model % 64 == 0 && m.d_model <= 2048 &&
          m.n_heads * 64 == m.d_model && m.d_ffn >= 64 && m.d_ffn % 64 == 0 && m.vocab >= 2 && m.max_pos >= 2 &&
@@ -891,9 +946,9 @@ int enqueue_verify(asr_spec* h, int k) {
                        h->row_key, h->status, tr, h->st, h->tl_cur, h->cur_tree ? h->parent_buf : nullptr);
   }
   const int N = B * (k + 1);
-  h->last_fused = h->fr_C > 0 && h->use_fewrow && N <= VF_ROWS && B <= VF_ROWS && !h->cur_tree;
-  if (h->last_fused) {   // few rows: six launches per layer, then LayerNorm + LM head
-    if (int rc = run_layers_few(h)) return rc;
+  h->last_fused = few_rows(h, N);
+  if (h->last_fused) {   // few rows: GEMVs, then LayerNorm + LM head
+    if (int rc = run_layers_few(h, N)) return rc;
     {
       Prof p(h, ASR_PROF_LAYERNORM, 1);
       Tl t(h, ASR_TL_LAYERNORM);
@@ -1229,10 +1284,8 @@ int asr_spec_create(const asr_model_dims* dims, const asr_weights* weights, void
   CK(cudaMemset(h->counters, 0, 8 * sizeof(unsigned long long)));
   if (const char* e = std::getenv("ASRSPEC_FEWROW")) h->use_fewrow = std::atoi(e) != 0;
   if (h->bf16) {
-    int C = 0;
     int n_sm = 0, gd = 0;
-    if (fr_configure(d, F, h->H, h->maxpos, &C, &n_sm, &gd)) {
-      h->fr_C = C;
+    if (fr_configure(d, F, &n_sm, &gd)) {
       h->fr_sms = n_sm;
       h->fr_gd = gd;
       for (int l = 0; l < L; ++l) {   // packed copies of the layer weights
@@ -1241,8 +1294,7 @@ int asr_spec_create(const asr_model_dims* dims, const asr_weights* weights, void
           void* src;
           void** dst;
           int N, K;
-        } mats[6] = {{w.wqkv, &w.p_qkv, 3 * d, d}, {w.wo, &w.p_wo, d, d},  {w.wcq, &w.p_wcq, d, d},
-                     {w.wco, &w.p_wco, d, d},     {w.w1, &w.p_w1, F, d},   {w.w2, &w.p_w2, d, F}};
+        } mats[4] = {{w.wo, &w.p_wo, d, d}, {w.wco, &w.p_wco, d, d}, {w.w1, &w.p_w1, F, d}, {w.w2, &w.p_w2, d, F}};
         for (auto& m : mats) {
           if ((rc = dalloc(h, m.dst, (size_t)m.N * m.K * 2))) return finish(rc);
           CK(launch_fr_pack(m.src, *m.dst, m.N, m.K, h->st));

@@ -240,6 +240,7 @@ gemm_wide_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant
         }
         if (MODE == EPI_RESID && epi.xg != nullptr) s_op[3][f] = __ldg(epi.xg_gain + m0 + f);
       }
+      if (t == 0) prefetch_share(epi.pf, epi.pf_bytes, cta_id, gridDim.x * gridDim.y);
     }
     pdl_wait();
     pdl_launch();
@@ -247,32 +248,39 @@ gemm_wide_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant
       // Folded LayerNorm: row statistics combined from the producer's equal
       // slices, one pass shifted by the first slice's mean:
       // mean = shift + E / S, M2 = sum M2_s + c (sum e_s^2 - E^2 / S)
+      // (up to 32 rows: 2, 4 or 8 threads per row, 40 slices each in flight)
       if (epi.ln_part != nullptr) {
-        const int S = epi.ln_S;
-        for (int rl = t; rl < BN; rl += NT) {
-          const int n = n0 + rl;
-          const bool ok = n < n_valid;
-          const float2* pr = epi.ln_part + (ok ? n : 0);
-          const float shift = ok ? pr[0].x : 0.f;
+        const int S = epi.ln_S, live = n_valid - n0 < BN ? n_valid - n0 : BN;
+        const int tpr = live <= NT / 8 ? 8 : live <= NT / 4 ? 4 : live <= NT / 2 ? 2 : 1;   // uniform over the CTA
+        const int sub = t % tpr;
+        for (int rl = t / tpr; rl < (live + NT / tpr - 1) / (NT / tpr) * (NT / tpr); rl += NT / tpr) {   // whole warps
+          const bool ok = rl < live;
+          const float2* pr = epi.ln_part + n0 + (ok ? rl : 0);
+          const float shift = pr[0].x;
           float e1 = 0.f, e2 = 0.f, m2 = 0.f;
-          if (ok)
-            for (int j0 = 0; j0 < S; j0 += 8) {   // eight slices' loads in flight
-              float2 p[8];
+          for (int j0 = sub; j0 < S; j0 += 40 * tpr) {
+            float2 p[40];
 #pragma unroll
-              for (int u = 0; u < 8; ++u)
-                p[u] = j0 + u < S ? pr[(size_t)(j0 + u) * epi.ln_stride] : make_float2(shift, 0.f);
+            for (int u = 0; u < 40; ++u)
+              p[u] = j0 + u * tpr < S ? pr[(size_t)(j0 + u * tpr) * epi.ln_stride] : make_float2(shift, 0.f);
 #pragma unroll
-              for (int u = 0; u < 8; ++u) {
-                const float es = p[u].x - shift;
-                e1 += es;
-                e2 += es * es;
-                m2 += p[u].y;
-              }
+            for (int u = 0; u < 40; ++u) {
+              const float es = p[u].x - shift;
+              e1 += es;
+              e2 += es * es;
+              m2 += p[u].y;
             }
-          const float mean = shift + e1 / (float)S;
-          const float q = m2 + (float)epi.ln_c * fmaxf(e2 - e1 * e1 / (float)S, 0.f);
-          ln_mu[rl] = ok ? mean : 0.f;
-          ln_rs[rl] = ok ? rsqrtf(q / (float)(S * epi.ln_c) + 1e-5f) : 0.f;
+          }
+          for (int o = tpr >> 1; o > 0; o >>= 1) {
+            e1 += __shfl_xor_sync(0xffffffffu, e1, o);
+            e2 += __shfl_xor_sync(0xffffffffu, e2, o);
+            m2 += __shfl_xor_sync(0xffffffffu, m2, o);
+          }
+          if (ok && sub == 0) {
+            const float q = m2 + (float)epi.ln_c * fmaxf(e2 - e1 * e1 / (float)S, 0.f);
+            ln_mu[rl] = shift + e1 / (float)S;
+            ln_rs[rl] = rsqrtf(q / (float)(S * epi.ln_c) + 1e-5f);
+          }
         }
       }
       if constexpr (MODE == EPI_QKV)

@@ -156,6 +156,8 @@ struct AttnArgs {
   bool tree = false;       // self-attention of a tree verify: slots past kv_len visible by plan.row_mask
   unsigned long long* tl = nullptr;   // launch timeline slot (tl_mark), or null
   int* status = nullptr;   // device status word (bounds-check mode)
+  const void* pf = nullptr;           // tensor-core path: a later launch's weights, prefetched into L2 (or null)
+  uint32_t pf_bytes = 0;
 };
 void launch_attention_f32(const AttnArgs& a, cudaStream_t st);   // fp32 caches
 void launch_attention_tc(const AttnArgs& a, int* status, cudaStream_t st);
@@ -193,11 +195,10 @@ void launch_tree_commit(const int* path, int k, const int* accepted, const int* 
                         int max_pos, int b_max, void* kself, void* vself, int es, int* status, cudaStream_t st);
 
 // ---- Few-row verify layers (csrc/fewrow.cu) ------------------------------------
-// A step of at most VF_ROWS rows runs each decoder layer as six launches:
-// LayerNorm + QKV + self-attention (one cluster per head), output projection,
-// LayerNorm + cross query + cross-attention (one cluster per head), output
-// projection, LayerNorm + MLP up, MLP down; the projections as GEMVs over
-// 8-feature tiles (no split-K exchange).
+// A step of at most VF_ROWS rows runs each decoder layer as eight launches:
+// QKV on the many-row GEMM, self-attention, output projection; cross query on
+// the GEMM, cross-attention, output projection; LayerNorm + MLP up, MLP down;
+// the output and MLP projections as GEMVs over 8-feature tiles.
 constexpr int VF_ROWS = 9;
 enum FrMode : int { FR_RESID = 0, FR_GELU = 1 };
 struct FrGemv {
@@ -209,6 +210,10 @@ struct FrGemv {
   const float *ln_g, *ln_b;
   const __nv_bfloat16* a;   // FR_RESID: bf16 input rows [R][K]
   float* x_out;             // FR_RESID: x[r][m] += y + bias  ([R][N])
+  __nv_bfloat16* xg;        // FR_RESID, or null: bf16(gain * x), the operand of the next folded LayerNorm ([R][N])
+  const float* xg_gain;
+  float2* st_part;          // with xg: (mean, sum of squared deviations) of each 8-feature slice [N / 8][st_stride]
+  int st_stride;
   __nv_bfloat16* h_out;     // FR_GELU: bf16(gelu(y + bias))  ([R][N])
   const int* n_rows;
   int* status;
@@ -217,52 +222,22 @@ struct FrGemv {
   const void* pf;              // a later launch's weights, prefetched into L2 (or null)
   uint32_t pf_bytes;
 };
-struct FrHead {
-  const __nv_bfloat16* W;   // self: fused QKV weights [3d][d]; cross: query weights [d][d]
-  const float* bias;
-  const float *x, *ln_g, *ln_b;   // the residual stream and the LayerNorm in front of W
-  int d, H, C, B, max_pos;
-  int tiles_max;            // weight tiles per CTA, at most
-  int mrg_slots;            // partials a merging CTA can hold per row
-  RowPlan plan;
-  const int* kv_len;
-  const int* enc_len;
-  __nv_bfloat16 *ks, *vs;   // self: this layer's caches [B_max][H][max_pos][64] (new rows appended)
-  long long row0;           // tensor-map row of this layer's (utterance 0, head 0, key 0)
-  long long vofs;           // cross: rows from the K half to the V half of the encoder cache
-  int t_alloc;              // tensor-map rows per (utterance, head)
-  __nv_bfloat16* att;       // [R][d] attention output
-  float* q_anchor;          // cross at the anchor layer: fp32 queries [R][d], else null
-  float* ml;                // cross at the anchor layer: softmax (max, sum) [R][H][2], else null
-  int* status;
-  unsigned long long* tl;
-  unsigned long long* trace;   // per-CTA phase stamps [CTA][FR_TRACE_PHASES] (diagnostics), or null
-  const void* pf;              // a later launch's weights, prefetched into L2 (or null)
-  uint32_t pf_bytes;
-};
-// Phase stamps of a traced few-row launch, GPU global timer (ns), thread 0 of
+// Phase stamps of a traced GEMV launch, GPU global timer (ns), thread 0 of
 // each CTA: 0 entry, 1 past the wait on the previous launch, 2 input rows
-// ready, 3 weights landed, 4 projection reduced, 5 exchange landed (head:
-// gathered q/k/v; K-split group: the other ranks' partials), 6 attention
-// done (head), 7 exit; head kernels also 8 first K/V chunk landed, 9 first
-// chunk's attention combined, 10 merge inputs landed, 11 (GEMVs without a
-// LayerNorm) bf16 input rows landed.  Up to FR_TRACE_CTAS
-// CTAs per launch.
+// ready, 3 weights landed, 4 projection reduced, 5 exchange landed (K-split
+// group: the other ranks' partials), 7 exit, 11 (without a LayerNorm) bf16
+// input rows landed.  Up to FR_TRACE_CTAS CTAs per launch.
 constexpr int FR_TRACE_PHASES = 12;
 constexpr int FR_TRACE_CTAS = 320;
-// 1 and the cluster size per head when the kernels run for these dimensions on this device
-// (gd_out: the MLP down-projection's groups of F / d CTAs)
-int fr_configure(int d, int F, int H, int max_pos, int* C_out, int* sms_out, int* gd_out);
+// 1 when the kernels run for these dimensions on this device (gd_out: the MLP
+// down-projection's groups of F / d CTAs)
+int fr_configure(int d, int F, int* sms_out, int* gd_out);
 size_t fr_gemv_smem(int d, int K, int tiles_max, int ks);
-size_t fr_head_smem(int d, int tiles_max, bool self_attn, int mrg_slots);
 // groups: CTA groups of ks (one cluster each); a.tiles_max = ceil(N / 8 / groups)
 // Pack a bf16 [N][K] weight matrix (N, K multiples of 8) into the few-row
 // kernels' tile layout: 8-row tiles, contiguous, 16-byte pieces piece-major.
 cudaError_t launch_fr_pack(const void* src, void* dst, int N, int K, cudaStream_t st);
 cudaError_t launch_fr_gemv(const FrGemv& a, int mode, int ks, int groups, int d, cudaStream_t st, bool pdl);
-cudaError_t launch_fr_self(const CUtensorMap* kmap, const CUtensorMap* vmap, const FrHead& a, cudaStream_t st,
-                           bool pdl);
-cudaError_t launch_fr_cross(const CUtensorMap* xmap, const FrHead& a, cudaStream_t st, bool pdl);
 
 // ---- Draft side (csrc/draft.cu) ---------------------------------------------------
 // Window centre of the draft's audio cross-attention for proposals

@@ -15,7 +15,7 @@ anchor-readout share against batch size), --gemm IMPL,M,N,K (one GEMM shape
 through the kernel test entry, for captures of a single kernel).
 
 Kernel launches per round (bf16 decoders): at most 9 rows (e.g. batch 1):
-2 + 6 per layer + 3 (few-row layers, final LayerNorm, LM head, accept);
+2 + 8 per layer + 3 (few-row layers, final LayerNorm, LM head, accept);
 more rows: 2 + 8 per layer + 2 (tensor-core chain, LayerNorm folded).
 """
 from __future__ import annotations
@@ -65,23 +65,25 @@ def timeline_summary(ns, kinds, rounds):
     return "\n".join(lines)
 
 
-FEWROW_KINDS = ["qkv_self", "self_out", "query_cross", "cross_out", "mlp_up", "mlp_down"]
+FEWROW_KINDS = ["qkv", "self_out", "cross_query", "cross_out", "mlp_up", "mlp_down"]
 FEWROW_PHASES = ["entry", "past_wait", "rows", "weights", "reduced", "exchange", "attention", "exit", "kv_in",
                  "combined", "merge_in", "inputs_in"]
 
 
 def fewrow_trace_summary(tr):
-    """Per few-row launch kind (averaged over layers): each phase's median and
-    maximum over CTAs, in us after the previous launch's last exit (negative:
-    the CTA was resident before it), and the launch's span from that exit to
-    its own last exit."""
+    """Per projection of the few-row layers (averaged over layers): each phase's
+    median and maximum over CTAs, in us after the previous projection's last
+    exit (negative: the CTA was resident before it; attention, between QKV and
+    its output projection, is not traced), and the span from that exit to its
+    own last exit.  qkv and cross_query are tensor-core launches: their phases
+    have the GEMM trace's meaning under the same numbers."""
     tr = tr.astype(np.int64)
     n = tr.shape[0]
     lines = [f"  few-row trace: {n} launches; us after the previous launch's last CTA exit, median / max over CTAs"]
     lines.append("  " + f"{'kind':<12}" + "".join(f"{p:>16}" for p in FEWROW_PHASES) + f"{'span':>9}")
     acc = {k: [] for k in FEWROW_KINDS}
     for i in range(1, n):
-        prev_exit = tr[i - 1][:, 7].max()
+        prev_exit = tr[i - 1][:, [4, 7]].max()   # GEMVs exit at 7, tensor-core launches at 4
         cta = tr[i][:, 0] > 0
         with np.errstate(all="ignore"):
             rel = np.where(tr[i][cta] > 0, (tr[i][cta] - prev_exit) / 1e3, np.nan)
@@ -95,7 +97,7 @@ def fewrow_trace_summary(tr):
         mx = np.nanmean([np.nanmax(r, axis=0) for r in acc[k]], axis=0)
         cells = "".join(f"{a:>8.2f}/{b:<7.2f}" if np.isfinite(a) else f"{'-':>16}"
                         for a, b in zip(med[:12], mx[:12]))
-        lines.append(f"  {k:<12}{cells}{mx[7]:>9.2f}")
+        lines.append(f"  {k:<12}{cells}{max(mx[4], mx[7]):>9.2f}")
     return "\n".join(lines)
 
 
