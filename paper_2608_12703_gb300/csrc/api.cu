@@ -44,6 +44,9 @@ struct DraftW {
         *b_cross = nullptr;
   float *ln1g = nullptr, *ln1b = nullptr, *ln2g = nullptr, *ln2b = nullptr, *ln3g = nullptr, *ln3b = nullptr,
         *lnfg = nullptr, *lnfb = nullptr;
+  // folded LayerNorms, as the target's
+  float *c1_qkv = nullptr, *c2_qkv = nullptr, *c1_cq = nullptr, *c2_cq = nullptr, *c1_fc1 = nullptr, *c2_fc1 = nullptr,
+        *c1_lm = nullptr, *c2_lm = nullptr;
   CUtensorMap m_in, m_qkv, m_wo, m_wcq, m_wco, m_w1, m_w2;
 };
 
@@ -159,9 +162,10 @@ struct asr_spec {
   void *d_xin = nullptr, *d_xn = nullptr, *d_att = nullptr, *d_h = nullptr, *d_xf = nullptr;
   RowPlan d_plan{};
   int *d_row_src = nullptr, *d_row_lo = nullptr, *d_row_hi = nullptr, *d_win_lo = nullptr, *d_win_hi = nullptr;
-  int *d_lens = nullptr, *d_nprop = nullptr, *d_last_row = nullptr, *d_prev_pos = nullptr, *d_out = nullptr;
+  DraftState d_state[2] = {};
+  int* d_out = nullptr;
   int *d_total = nullptr, *d_centers = nullptr, *d_lens_out = nullptr;
-  unsigned long long* d_row_key = nullptr;
+  float2* d_ln_part = nullptr;   // the draft's folded-LayerNorm statistics, slices of at least 8 features
   bool d_after_verify = false;
   float d_threshold = 0.f;            // confidence threshold of the proposals (0 = off)
   float* d_logits = nullptr;          // threshold on: the pass's logits [R_max][V]
@@ -814,11 +818,20 @@ int run_layers_few(asr_spec* h, int N) {
 // self-attention over the draft's cache (K/V of the rows appended) -> out
 // projection; LayerNorm -> cross-attention over the draft's encoder K/V
 // (window per row) -> out projection; LayerNorm -> MLP (2 d, GELU); final
-// LayerNorm -> the target's tied LM head with argmax (when `lm`).
-int draft_block(asr_spec* h, const RowPlan& plan, int rows, bool lm) {
+// LayerNorm -> the target's tied LM head with argmax into row_key (unless null).
+int draft_block(asr_spec* h, const RowPlan& plan, int rows, unsigned long long* row_key) {
   const int d = h->d, F2 = 2 * h->d;
   const int rows_per_utt = (rows + h->B - 1) / h->B;
+  const bool fold = h->ln_fold, pdl = h->use_pdl;
   DraftW& w = h->dw;
+  struct LnScope {   // the target's slice layout is the last verification's
+    asr_spec* h;
+    int S, c;
+    ~LnScope() {
+      h->ln_S = S;
+      h->ln_c = c;
+    }
+  } scope{h, h->ln_S, h->ln_c};
   Epi base{};
   base.n_valid = plan.n_rows;
   base.d = d;
@@ -837,12 +850,34 @@ int draft_block(asr_spec* h, const RowPlan& plan, int rows, bool lm) {
   A.status = h->status;
   A.plan = plan;
   Epi e = base;
+  e.n_valid = nullptr;   // the row count comes from the launch just before this one, too late for a GEMM's set-up
   e.bias = w.b_in;
   e.out_f32 = h->d_x;
   if (int rc = gemm_rows(h, w.w_in, &w.m_in, d, 4 * d, h->d_xin, BUF_DIN, rows, EPI_Q, e)) return rc;
-  launch_draft_embed(A, rows, h->w_tok, h->w_pos, h->d_x, h->st);
-  auto ln = [&](const float* g, const float* b, void* y) {
-    launch_layernorm(h->d_x, g, b, y, 1, plan.n_rows, rows, d, h->st, false, nullptr);
+  __nv_bfloat16* xn = static_cast<__nv_bfloat16*>(h->d_xn);
+  launch_draft_embed(A, rows, h->w_tok, h->w_pos, h->d_x, fold ? xn : nullptr, w.ln1g, h->d_ln_part, h->st, pdl);
+  h->ln_S = 1;
+  h->ln_c = d;
+  // the LayerNorm in front of a projection: folded (xn holds bf16(g x), its
+  // producer's slices the statistics), or a launch
+  auto ln = [&](Epi& c, const float* g, const float* b, const float* c1, const float* c2, void* y) {
+    if (fold) {
+      c.ln_part = h->d_ln_part;
+      c.ln_S = h->ln_S;
+      c.ln_c = h->ln_c;
+      c.ln_stride = h->R_pad;
+      c.ln_c1 = c1;
+      c.ln_c2 = c2;
+    } else {
+      launch_layernorm(h->d_x, g, b, y, 1, plan.n_rows, rows, d, h->st, false, nullptr);
+    }
+  };
+  auto producer = [&](Epi& c, const float* next_gain) {
+    if (!fold) return;
+    c.xg = xn;
+    c.xg_gain = next_gain;
+    c.st_part = h->d_ln_part;
+    c.st_stride = h->R_pad;
   };
   DraftAttn at{};
   at.q = h->d_q;
@@ -855,8 +890,8 @@ int draft_block(asr_spec* h, const RowPlan& plan, int rows, bool lm) {
   at.out = static_cast<__nv_bfloat16*>(h->d_att);
   at.status = h->status;
   // self-attention block
-  ln(w.ln1g, w.ln1b, h->d_xn);
   e = base;
+  ln(e, w.ln1g, w.ln1b, w.c1_qkv, w.c2_qkv, h->d_xn);
   e.bias = w.bqkv;
   e.out_f32 = h->d_q;
   e.kcache = h->d_ks;
@@ -866,14 +901,15 @@ int draft_block(asr_spec* h, const RowPlan& plan, int rows, bool lm) {
   at.vc = static_cast<const __nv_bfloat16*>(h->d_vs);
   at.t_alloc = h->maxpos;
   at.causal = 1;
-  launch_draft_attn(at, rows_per_utt, h->st);
+  launch_draft_attn(at, rows_per_utt, h->st, pdl);
   e = base;
   e.bias = w.bo;
   e.x = h->d_x;
+  producer(e, w.ln2g);
   if (int rc = gemm_rows(h, w.wo, &w.m_wo, d, d, h->d_att, BUF_DATT, rows, EPI_RESID, e)) return rc;
   // cross-attention block
-  ln(w.ln2g, w.ln2b, h->d_xn);
   e = base;
+  ln(e, w.ln2g, w.ln2b, w.c1_cq, w.c2_cq, h->d_xn);
   e.bias = w.bcq;
   e.out_f32 = h->d_q;
   if (int rc = gemm_rows(h, w.wcq, &w.m_wcq, d, d, h->d_xn, BUF_DXN, rows, EPI_Q, e)) return rc;
@@ -882,34 +918,37 @@ int draft_block(asr_spec* h, const RowPlan& plan, int rows, bool lm) {
   at.vc = static_cast<const __nv_bfloat16*>(h->d_xkv) + half;
   at.t_alloc = h->Tmax;
   at.causal = 0;
-  launch_draft_attn(at, rows_per_utt, h->st);
+  launch_draft_attn(at, rows_per_utt, h->st, pdl);
   e = base;
   e.bias = w.bco;
   e.x = h->d_x;
+  producer(e, w.ln3g);
   if (int rc = gemm_rows(h, w.wco, &w.m_wco, d, d, h->d_att, BUF_DATT, rows, EPI_RESID, e)) return rc;
   // MLP block
-  ln(w.ln3g, w.ln3b, h->d_xn);
   e = base;
+  ln(e, w.ln3g, w.ln3b, w.c1_fc1, w.c2_fc1, h->d_xn);
   e.bias = w.b1;
   e.act = h->d_h;
   if (int rc = gemm_rows(h, w.w1, &w.m_w1, F2, d, h->d_xn, BUF_DXN, rows, EPI_GELU, e)) return rc;
   e = base;
   e.bias = w.b2;
   e.x = h->d_x;
+  producer(e, w.lnfg);
   if (int rc = gemm_rows(h, w.w2, &w.m_w2, d, F2, h->d_h, BUF_DH, rows, EPI_RESID, e)) return rc;
-  if (!lm) return 0;
-  ln(w.lnfg, w.lnfb, h->d_xf);
+  if (!row_key) return 0;
   e = Epi{};
+  ln(e, w.lnfg, w.lnfb, w.c1_lm, w.c2_lm, h->d_xf);
   e.n_valid = plan.n_rows;
-  e.row_key = h->d_row_key;
+  e.row_key = row_key;
   e.d = d;
-  if (h->d_threshold <= 0.f)
-    return gemm_rows(h, h->w_tok, &h->m_tok, h->V, d, h->d_xf, BUF_DXF, rows, EPI_ARGMAX, e);
+  const void* xl = fold ? h->d_xn : h->d_xf;
+  const int xl_id = fold ? BUF_DXN : BUF_DXF;
+  if (h->d_threshold <= 0.f) return gemm_rows(h, h->w_tok, &h->m_tok, h->V, d, xl, xl_id, rows, EPI_ARGMAX, e);
   // confidence threshold: the logits, then per row the argmax and its probability
   e.out_f32 = h->d_logits;
   e.ld = h->V;
-  if (int rc = gemm_rows(h, h->w_tok, &h->m_tok, h->V, d, h->d_xf, BUF_DXF, rows, EPI_F32, e)) return rc;
-  launch_draft_softmax(h->d_logits, h->V, plan.n_rows, rows, h->d_row_key, h->d_row_p, h->st);
+  if (int rc = gemm_rows(h, h->w_tok, &h->m_tok, h->V, d, xl, xl_id, rows, EPI_F32, e)) return rc;
+  launch_draft_softmax(h->d_logits, h->V, plan.n_rows, rows, row_key, h->d_row_p, h->st, pdl);
   return 0;
 }
 
@@ -931,6 +970,9 @@ int copy_out(asr_spec* h, int32_t* dst, const int* src, size_t n) {
   CK(cudaMemcpyAsync(dst, src, n * 4, h->host_io ? cudaMemcpyDeviceToHost : cudaMemcpyDeviceToDevice, h->st));
   return 0;
 }
+
+// Aligned for int32 loads and stores by a kernel.
+bool words(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 3) == 0; }
 
 // The verify body on the handle's stream: rows, decoder layers, LM head with
 // fused argmax, acceptance and commit, anchor readout.  Reads the internal
@@ -1437,7 +1479,7 @@ int asr_spec_prefill(asr_spec_handle h, const int32_t* prompt, int32_t P0) {
       A.row_hi = h->d_row_hi;
       A.x_in = static_cast<__nv_bfloat16*>(h->d_xin);
       launch_draft_prefill_gather(A, h->B * c, h->st);
-      if (int rc = draft_block(h, h->plan, h->B * c, false)) return rc;
+      if (int rc = draft_block(h, h->plan, h->B * c, nullptr)) return rc;
     }
     Prof p(h, ASR_PROF_OTHER, 1);
     launch_prefill_advance(h->B, c, h->plan.n_utt_rows, h->kv_len, h->st);
@@ -1451,9 +1493,6 @@ int asr_spec_prefill(asr_spec_handle h, const int32_t* prompt, int32_t P0) {
 }
 
 namespace {
-
-// Aligned for int32 loads and stores by a kernel.
-bool words(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 3) == 0; }
 
 // The verify call: inputs into the internal buffers, the body (a CUDA graph per
 // (B, k, linear or tree), captured on first use), outputs out.
@@ -1645,11 +1684,27 @@ int asr_spec_draft_create(asr_spec_handle h, const asr_weights* dw) {
       (rc = dalloc(h, &h->d_x, R * d * 4)) || (rc = dalloc(h, &h->d_q, R * 3 * d * 4)) ||
       (rc = dalloc(h, &h->d_xin, R * 4 * d * 2)) || (rc = dalloc(h, &h->d_xn, R * d * 2)) ||
       (rc = dalloc(h, &h->d_att, R * d * 2)) || (rc = dalloc(h, &h->d_h, R * F2 * 2)) ||
-      (rc = dalloc(h, &h->d_xf, R * d * 2)) || (rc = dalloc(h, &h->d_row_key, R * 8)))
+      (rc = dalloc(h, &h->d_xf, R * d * 2)) || (rc = dalloc(h, &h->d_state[0].row_key, R * 8)) ||
+      (rc = dalloc(h, &h->d_state[1].row_key, R * 8)))
     return rc;
+  if (h->ln_fold) {
+    if ((rc = dalloc(h, &h->d_ln_part, (size_t)(d / 8) * R * sizeof(float2)))) return rc;
+    auto fold = [&](const void* W, const float* g, const float* b, int M, float** c1, float** c2) {
+      int r = dalloc(h, c1, (size_t)M * 4);
+      if (!r) r = dalloc(h, c2, (size_t)M * 4);
+      if (!r) launch_ln_fold(W, g, b, M, d, *c1, *c2, h->st);
+      return r;
+    };
+    if ((rc = fold(w.wqkv, w.ln1g, w.ln1b, 3 * d, &w.c1_qkv, &w.c2_qkv)) ||
+        (rc = fold(w.wcq, w.ln2g, w.ln2b, d, &w.c1_cq, &w.c2_cq)) ||
+        (rc = fold(w.w1, w.ln3g, w.ln3b, F2, &w.c1_fc1, &w.c2_fc1)) ||
+        (rc = fold(h->w_tok, w.lnfg, w.lnfb, h->V, &w.c1_lm, &w.c2_lm)))
+      return rc;
+    CK(cudaGetLastError());
+  }
   RowPlan& p = h->d_plan;
   int* ints = nullptr;
-  const size_t n_int = 7 * R + (Bm + 1) + 1 + Bm + 3 * R + 9 * Bm + Bm * std::max(h->kmax, 1);
+  const size_t n_int = 7 * R + (Bm + 1) + 1 + Bm + 3 * R + 13 * Bm + Bm * std::max(h->kmax, 1);
   if ((rc = dalloc(h, &ints, n_int * 4))) return rc;
   CK(cudaMemset(ints, 0, n_int * 4));
   int* q = ints;
@@ -1673,10 +1728,12 @@ int asr_spec_draft_create(asr_spec_handle h, const asr_weights* dw) {
   h->d_row_hi = cut(R);
   h->d_win_lo = cut(Bm);
   h->d_win_hi = cut(Bm);
-  h->d_lens = cut(Bm);
-  h->d_nprop = cut(Bm);
-  h->d_last_row = cut(Bm);
-  h->d_prev_pos = cut(Bm);
+  for (DraftState& st : h->d_state) {
+    st.lens = cut(Bm);
+    st.n_prop = cut(Bm);
+    st.last_row = cut(Bm);
+    st.pos = cut(Bm);
+  }
   h->d_total = cut(Bm);
   h->d_centers = cut(Bm);
   h->d_lens_out = cut(Bm);
@@ -1699,9 +1756,13 @@ int asr_spec_draft_propose(asr_spec_handle h, int32_t k, int32_t window, const i
   if (!total_len || !lens_out || (k > 0 && !draft_out) || (window == DRAFT_WIN_RANDOM && !centers))
     return fail(h, ASR_E_INVAL, "null pointer");
   const int B = h->B;
-  if (int rc = copy_in(h, h->d_total, total_len, B)) return rc;
-  if (window == DRAFT_WIN_RANDOM)
-    if (int rc = copy_in(h, h->d_centers, centers, B)) return rc;
+  // device arrays are read and written where they are, host ones copied
+  const bool by_kernel = !h->host_io && words(total_len) && words(centers) && words(draft_out) && words(lens_out);
+  if (!by_kernel) {
+    if (int rc = copy_in(h, h->d_total, total_len, B)) return rc;
+    if (window == DRAFT_WIN_RANDOM)
+      if (int rc = copy_in(h, h->d_centers, centers, B)) return rc;
+  }
   DraftArgs A{};
   A.B = B;
   A.d = h->d;
@@ -1716,13 +1777,13 @@ int asr_spec_draft_propose(asr_spec_handle h, int32_t k, int32_t window, const i
   A.kv_len = h->kv_len;
   A.pending = h->pending;
   A.enc_len = h->enc_len;
-  A.total_len = h->d_total;
+  A.total_len = by_kernel ? total_len : h->d_total;
   A.v_row_start = h->plan.row_start;
   A.v_n_utt_rows = h->plan.n_utt_rows;
   A.accepted = h->out4;
   A.anchor = h->out4 + 3 * h->Bmax;
   A.v_draft = h->draft_buf;
-  A.centers = h->d_centers;
+  A.centers = by_kernel ? centers : h->d_centers;
   A.taps = h->d_taps;
   A.last_tap = h->d_last_tap;
   A.x_prev = h->d_x;
@@ -1732,33 +1793,30 @@ int asr_spec_draft_propose(asr_spec_handle h, int32_t k, int32_t window, const i
   A.row_hi = h->d_row_hi;
   A.win_lo = h->d_win_lo;
   A.win_hi = h->d_win_hi;
-  A.lens = h->d_lens;
-  A.n_prop = h->d_nprop;
-  A.last_row = h->d_last_row;
-  A.prev_pos = h->d_prev_pos;
+  A.state[0] = h->d_state[0];
+  A.state[1] = h->d_state[1];
   A.draft_out = h->d_out;
-  A.row_key = h->d_row_key;
   A.x_in = static_cast<__nv_bfloat16*>(h->d_xin);
   A.threshold = h->d_threshold;
   A.row_p = h->d_row_p;
   // pass 0: catch-up of the last verification's accepted drafts + the restart
   const int rows0 = std::min(h->R_pad, B * (h->kmax + 1));
   launch_draft_round_plan(A, h->st);
-  launch_draft_gather(A, rows0, h->st);
-  if (int rc = draft_block(h, h->d_plan, rows0, true)) return rc;
-  launch_draft_take(A, h->st);
+  launch_draft_gather(A, rows0, h->st, h->use_pdl);
+  if (int rc = draft_block(h, h->d_plan, rows0, A.state[0].row_key)) return rc;
   for (int i = 1; i < k; ++i) {   // continuation proposals, one row per utterance still proposing
-    launch_draft_next_plan(A, i, h->st);
-    launch_draft_gather(A, B, h->st);
-    if (int rc = draft_block(h, h->d_plan, B, true)) return rc;
-    launch_draft_take(A, h->st);
+    launch_draft_step(A, i, h->st, h->use_pdl);
+    if (int rc = draft_block(h, h->d_plan, B, A.state[i & 1].row_key)) return rc;
   }
-  launch_draft_finish(A, h->d_lens_out, h->st);
+  launch_draft_finish(A, k > 0 ? (k - 1) & 1 : 0, by_kernel && k > 0 ? draft_out : h->d_out,
+                      by_kernel ? lens_out : h->d_lens_out, h->st, h->use_pdl);
   CK(cudaGetLastError());
   h->d_after_verify = false;
-  if (k > 0)
-    if (int rc = copy_out(h, draft_out, h->d_out, (size_t)B * k)) return rc;
-  if (int rc = copy_out(h, lens_out, h->d_lens_out, B)) return rc;
+  if (!by_kernel) {
+    if (k > 0)
+      if (int rc = copy_out(h, draft_out, h->d_out, (size_t)B * k)) return rc;
+    if (int rc = copy_out(h, lens_out, h->d_lens_out, B)) return rc;
+  }
   if (h->host_io) CK(cudaStreamSynchronize(h->st));
   return ASR_OK;
 }

@@ -13,7 +13,14 @@
 // the new committed length (the restart, whose argmax is proposal 1); passes
 // 1 .. k - 1 score one continuation row per utterance still proposing.  The
 // block itself runs on the library's GEMMs; these kernels only lay out rows
-// and move inputs.
+// and move inputs.  A pass is a chain of launches of a few microseconds each, so
+// what it costs is their number: between two passes one kernel takes the
+// proposals, lays out the next rows and gathers their inputs (every CTA works
+// out all utterances' rows, so nothing waits for a plan), the LayerNorms are
+// folded into the projections, and every kernel is a dependent launch.  Two
+// rounds of the cached loop at batch 1 (d = 1280, 4 target layers, k = 8):
+// 2318 us with 18 launches a pass, five of them one-CTA kernels without dependent
+// launch, 1680 with 12.
 #include <cmath>
 
 #include "kernels.h"
@@ -70,6 +77,7 @@ __device__ __forceinline__ void window_of(int kind, int anchor, int T, const int
 // row, -1 the saved tap of utterance b, -2 zeros.
 __global__ void __launch_bounds__(DP_T) draft_round_plan_kernel(DraftArgs A) {
   const int b = threadIdx.x;
+  const DraftState S = A.state[0];
   int n_rows = 0, n_acc = 0, lens = -1, r0v = 0;
   bool scored = false;
   if (b < A.B) {
@@ -97,11 +105,12 @@ __global__ void __launch_bounds__(DP_T) draft_round_plan_kernel(DraftArgs A) {
     window_of(A.win_kind, A.after_verify ? A.anchor[b] : 0, T, A.centers, b, lo, hi);
     A.plan.row_start[b] = start;
     A.plan.n_utt_rows[b] = n_rows;
-    A.lens[b] = lens;
-    A.n_prop[b] = 0;
+    S.lens[b] = lens;
+    S.n_prop[b] = 0;
+    S.pos[b] = P;
     A.win_lo[b] = lo;
     A.win_hi[b] = hi;
-    A.last_row[b] = lens >= 0 ? start + n_acc : -1;
+    S.last_row[b] = lens >= 0 ? start + n_acc : -1;
     const int P_old = P - 1 - n_acc;   // committed length before the verification (after_verify)
     for (int j = 1; j <= n_acc; ++j) {   // catch-up: unrestricted audio attention
       const int r = start + j - 1;
@@ -114,7 +123,7 @@ __global__ void __launch_bounds__(DP_T) draft_round_plan_kernel(DraftArgs A) {
       A.row_src[r] = r0v + j - 1;
       A.row_lo[r] = 0;
       A.row_hi[r] = T;
-      A.row_key[r] = 0ull;
+      S.row_key[r] = 0ull;
     }
     if (lens >= 0) {   // restart
       const int r = start + n_acc;
@@ -126,7 +135,7 @@ __global__ void __launch_bounds__(DP_T) draft_round_plan_kernel(DraftArgs A) {
       A.row_src[r] = scored ? r0v + n_acc : (A.after_verify ? -2 : -1);
       A.row_lo[r] = lo;
       A.row_hi[r] = hi;
-      A.row_key[r] = 0ull;
+      S.row_key[r] = 0ull;
     }
   }
   if (threadIdx.x == 0) {
@@ -135,58 +144,107 @@ __global__ void __launch_bounds__(DP_T) draft_round_plan_kernel(DraftArgs A) {
   }
 }
 
-// Pass i >= 1: one continuation row per utterance whose i proposals so far
-// leave it short of lens[b]: position one past its previous row, the
-// previous proposal as token, the previous row's block output (for all four
-// representations) as features, the round's window.
-__global__ void __launch_bounds__(DP_T) draft_next_plan_kernel(DraftArgs A, int i) {
-  const int b = threadIdx.x;
-  const bool on = b < A.B && A.lens[b] > i && A.n_prop[b] == i && A.last_row[b] >= 0;
+// After a pass's LM head: an utterance with a row in the pass takes its
+// argmax as the next proposal (until it holds lens of them, or, with the
+// confidence threshold on, until the argmax's probability falls below it: the
+// block then ends unproposed).
+struct Take {
+  int lens, n, tok;   // after the pass; tok: the proposal taken, or -1
+};
+__device__ __forceinline__ Take draft_take(const DraftArgs& A, const DraftState& S, int b) {
+  Take t{S.lens[b], S.n_prop[b], -1};
+  const int r = S.last_row[b];
+  if (r >= 0 && t.n < t.lens) {
+    if (A.threshold > 0.f && A.row_p[r] < A.threshold) {   // not confident: the block ends here
+      t.lens = t.n;
+    } else {
+      const uint32_t tok = argmax_index(S.row_key[r]);
+      t.tok = tok < (uint32_t)A.vocab ? (int)tok : 0;
+      ++t.n;
+    }
+  }
+  return t;
+}
+
+// Between pass i - 1 and pass i >= 1, one CTA per utterance: takes the
+// proposals of pass i - 1 and lays out one continuation row per utterance
+// whose i proposals leave it short of lens: position one past its previous
+// row, the proposal as token, the round's window, and as features the previous
+// row's block output four times (bf16).  Every CTA works out all utterances'
+// decisions and row numbers from the state that pass i - 1 left (state[(i - 1)
+// & 1]) and writes its own utterance's into the other copy.
+__global__ void __launch_bounds__(DP_T) draft_step_kernel(DraftArgs A, int i) {
+  __shared__ int s_take[3], s_on, s_row;
+  pdl_wait();
+  pdl_launch();
+  const DraftState S = A.state[(i - 1) & 1], N = A.state[i & 1];
+  const int u = threadIdx.x, b = blockIdx.x, d = A.d;
+  Take t{-1, 0, -1};
+  bool on = false;
+  if (u < A.B) {
+    t = draft_take(A, S, u);
+    on = t.lens > i && t.n == i && S.last_row[u] >= 0;
+  }
   int total;
-  const int r = excl_scan(on ? 1 : 0, &total);
-  if (b < A.B) {
+  const int r_u = excl_scan(on ? 1 : 0, &total);
+  if (u == b) {
+    s_take[0] = t.lens;
+    s_take[1] = t.n;
+    s_take[2] = t.tok;
+    s_on = on;
+    s_row = r_u;
+  }
+  __syncthreads();
+  const int r = s_row, old = S.last_row[b];
+  if (u == 0) {
+    const int tok = s_take[2], pos = S.pos[b] + 1;
+    if (tok >= 0) A.draft_out[(size_t)b * A.k + s_take[1] - 1] = tok;
+    N.lens[b] = s_take[0];
+    N.n_prop[b] = s_take[1];
+    N.last_row[b] = s_on ? r : -1;
+    N.pos[b] = pos;
     A.plan.row_start[b] = r;
-    A.plan.n_utt_rows[b] = on ? 1 : 0;
-    if (on) {
-      const int pr = A.last_row[b];
-      const int pos = A.prev_pos[b] + 1;
+    A.plan.n_utt_rows[b] = s_on ? 1 : 0;
+    if (s_on) {
       A.plan.row_b[r] = b;
       A.plan.row_i[r] = 0;
       A.plan.row_pos[r] = pos;
       A.plan.row_epos[r] = pos;
-      A.plan.row_tok[r] = A.draft_out[(size_t)b * A.k + i - 1];
-      A.row_src[r] = -3 - pr;   // the previous pass's block output of row pr
+      A.plan.row_tok[r] = tok;
       A.row_lo[r] = A.win_lo[b];
       A.row_hi[r] = A.win_hi[b];
-      A.row_key[r] = 0ull;
-      A.last_row[b] = r;
-    } else if (b < A.B) {
-      A.last_row[b] = -1;
+      N.row_key[r] = 0ull;
+    }
+    if (b == 0) {
+      A.plan.row_start[A.B] = total;
+      *A.plan.n_rows = total;
     }
   }
-  if (threadIdx.x == 0) {
-    A.plan.row_start[A.B] = total;
-    *A.plan.n_rows = total;
+  if (!s_on || bounds_bad(A.status, old < 0 || old >= A.r_max || r >= A.r_max)) return;   // uniform over the CTA
+  for (int c = 2 * u; c < d; c += 2 * DP_T) {
+    const float2 v = *reinterpret_cast<const float2*>(A.x_prev + (size_t)old * d + c);
+    const __nv_bfloat162 h = __floats2bfloat162_rn(v.x, v.y);
+#pragma unroll
+    for (int f = 0; f < 4; ++f) *reinterpret_cast<__nv_bfloat162*>(A.x_in + ((size_t)r * 4 + f) * d + c) = h;
   }
 }
 
-// x_in[r] = bf16 of the row's four representations ([4][d]): a tap row, the
-// saved tap of its utterance, zeros, or (continuation) the previous pass's
-// block output x_prev[pr] four times.  Grid-stride over rows x 4 d / 2.
+// Pass 0: x_in[r] = bf16 of the row's four representations ([4][d]): a tap
+// row, the saved tap of its utterance, or zeros.  Grid-stride over rows x 4 d / 2.
 __global__ void draft_gather_kernel(DraftArgs A) {
+  pdl_wait();
+  pdl_launch();
   const int R = *A.plan.n_rows, d = A.d;
   const int per = 2 * d;   // bf16 pairs per row
   for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < R * per; e += gridDim.x * blockDim.x) {
     const int r = e / per, c = 2 * (e - r * per);   // column c, c + 1 of [4 d]
     const int src = A.row_src[r];
-    if (bounds_bad(A.status, src >= A.r_max || (src <= -3 && -3 - src >= A.r_max) || r >= A.r_max ||
-                                 (src == -1 && (A.plan.row_b[r] < 0 || A.plan.row_b[r] >= A.B))))
+    if (bounds_bad(A.status, src >= A.r_max || r >= A.r_max || (src == -1 && (A.plan.row_b[r] < 0 || A.plan.row_b[r] >= A.B))))
       continue;
     float2 v;
     if (src >= 0) v = *reinterpret_cast<const float2*>(A.taps + (size_t)src * 4 * d + c);
     else if (src == -1) v = *reinterpret_cast<const float2*>(A.last_tap + (size_t)A.plan.row_b[r] * 4 * d + c);
-    else if (src == -2) v = make_float2(0.f, 0.f);
-    else v = *reinterpret_cast<const float2*>(A.x_prev + (size_t)(-3 - src) * d + (c % d));
+    else v = make_float2(0.f, 0.f);
     *reinterpret_cast<__nv_bfloat162*>(A.x_in + (size_t)r * 4 * d + c) = __floats2bfloat162_rn(v.x, v.y);
   }
 }
@@ -227,39 +285,53 @@ __global__ void draft_prefill_save_kernel(DraftArgs A) {
 }
 
 // x[r] += tok_emb[token] + pos_emb[position]  (the draft's input combination:
-// w_in [f_1; ..; f_4] + b_in was written by the input GEMM)
-__global__ void draft_embed_kernel(DraftArgs A, const __nv_bfloat16* tok_emb, const __nv_bfloat16* pos_emb, float* x) {
-  const int R = *A.plan.n_rows, d = A.d;
-  for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < R * d; e += gridDim.x * blockDim.x) {
-    const int r = e / d, c = e - r * d;
-    const int tok = A.plan.row_tok[r], pos = A.plan.row_epos[r];
-    if (bounds_bad(A.status, tok < 0 || tok >= A.vocab || pos < 0 || pos >= A.max_pos || r >= A.r_max)) continue;
-    x[e] += __bfloat162float(tok_emb[(size_t)A.plan.row_tok[r] * d + c]) +
-            __bfloat162float(pos_emb[(size_t)A.plan.row_epos[r] * d + c]);
-  }
-}
-
-// After a pass's LM head: each utterance with a row in the pass takes its
-// argmax as the next proposal (until it holds lens[b] of them, or, with the
-// confidence threshold on, until the argmax's probability falls below it:
-// the block then ends unproposed) and keeps the row's position for the next
-// continuation row.
-__global__ void draft_take_kernel(DraftArgs A) {
-  const int b = blockIdx.x * blockDim.x + threadIdx.x;
-  if (b >= A.B) return;
-  const int r = A.last_row[b];
-  if (r < 0) return;
-  const int n = A.n_prop[b];
-  A.prev_pos[b] = A.plan.row_pos[r];
-  if (n < A.lens[b]) {
-    if (A.threshold > 0.f && A.row_p[r] < A.threshold) {   // not confident: the block ends here
-      A.lens[b] = n;
-      return;
+// w_in [f_1; ..; f_4] + b_in was written by the input GEMM); with xg also the
+// first folded LayerNorm's operand bf16(gain * (x - mean)), centred since the
+// CTA holds the whole row, and its statistics as one slice of d features of mean
+// 0.  One CTA per row (d <= 2048: 16 values per thread).
+__global__ void __launch_bounds__(128)
+draft_embed_kernel(DraftArgs A, const __nv_bfloat16* __restrict__ tok_emb, const __nv_bfloat16* __restrict__ pos_emb,
+                   float* x, __nv_bfloat16* __restrict__ xg, const float* __restrict__ gain,
+                   float2* __restrict__ st_part) {
+  __shared__ float red[4];
+  pdl_wait();
+  pdl_launch();
+  const int r = blockIdx.x, d = A.d, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  if (r >= *A.plan.n_rows) return;   // uniform over the CTA
+  const int tok = A.plan.row_tok[r], pos = A.plan.row_epos[r];
+  if (bounds_bad(A.status, tok < 0 || tok >= A.vocab || pos < 0 || pos >= A.max_pos || r >= A.r_max)) return;
+  float v[16], s = 0.f;
+#pragma unroll
+  for (int i = 0; i < 16; ++i) {
+    const int c = threadIdx.x + 128 * i;
+    v[i] = 0.f;
+    if (c < d) {
+      v[i] = x[(size_t)r * d + c] +
+             (__bfloat162float(tok_emb[(size_t)tok * d + c]) + __bfloat162float(pos_emb[(size_t)pos * d + c]));
+      x[(size_t)r * d + c] = v[i];
     }
-    const uint32_t tok = argmax_index(A.row_key[r]);
-    A.draft_out[(size_t)b * A.k + n] = tok < (uint32_t)A.vocab ? (int)tok : 0;
-    A.n_prop[b] = n + 1;
+    s += v[i];
   }
+  if (xg == nullptr) return;
+  s = warp_sum(s);
+  if (lane == 0) red[warp] = s;
+  __syncthreads();
+  const float mean = ((red[0] + red[1]) + (red[2] + red[3])) / (float)d;
+  __syncthreads();
+  float q = 0.f;
+#pragma unroll
+  for (int i = 0; i < 16; ++i) {
+    const int c = threadIdx.x + 128 * i;
+    if (c < d) {
+      const float dv = v[i] - mean;
+      q += dv * dv;
+      xg[(size_t)r * d + c] = __float2bfloat16_rn(gain[c] * dv);
+    }
+  }
+  q = warp_sum(q);
+  if (lane == 0) red[warp] = q;
+  __syncthreads();
+  if (threadIdx.x == 0) st_part[r] = make_float2(0.f, (red[0] + red[1]) + (red[2] + red[3]));
 }
 
 // Softmax statistics of one row of logits (one CTA per row, fixed reduction
@@ -270,6 +342,8 @@ __global__ void __launch_bounds__(256) draft_softmax_kernel(const float* __restr
                                                             float* row_p) {
   __shared__ float s_m[8], s_s[8];
   __shared__ int s_i[8];
+  pdl_wait();
+  pdl_launch();
   const int r = blockIdx.x;
   if (r >= *n_rows) return;   // uniform over the CTA
   const float* l = logits + (size_t)r * V;
@@ -317,10 +391,19 @@ __global__ void __launch_bounds__(256) draft_softmax_kernel(const float* __restr
   }
 }
 
-// lens_out[b] = proposals made (or -1 for an utterance that holds its transcript)
-__global__ void draft_finish_kernel(DraftArgs A, int* lens_out) {
+// After the last pass (copy `par` of the state): its proposals, and the
+// round's outputs: lens_out[b] = proposals made (or -1 for an utterance that
+// holds its transcript), out[b][j] the proposals (out may be draft_out itself).
+__global__ void draft_finish_kernel(DraftArgs A, int par, int* out, int* lens_out) {
+  pdl_wait();
+  pdl_launch();
   const int b = blockIdx.x * blockDim.x + threadIdx.x;
-  if (b < A.B) lens_out[b] = A.lens[b] < 0 ? -1 : A.n_prop[b];
+  if (b >= A.B) return;
+  const Take t = draft_take(A, A.state[par], b);
+  if (t.tok >= 0) A.draft_out[(size_t)b * A.k + t.n - 1] = t.tok;
+  if (out != A.draft_out)
+    for (int j = 0; j < A.k; ++j) out[(size_t)b * A.k + j] = A.draft_out[(size_t)b * A.k + j];
+  lens_out[b] = t.lens < 0 ? -1 : t.n;
 }
 
 // Attention of the draft's block for up to NR rows of one (utterance, head):
@@ -334,15 +417,18 @@ __global__ void draft_finish_kernel(DraftArgs A, int* lens_out) {
 // and DA_U of those steps in flight, keys and values requested together; each
 // eight-lane group keeps its own online softmax, merged in a fixed order at
 // the end.  Rows of one utterance share the loads (NR = 4 for catch-up passes,
-// 1 where every utterance has one row).  The row-by-row kernel
-// with four-byte loads before it took 55 us a launch on average over two
-// rounds of the cached loop at batch 1 (d = 1280, k = 8, 1500 frames).
+// 1 where every utterance has one row).  At batch 1 (d =
+// 1280, k = 8, 1500 frames) 5.4 us a launch for one row and 11.5 for a catch-up
+// of nine; the row-by-row kernel with four-byte loads before it took 55 on
+// average over two rounds of the cached loop.
 constexpr int DA_T = 256, DA_U = 4;
 
 template <int NR>
 __global__ void __launch_bounds__(DA_T) draft_attn_kernel(DraftAttn a) {
   __shared__ float s_m[DA_T / 32][NR], s_l[DA_T / 32][NR], s_o[DA_T / 32][NR][64];
   __shared__ int s_ok[NR];   // 0: a row refused by the bounds-check mode
+  pdl_wait();
+  pdl_launch();
   const int hh = blockIdx.x, b = blockIdx.y, tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int i0 = blockIdx.z * NR, nr = min(NR, a.plan.n_utt_rows[b] - i0);
   if (nr <= 0) return;
@@ -473,12 +559,12 @@ __global__ void __launch_bounds__(DA_T) draft_attn_kernel(DraftAttn a) {
 void launch_draft_round_plan(const DraftArgs& a, cudaStream_t st) {
   draft_round_plan_kernel<<<1, DP_T, 0, st>>>(a);
 }
-void launch_draft_next_plan(const DraftArgs& a, int i, cudaStream_t st) {
-  draft_next_plan_kernel<<<1, DP_T, 0, st>>>(a, i);
+void launch_draft_step(const DraftArgs& a, int i, cudaStream_t st, bool pdl) {
+  launch_ex(draft_step_kernel, dim3(a.B), dim3(DP_T), 0, st, pdl, 1, a, i);
 }
-void launch_draft_gather(const DraftArgs& a, int rows_max, cudaStream_t st) {
+void launch_draft_gather(const DraftArgs& a, int rows_max, cudaStream_t st, bool pdl) {
   const int blocks = std::max(1, std::min(1024, (rows_max * 2 * a.d + 255) / 256));
-  draft_gather_kernel<<<blocks, 256, 0, st>>>(a);
+  launch_ex(draft_gather_kernel, dim3(blocks), dim3(256), 0, st, pdl, 1, a);
 }
 void launch_draft_prefill_gather(const DraftArgs& a, int rows_max, cudaStream_t st) {
   const int blocks = std::max(1, std::min(1024, (rows_max * 2 * a.d + 255) / 256));
@@ -486,26 +572,24 @@ void launch_draft_prefill_gather(const DraftArgs& a, int rows_max, cudaStream_t 
   draft_prefill_save_kernel<<<std::max(1, std::min(1024, (a.B * 4 * a.d + 255) / 256)), 256, 0, st>>>(a);
 }
 void launch_draft_embed(const DraftArgs& a, int rows_max, const void* tok_emb, const void* pos_emb, float* x,
-                        cudaStream_t st) {
-  const int blocks = std::max(1, std::min(1024, (rows_max * a.d + 255) / 256));
-  draft_embed_kernel<<<blocks, 256, 0, st>>>(a, static_cast<const __nv_bfloat16*>(tok_emb),
-                                              static_cast<const __nv_bfloat16*>(pos_emb), x);
+                        __nv_bfloat16* xg, const float* gain, float2* st_part, cudaStream_t st, bool pdl) {
+  launch_ex(draft_embed_kernel, dim3(std::max(1, rows_max)), dim3(128), 0, st, pdl, 1, a,
+            static_cast<const __nv_bfloat16*>(tok_emb), static_cast<const __nv_bfloat16*>(pos_emb), x, xg, gain,
+            st_part);
 }
-void launch_draft_take(const DraftArgs& a, cudaStream_t st) {
-  draft_take_kernel<<<(a.B + 255) / 256, 256, 0, st>>>(a);
-}
-void launch_draft_finish(const DraftArgs& a, int* lens_out, cudaStream_t st) {
-  draft_finish_kernel<<<(a.B + 255) / 256, 256, 0, st>>>(a, lens_out);
+void launch_draft_finish(const DraftArgs& a, int par, int* out, int* lens_out, cudaStream_t st, bool pdl) {
+  launch_ex(draft_finish_kernel, dim3((a.B + 127) / 128), dim3(128), 0, st, pdl, 1, a, par, out, lens_out);
 }
 void launch_draft_softmax(const float* logits, int V, const int* n_rows, int rows_max, unsigned long long* row_key,
-                          float* row_p, cudaStream_t st) {
-  draft_softmax_kernel<<<std::max(1, rows_max), 256, 0, st>>>(logits, V, n_rows, row_key, row_p);
+                          float* row_p, cudaStream_t st, bool pdl) {
+  launch_ex(draft_softmax_kernel, dim3(std::max(1, rows_max)), dim3(256), 0, st, pdl, 1, logits, V, n_rows, row_key,
+            row_p);
 }
 // One row per utterance (every continuation pass): a CTA per row and head.
 // More: groups of four rows share the key and value loads.
-void launch_draft_attn(const DraftAttn& a, int rows_per_utt, cudaStream_t st) {
-  if (rows_per_utt <= 1) draft_attn_kernel<1><<<dim3(a.H, a.B), DA_T, 0, st>>>(a);
-  else draft_attn_kernel<4><<<dim3(a.H, a.B, (rows_per_utt + 3) / 4), DA_T, 0, st>>>(a);
+void launch_draft_attn(const DraftAttn& a, int rows_per_utt, cudaStream_t st, bool pdl) {
+  if (rows_per_utt <= 1) launch_ex(draft_attn_kernel<1>, dim3(a.H, a.B), dim3(DA_T), 0, st, pdl, 1, a);
+  else launch_ex(draft_attn_kernel<4>, dim3(a.H, a.B, (rows_per_utt + 3) / 4), dim3(DA_T), 0, st, pdl, 1, a);
 }
 
 }  // namespace asrspec

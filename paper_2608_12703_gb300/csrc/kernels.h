@@ -244,6 +244,12 @@ cudaError_t launch_fr_gemv(const FrGemv& a, int mode, int ks, int groups, int d,
 // (App. "Window geometry"): the verification anchor (deployed), 500 ms later
 // (shifted control), a given frame (random control), or no window.
 enum DraftWin : int { DRAFT_WIN_ANCHOR = 0, DRAFT_WIN_SHIFTED = 1, DRAFT_WIN_RANDOM = 2, DRAFT_WIN_NONE = 3 };
+// What a pass leaves to the next, per utterance; two copies, so that a step
+// reads one while it writes the other.
+struct DraftState {
+  int *lens, *n_prop, *last_row, *pos;   // [B_max] proposals wanted and made; the pass's row (-1: none), its position
+  unsigned long long* row_key;           // [R_max] LM-head argmax keys of the pass
+};
 struct DraftArgs {
   int B, d, k, k_verify, win_kind;
   int vocab, max_pos, r_max;   // token ids, positions, rows of the pass buffers
@@ -260,9 +266,8 @@ struct DraftArgs {
   RowPlan plan;              // the draft pass's rows
   int *row_src, *row_lo, *row_hi;   // [R_max] feature source; audio window [lo, hi) per row
   int *win_lo, *win_hi;      // [B_max] the round's window
-  int *lens, *n_prop, *last_row, *prev_pos;   // [B_max]
+  DraftState state[2];       // pass i: state[i & 1]
   int* draft_out;            // [B][k] proposals
-  unsigned long long* row_key;   // [R_max] LM-head argmax keys of the pass
   __nv_bfloat16* x_in;       // [R_max][4 d] the pass's input representations
   float threshold;           // confidence threshold on the proposal's probability (0 = off)
   const float* row_p;        // [R_max] softmax probability of each row's argmax (threshold on)
@@ -277,19 +282,19 @@ struct DraftAttn {
   int* status;               // device status word (bounds-check mode)
 };
 void launch_draft_round_plan(const DraftArgs& a, cudaStream_t st);
-void launch_draft_next_plan(const DraftArgs& a, int i, cudaStream_t st);
-void launch_draft_gather(const DraftArgs& a, int rows_max, cudaStream_t st);
+void launch_draft_step(const DraftArgs& a, int i, cudaStream_t st, bool pdl);
+void launch_draft_gather(const DraftArgs& a, int rows_max, cudaStream_t st, bool pdl);
 void launch_draft_prefill_gather(const DraftArgs& a, int rows_max, cudaStream_t st);
+// xg / gain / st_part: as launch_embed's
 void launch_draft_embed(const DraftArgs& a, int rows_max, const void* tok_emb, const void* pos_emb, float* x,
-                        cudaStream_t st);
-void launch_draft_take(const DraftArgs& a, cudaStream_t st);
-void launch_draft_finish(const DraftArgs& a, int* lens_out, cudaStream_t st);
+                        __nv_bfloat16* xg, const float* gain, float2* st_part, cudaStream_t st, bool pdl);
+void launch_draft_finish(const DraftArgs& a, int par, int* out, int* lens_out, cudaStream_t st, bool pdl);
 // rows_per_utt: the most rows of one utterance in the pass
-void launch_draft_attn(const DraftAttn& a, int rows_per_utt, cudaStream_t st);
+void launch_draft_attn(const DraftAttn& a, int rows_per_utt, cudaStream_t st, bool pdl);
 // Per row of logits [rows][V] (fp32): the argmax key (as the LM-head epilogue
 // writes it: lowest index on ties) and the softmax probability of the argmax.
 void launch_draft_softmax(const float* logits, int V, const int* n_rows, int rows_max, unsigned long long* row_key,
-                          float* row_p, cudaStream_t st);
+                          float* row_p, cudaStream_t st, bool pdl);
 
 // ---- Accept / commit ------------------------------------------------------------
 void launch_prefill_advance(int B, int c, const int* n_utt_rows, int* kv_len, cudaStream_t st);

@@ -217,6 +217,51 @@ def test_draft_attention_edges(built_lib, cuda, k):
     _check(f"attention edges k{k}", st, ds, seqs, truth, total)
 
 
+def test_draft_many_utterances(built_lib, cuda):
+    """More utterances than a warp or half a plan CTA holds: row numbers of the
+    steps between passes, with some that finish early and some that never draft."""
+    B = 131
+    enc_lens = [1 + (b * 7) % 13 for b in range(B)]
+    total = [W.PROMPT_LEN + (0 if b % 17 == 3 else 1 + b % 5) for b in range(B)]
+    st, ds, seqs, truth, _ = run_lockstep(enc_lens, total, 3, "shifted")
+    _check("131 utterances", st, ds, seqs, truth, total)
+
+
+@pytest.mark.parametrize("k", [1, 4])
+def test_draft_host_io_equals_device_io(built_lib, cuda, k):
+    """The same rounds with host arrays (copied) and with device arrays (read
+    and written in place): drafts, lens and the verifications that follow."""
+    from paper_2608_12703_gb300 import asrspec as A
+    from paper_2608_12703_gb300.session import DraftModel, Session
+    enc_lens, total = [120, 33, 61], [W.PROMPT_LEN + n for n in (12, 3, 9)]
+    blob, dblob = W.make_weights(DIMS, std=STD), W.make_draft_weights(DIMS, std=STD)
+    enc, prompt = W.make_encoder_states(DIMS, enc_lens, 120), W.make_prompt(DIMS, 3)
+    logs = []
+    for host in (False, True):
+        sess = Session(DIMS, blob, max_batch=3, max_draft=k)
+        dm = DraftModel(sess, dblob, total, k, "random")
+        dm.set_centers([100, 2, 30])
+        sess.encode_cache(enc, enc_lens)
+        sess.prefill(prompt)
+        sess.set_host_io(host)
+        log = []
+        for _ in range(4):
+            if host:
+                d, l = np.full((3, k), -7, np.int32), np.zeros(3, np.int32)
+                A.asr_spec_draft_propose(sess.h, k, A.DRAFT_WIN["random"], np.array([100, 2, 30], np.int32),
+                                         np.array(total, np.int32), d, l)
+            else:
+                dd, ll = dm.propose(k)
+                d, l = sess.host(dd).copy(), sess.host(ll).copy()
+            o = sess.verify(d, l)
+            log.append(([list(d[b, :max(l[b], 0)]) for b in range(3)], list(l), list(o.accepted), list(o.bonus)))
+        sess.set_host_io(False)
+        assert sess.status() == 0
+        sess.close()
+        logs.append(log)
+    assert logs[0] == logs[1]
+
+
 def test_draft_long_prompt(built_lib, cuda):
     """A prompt of 41 tokens: its 40 rows in one prefill step, ten groups of the draft's attention."""
     total = [41 + n for n in (12, 9)]
