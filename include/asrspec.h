@@ -337,7 +337,7 @@ int asr_spec_timeline_read(asr_spec_handle h, uint64_t* ns, int32_t* kind, int32
  * query, cross out, MLP up, MLP down; their first 320 CTAs), the GPU global
  * timer (ns) at 12 phases (0 where a launch has no such phase); verify then
  * launches directly (no graph).  Tensor-core projections (all of them, or with
- * the few-row layers, batch x (k + 1) <= 9 rows, QKV and the cross query):
+ * the few-row layers, batch x (k + 1) <= 16 rows, QKV and the cross query):
  * 0 entry, 1 set-up done, 2 first k-block landed,
  * 3 MMAs done, 4 exit, 5 K-split partial staged (one CTA per tile: tile
  * staged in shared memory), 6 partials landed (staging barrier passed),

@@ -683,6 +683,7 @@ int run_layers_few(asr_spec* h, int N) {
   a.out_bf16 = 1;
   a.rows_max = rows_max;
   FrGemv g{};
+  g.rows = N;
   g.n_rows = h->plan.n_rows;
   g.status = h->status;
   g.x = h->x;

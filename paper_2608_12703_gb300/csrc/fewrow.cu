@@ -1,6 +1,7 @@
-// Few-row projections (at most 9 scored rows, e.g. batch 1 with k = 8).
+// Few-row projections (at most 16 scored rows, e.g. batch 1 with k = 8, or an
+// 11-node tree).
 //
-// A verification step at batch 1 moves the whole decoder's weights for 9
+// A verification step at batch 1 moves the whole decoder's weights for a few
 // rows (Sec. 3 "Speculative Loop": the target scores the draft block in one
 // pass), so every projection is matrix-vector-like and the step is a chain of
 // dependent exchanges: what a launch costs is its exchange latency, not its
@@ -15,7 +16,8 @@
 // (One cluster per head for LayerNorm + QKV + self-attention, and for the
 // cross query + cross-attention, took 11.5 and 10.7 us a layer at d = 1280 and
 // 9 rows, a round of the full decoder 1349 us; with the pairs of launches and
-// the operands requested early in the GEMVs it takes 1272.)
+// the operands requested early in the GEMVs it takes 1272.  10 to 16 rows gain 3
+// to 5 % over the GEMM chain: 12 rows, 8 layers 411 to 392 us, 14 rows 418 to 397.)
 // Every CTA computes whole 8-feature output tiles over its K range (mma.sync
 // m16n8k16, the rows padded to 16 as M, 8 weight rows as N; the K range
 // split over 8 warps and summed in warp order), so no split-K exchange is
@@ -55,8 +57,8 @@ __device__ __forceinline__ void fr_stamp(unsigned long long* tr, int phase) {
 // gain and bias of columns 4 (l + 32 i) .. + 3 (i < KSW), loaded before the
 // kernel waits on its predecessor (they are constants); after the wait, warp
 // w reads rows w and w + 8 of the residual stream straight from L2 into
-// registers (all FR_R row slots exist; the ones past the live rows are read
-// and not used), and writes bf16(LayerNorm(x_r) * g + b), fp32 statistics,
+// registers (all `rows` slots exist; the ones past the live rows are read and
+// not used), and writes bf16(LayerNorm(x_r) * g + b), fp32 statistics,
 // into the MMA operand rows.
 template <int KSW>
 struct LnRegs {
@@ -72,14 +74,14 @@ __device__ __forceinline__ void fr_ln_params(LnRegs<KSW>& p, const float* g, con
   }
 }
 template <int KSW>
-__device__ __forceinline__ void fr_ln_fetch(float4 (&v)[2][KSW], const float* x) {
+__device__ __forceinline__ void fr_ln_fetch(float4 (&v)[2][KSW], const float* x, int rows) {
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
 #pragma unroll
   for (int j = 0; j < 2; ++j) {
     const int r = warp + 8 * j;
     const float4* xr = reinterpret_cast<const float4*>(x + (size_t)r * KSW * 128);
 #pragma unroll
-    for (int i = 0; i < KSW; ++i) v[j][i] = r < FR_R ? __ldcg(xr + lane + 32 * i) : make_float4(0.f, 0.f, 0.f, 0.f);
+    for (int i = 0; i < KSW; ++i) v[j][i] = r < rows ? __ldcg(xr + lane + 32 * i) : make_float4(0.f, 0.f, 0.f, 0.f);
   }
 }
 template <int KSW>
@@ -168,42 +170,43 @@ __device__ __forceinline__ void fr_mma_panel(float (&acc)[FR_MAXT][4], uint32_t 
   }
 }
 
-// The 8 warps' partial tiles into red, then thread o < ntile * 4 * FR_R takes
-// output pair (tile i, row r, features 2 n2, 2 n2 + 1), summed in warp order.
+// The 8 warps' partial tiles into red.  Then output pair o (tile o / (4 rows),
+// row (o mod 4 rows) / 4, features 2 (o mod 4), + 1) is its eight partials summed
+// in warp order; thread tid takes the pairs tid and tid + 256 (FR_MAXT tiles of
+// FR_R rows are 320).
+constexpr int FR_PO = (FR_MAXT * 4 * FR_R + FR_T - 1) / FR_T;
 struct Pair {
   int i, r, n2;
-  float v0, v1;
   bool has;
 };
-__device__ __forceinline__ Pair fr_reduce(const float (&acc)[FR_MAXT][4], float* red, int ntile, bool live) {
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
-  if (live) {
-#pragma unroll
-    for (int i = 0; i < FR_MAXT; ++i) {
-      if (i < ntile) {
-        float* o = red + (warp * FR_MAXT + i) * 128;
-        *reinterpret_cast<float2*>(o + g * 8 + 2 * t) = make_float2(acc[i][0], acc[i][1]);
-        *reinterpret_cast<float2*>(o + (g + 8) * 8 + 2 * t) = make_float2(acc[i][2], acc[i][3]);
-      }
-    }
-  }
-  __syncthreads();
-  Pair p{0, 0, 0, 0.f, 0.f, false};
-  const int o = threadIdx.x;
-  if (live && o < ntile * 4 * FR_R) {
-    p.has = true;
-    p.i = o / (4 * FR_R);
-    const int rem = o - p.i * 4 * FR_R;
-    p.r = rem >> 2;
-    p.n2 = rem & 3;
-#pragma unroll
-    for (int w = 0; w < 8; ++w) {
-      const float2 v = *reinterpret_cast<const float2*>(red + (w * FR_MAXT + p.i) * 128 + p.r * 8 + 2 * p.n2);
-      p.v0 += v.x;
-      p.v1 += v.y;
-    }
-  }
+__device__ __forceinline__ Pair fr_pair(int o, int ntile, int rows) {
+  Pair p;
+  p.has = o < ntile * 4 * rows;
+  p.i = o / (4 * rows);
+  p.r = (o - p.i * 4 * rows) >> 2;
+  p.n2 = o & 3;
   return p;
+}
+__device__ __forceinline__ void fr_stage(const float (&acc)[FR_MAXT][4], float* red, int ntile) {
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
+#pragma unroll
+  for (int i = 0; i < FR_MAXT; ++i) {
+    if (i < ntile) {
+      float* o = red + (warp * FR_MAXT + i) * 128;
+      *reinterpret_cast<float2*>(o + g * 8 + 2 * t) = make_float2(acc[i][0], acc[i][1]);
+      *reinterpret_cast<float2*>(o + (g + 8) * 8 + 2 * t) = make_float2(acc[i][2], acc[i][3]);
+    }
+  }
+}
+__device__ __forceinline__ float2 fr_sum(const float* red, const Pair& p) {
+  float2 s = make_float2(0.f, 0.f);
+#pragma unroll
+  for (int w = 0; w < 8; ++w) {
+    const float2 v = *reinterpret_cast<const float2*>(red + (w * FR_MAXT + p.i) * 128 + p.r * 8 + 2 * p.n2);
+    s.x += v.x;
+    s.y += v.y;
+  }
+  return s;
 }
 
 // ---------------------------------------------------------------------------
@@ -241,7 +244,7 @@ __global__ void __launch_bounds__(FR_T, 1) fr_gemv_kernel(const __grid_constant_
     mbar_init(&abar, 1);
     mbar_init(&rbar, 1);
     fence_mbar_init();
-    if (KS > 1 && ks == 0) mbar_arrive_expect_tx(&rbar, (uint32_t)((KS - 1) * ntile * 4 * FR_R * 8));
+    if (KS > 1 && ks == 0) mbar_arrive_expect_tx(&rbar, (uint32_t)((KS - 1) * ntile * 4 * A.rows * 8));
     mbar_arrive_expect_tx(&wbar, (uint32_t)ntile * wtile);
     for (int i = 0; i < ntile; ++i)
       bulk_load(wts + i * wtile, A.W + ((size_t)(t0 + i) * A.K + (size_t)ks * Kc) * 8, wtile, &wbar);
@@ -249,14 +252,21 @@ __global__ void __launch_bounds__(FR_T, 1) fr_gemv_kernel(const __grid_constant_
   }
   LnRegs<KSW> lnr;
   if constexpr (MODE == FR_GELU) fr_ln_params(lnr, A.ln_g, A.ln_b);
-  // this thread's output pair (fr_reduce): its constant operands now, its residual after the wait
-  const bool out_has = ks == 0 && tid < ntile * 4 * FR_R;
-  const int out_r = (tid % (4 * FR_R)) >> 2, out_m = 8 * (t0 + tid / (4 * FR_R)) + 2 * (tid & 3);
-  float2 out_b = make_float2(0.f, 0.f), out_g = out_b, out_x = out_b;
-  if (out_has) {   // N is even, so a pair lies inside or outside
-    if (out_m < A.N) {
-      out_b = __ldg(reinterpret_cast<const float2*>(A.bias + out_m));
-      if (MODE == FR_RESID && A.xg) out_g = __ldg(reinterpret_cast<const float2*>(A.xg_gain + out_m));
+  // this thread's output pairs: their constant operands now, their residuals after the wait
+  const int n_out = ntile * 4 * A.rows;
+  Pair pr[FR_PO];
+  float2 out_b[FR_PO], out_g[FR_PO], out_x[FR_PO], out_v[FR_PO];
+#pragma unroll
+  for (int u = 0; u < FR_PO; ++u) {
+    pr[u].has = false;
+    out_b[u] = out_g[u] = out_x[u] = out_v[u] = make_float2(0.f, 0.f);
+    if (u * FR_T >= n_out) continue;   // uniform over the CTA: up to 12 rows have one pair per thread
+    pr[u] = fr_pair(tid + u * FR_T, ntile, A.rows);
+    const int m = 8 * (t0 + pr[u].i) + 2 * pr[u].n2;   // N is even, so a pair lies inside or outside
+    pr[u].has = pr[u].has && m < A.N;
+    if (ks == 0 && pr[u].has) {
+      out_b[u] = __ldg(reinterpret_cast<const float2*>(A.bias + m));
+      if (MODE == FR_RESID && A.xg) out_g[u] = __ldg(reinterpret_cast<const float2*>(A.xg_gain + m));
     }
   }
   __syncthreads();
@@ -265,22 +275,27 @@ __global__ void __launch_bounds__(FR_T, 1) fr_gemv_kernel(const __grid_constant_
   tl_mark(A.tl, TL_WORK);
   fr_stamp(A.trace, 1);
   pdl_launch();
-  // The input rows (written by the previous launch): all FR_R row slots,
+  // The input rows (written by the previous launch): all A.rows row slots,
   // requested at once without waiting to read how many are live (rows past
   // them are not used)
   float4 xv[2][KSW];
   if constexpr (MODE == FR_GELU) {
-    fr_ln_fetch<KSW>(xv, A.x);
+    fr_ln_fetch<KSW>(xv, A.x, A.rows);
   } else if (tid < 32) {   // panel p, row r: one bulk copy each, issued by the warp's lanes side by side
-    if (tid == 0) mbar_arrive_expect_tx(&abar, (uint32_t)(FR_R * np) * 2u * D);
+    if (tid == 0) mbar_arrive_expect_tx(&abar, (uint32_t)(A.rows * np) * 2u * D);
     __syncwarp();
-    for (int q = tid; q < FR_R * np; q += 32) {
-      const int p = q / FR_R, r = q - p * FR_R;
+    for (int q = tid; q < A.rows * np; q += 32) {
+      const int p = q / A.rows, r = q - p * A.rows;
       bulk_load(act + (p * FR_R + r) * P, A.a + (size_t)r * A.K + (size_t)ks * Kc + (size_t)p * D, 2u * D, &abar);
     }
   }
-  if constexpr (MODE == FR_RESID)   // every row slot exists
-    if (out_has && out_m < A.N) out_x = __ldcg(reinterpret_cast<const float2*>(A.x_out + (size_t)out_r * A.N + out_m));
+  if constexpr (MODE == FR_RESID) {   // every row slot exists
+#pragma unroll
+    for (int u = 0; u < FR_PO; ++u)
+      if (ks == 0 && pr[u].has)
+        out_x[u] = __ldcg(reinterpret_cast<const float2*>(A.x_out + (size_t)pr[u].r * A.N + 8 * (t0 + pr[u].i) +
+                                                          2 * pr[u].n2));
+  }
   const int R = *A.n_rows;   // uniform over the grid
   const bool live = R > 0;
   if constexpr (MODE == FR_GELU) {
@@ -299,54 +314,66 @@ __global__ void __launch_bounds__(FR_T, 1) fr_gemv_kernel(const __grid_constant_
   if (live)
     for (int p = 0; p < np; ++p)
       fr_mma_panel<KSW>(acc, smem_u32(act) + (uint32_t)(p * FR_R) * P, smem_u32(wts), wtile, p * (D / 8), ntile, R);
-  Pair pr = fr_reduce(acc, red, ntile, live);
+  if (live) fr_stage(acc, red, ntile);
+  __syncthreads();
+#pragma unroll
+  for (int u = 0; u < FR_PO; ++u)
+    if (live && u * FR_T < n_out && tid + u * FR_T < n_out) out_v[u] = fr_sum(red, pr[u]);
   tl_mark(A.tl, TL_MID);
   fr_stamp(A.trace, 4);
   if constexpr (KS > 1) {
     cluster_wait();   // rank 0's receive barrier exists
     if (live) {
       if (ks > 0) {
-        if (pr.has)
-          st_async_f2(dsmem_addr(&recv[(ks - 1) * FR_MAXT * 4 * FR_R + tid], 0), pr.v0, pr.v1,
-                      dsmem_addr(&rbar, 0));
+#pragma unroll
+        for (int u = 0; u < FR_PO; ++u)
+          if (tid + u * FR_T < n_out)
+            st_async_f2(dsmem_addr(&recv[(ks - 1) * FR_MAXT * 4 * FR_R + tid + u * FR_T], 0), out_v[u].x, out_v[u].y,
+                        dsmem_addr(&rbar, 0));
       } else {
         mbar_wait(&rbar, 0, A.status);
-        if (pr.has)
 #pragma unroll
-          for (int q = 0; q < KS - 1; ++q) {
-            const float2 o = recv[q * FR_MAXT * 4 * FR_R + tid];
-            pr.v0 += o.x;
-            pr.v1 += o.y;
-          }
+        for (int u = 0; u < FR_PO; ++u)
+          if (tid + u * FR_T < n_out)
+#pragma unroll
+            for (int q = 0; q < KS - 1; ++q) {
+              const float2 o = recv[q * FR_MAXT * 4 * FR_R + tid + u * FR_T];
+              out_v[u].x += o.x;
+              out_v[u].y += o.y;
+            }
       }
     }
   }
   fr_stamp(A.trace, 5);
-  // the folded LayerNorm's slice statistics: four consecutive lanes hold a row's 8 features of a tile
-  const float x0 = out_x.x + (pr.v0 + out_b.x), x1 = out_x.y + (pr.v1 + out_b.y);
-  float sl_mean = 0.f, sl_m2 = 0.f;
-  if (MODE == FR_RESID && A.xg) {   // uniform over the grid
-    sl_mean = x0 + x1;
-    sl_mean += __shfl_xor_sync(0xffffffffu, sl_mean, 1);
-    sl_mean += __shfl_xor_sync(0xffffffffu, sl_mean, 2);
-    sl_mean *= 0.125f;
-    sl_m2 = (x0 - sl_mean) * (x0 - sl_mean) + (x1 - sl_mean) * (x1 - sl_mean);
-    sl_m2 += __shfl_xor_sync(0xffffffffu, sl_m2, 1);
-    sl_m2 += __shfl_xor_sync(0xffffffffu, sl_m2, 2);
-  }
-  if (ks == 0 && pr.has && pr.r < R) {
-    const int m = 8 * (t0 + pr.i) + 2 * pr.n2;
-    if (m < A.N) {
+#pragma unroll
+  for (int u = 0; u < FR_PO; ++u) {
+    if (u * FR_T >= n_out) break;   // uniform over the CTA
+    const int m = 8 * (t0 + pr[u].i) + 2 * pr[u].n2;
+    const float v0 = out_v[u].x + out_b[u].x, v1 = out_v[u].y + out_b[u].y;
+    const float x0 = out_x[u].x + v0, x1 = out_x[u].y + v1;
+    // the folded LayerNorm's slice statistics: four consecutive lanes hold a row's 8 features of a tile
+    float sl_mean = 0.f, sl_m2 = 0.f;
+    if (MODE == FR_RESID && A.xg) {   // uniform over the grid
+      sl_mean = x0 + x1;
+      sl_mean += __shfl_xor_sync(0xffffffffu, sl_mean, 1);
+      sl_mean += __shfl_xor_sync(0xffffffffu, sl_mean, 2);
+      sl_mean *= 0.125f;
+      sl_m2 = (x0 - sl_mean) * (x0 - sl_mean) + (x1 - sl_mean) * (x1 - sl_mean);
+      sl_m2 += __shfl_xor_sync(0xffffffffu, sl_m2, 1);
+      sl_m2 += __shfl_xor_sync(0xffffffffu, sl_m2, 2);
+    }
+    if (ks == 0 && pr[u].has && pr[u].r < R) {
       if constexpr (MODE == FR_RESID) {
-        *reinterpret_cast<float2*>(A.x_out + (size_t)pr.r * A.N + m) = make_float2(x0, x1);
+        *reinterpret_cast<float2*>(A.x_out + (size_t)pr[u].r * A.N + m) = make_float2(x0, x1);
         if (A.xg) {
-          *reinterpret_cast<__nv_bfloat162*>(A.xg + (size_t)pr.r * A.N + m) =
-              __floats2bfloat162_rn(out_g.x * x0, out_g.y * x1);
-          if (pr.n2 == 0) A.st_part[(size_t)(t0 + pr.i) * A.st_stride + pr.r] = make_float2(sl_mean, sl_m2);
+          *reinterpret_cast<__nv_bfloat162*>(A.xg + (size_t)pr[u].r * A.N + m) =
+              __floats2bfloat162_rn(out_g[u].x * x0, out_g[u].y * x1);
+          if (pr[u].n2 == 0)
+            A.st_part[(size_t)(t0 + pr[u].i) * A.st_stride + pr[u].r] = make_float2(sl_mean, sl_m2);
         }
       } else {
-        *reinterpret_cast<__nv_bfloat162*>(A.h_out + (size_t)pr.r * A.N + m) =
-            __floats2bfloat162_rn(gelu_erf(pr.v0 + out_b.x), gelu_erf(pr.v1 + out_b.y));
+        *reinterpret_cast<__nv_bfloat162*>(A.h_out + (size_t)pr[u].r * A.N + m) =
+            __floats2bfloat162_rn(gelu_erf(v0), gelu_erf(v1));
       }
     }
   }

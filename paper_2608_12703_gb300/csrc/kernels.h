@@ -199,12 +199,13 @@ void launch_tree_commit(const int* path, int k, const int* accepted, const int* 
 // QKV on the many-row GEMM, self-attention, output projection; cross query on
 // the GEMM, cross-attention, output projection; LayerNorm + MLP up, MLP down;
 // the output and MLP projections as GEMVs over 8-feature tiles.
-constexpr int VF_ROWS = 9;
+constexpr int VF_ROWS = 16;
 enum FrMode : int { FR_RESID = 0, FR_GELU = 1 };
 struct FrGemv {
   const __nv_bfloat16* W;   // [N][K] weights
   const float* bias;        // [N]
   int N, K;                 // outputs, inputs
+  int rows;                 // rows of the step, at most (<= VF_ROWS)
   int tiles_max;            // 8-feature tiles per CTA, at most (<= 5): ceil(N / 8 / groups)
   const float* x;           // FR_GELU: the residual stream [R][K] (LayerNorm input)
   const float *ln_g, *ln_b;

@@ -14,7 +14,7 @@ few-row launches), --tree-nodes N (tree verifies beside the linear one), --enc-l
 anchor-readout share against batch size), --gemm IMPL,M,N,K (one GEMM shape
 through the kernel test entry, for captures of a single kernel).
 
-Kernel launches per round (bf16 decoders): at most 9 rows (e.g. batch 1):
+Kernel launches per round (bf16 decoders): at most 16 rows (e.g. batch 1):
 2 + 8 per layer + 3 (few-row layers, final LayerNorm, LM head, accept);
 more rows: 2 + 8 per layer + 2 (tensor-core chain, LayerNorm folded).
 """

@@ -77,6 +77,25 @@ def test_fewrow_small_decoder_against_oracle(built_lib, cuda, B, k, sched):
     assert_bounded(st)
 
 
+@pytest.mark.parametrize("d,heads,B,k", [(768, 12, 1, 15), (768, 12, 2, 4), (1280, 20, 4, 3), (512, 8, 3, 3), (1024, 16, 1, 11)])
+def test_fewrow_ten_to_sixteen_rows(built_lib, cuda, d, heads, B, k):
+    """More rows than the MMA's first eight, up to its sixteen; every width the
+    GEMVs are built for; more output pairs than threads (five tiles of 16 rows)."""
+    dims = W.ModelDims(n_layers=2, d_model=d, n_heads=heads, d_ffn=4 * d, vocab=900, dtype="bf16",
+                       max_pos=64, max_enc=200, anchor_layer=1)
+    blob = _blob(dims, 0.02)
+    enc_lens = [200, 77, 129, 1][:B]
+    enc = W.make_encoder_states(dims, enc_lens, 200)
+    prompt = W.make_prompt(dims, B)
+    total = [W.PROMPT_LEN + n for n in (25, 14, 20, 17)][:B]
+    wl = W.Workload("f", dims, B, k, tuple(t - W.PROMPT_LEN for t in total), tuple(enc_lens), (0.2,) * B, "half")
+    fac = _Traced(dims, blob, B, k)
+    st, _ = run_decode(dims, blob, enc, enc_lens, prompt, total, k, W.make_corruption(wl), fac)
+    _report(f"few-row d{d} B={B} k={k}", st)
+    assert fac.kinds.count(TL_QKV_SELF) == st.rounds * dims.n_layers > 0
+    assert_bounded(st)
+
+
 def test_fewrow_long_contexts(built_lib, cuda):
     """Contexts past two key chunks (a 300-token prompt: more self-attention
     chunks than a cluster has CTAs over three utterances) and a long-form
