@@ -1,8 +1,8 @@
-"""The few-row verify layers (six launches per layer: per-head clusters for
-LayerNorm + QKV + self-attention and LayerNorm + cross query +
-cross-attention, GEMVs for the projections) against the CPU oracle, against
-the tensor-core chain (ASRSPEC_FEWROW=0), and their launch structure.  A
-step takes them when the model is bf16 and batch x (k + 1) <= 9 rows."""
+"""The few-row verify layers (QKV and cross query on the K-split tensor-core
+projections, attention on the tensor-core kernel, GEMVs for the output and MLP
+projections) against the CPU oracle, against the tensor-core chain
+(ASRSPEC_FEWROW=0), and their launch structure.  A step takes them when the
+model is bf16 and batch x (k + 1) <= 16 rows."""
 import numpy as np
 import pytest
 
