@@ -117,14 +117,15 @@ __global__ void __launch_bounds__(FA_T) attn_f32_kernel(AttnArgs a) {
       float mx = m[i];
 #pragma unroll
       for (int u = 0; u < FA_U; ++u) mx = fmaxf(mx, s[i][u]);
-      const float c = mx == -INFINITY ? 0.f : expf(m[i] - mx);
+      const float mu = mx == -INFINITY ? 0.f : mx;   // no key yet: masked scores give 0, a NaN score stays NaN
+      const float c = expf(m[i] - mu);
       m[i] = mx;
       l[i] *= c;
 #pragma unroll
       for (int e = 0; e < 8; ++e) o[i][e] *= c;
 #pragma unroll
       for (int u = 0; u < FA_U; ++u) {
-        const float p = mx == -INFINITY ? 0.f : expf(s[i][u] - mx);
+        const float p = expf(s[i][u] - mu);
         const float4 v0 = vw[u][0], v1 = vw[u][1];
         l[i] += p;
         o[i][0] = fmaf(p, v0.x, o[i][0]); o[i][1] = fmaf(p, v0.y, o[i][1]);
@@ -141,7 +142,7 @@ __global__ void __launch_bounds__(FA_T) attn_f32_kernel(AttnArgs a) {
     for (int x = 8; x <= 16; x <<= 1) {
       const float om = __shfl_xor_sync(0xffffffffu, m[i], x), ol = __shfl_xor_sync(0xffffffffu, l[i], x);
       const float mx = fmaxf(m[i], om);
-      const float c0 = mx == -INFINITY ? 0.f : expf(m[i] - mx), c1 = mx == -INFINITY ? 0.f : expf(om - mx);
+      const float mu = mx == -INFINITY ? 0.f : mx, c0 = expf(m[i] - mu), c1 = expf(om - mu);
       m[i] = mx;
       l[i] = l[i] * c0 + ol * c1;
 #pragma unroll
@@ -160,12 +161,12 @@ __global__ void __launch_bounds__(FA_T) attn_f32_kernel(AttnArgs a) {
   const int i = tid >> 6, c = tid & 63;   // one output column of one row per thread
   float M = -INFINITY, L = 0.f, ot = 0.f;
   for (int w = 0; w < 8; ++w) M = fmaxf(M, s_m[w][i]);
-  if (M != -INFINITY)
-    for (int w = 0; w < 8; ++w) {
-      const float f = expf(s_m[w][i] - M);
-      L += s_l[w][i] * f;
-      ot += s_o[w][i][c] * f;
-    }
+  const float Mu = M == -INFINITY ? 0.f : M;
+  for (int w = 0; w < 8; ++w) {
+    const float f = expf(s_m[w][i] - Mu);
+    L += s_l[w][i] * f;
+    ot += s_o[w][i][c] * f;
+  }
   if (S > 1) {
     p_o[i][c] = ot;
     if (c == 0) {
@@ -192,7 +193,7 @@ __global__ void __launch_bounds__(FA_T) attn_f32_kernel(AttnArgs a) {
     for (int s2 = 0; s2 < 8; ++s2) M = fmaxf(M, om[s2]);
 #pragma unroll
     for (int s2 = 0; s2 < 8; ++s2) {
-      const float f = om[s2] == -INFINITY ? 0.f : expf(om[s2] - M);
+      const float f = expf(om[s2] - (M == -INFINITY ? 0.f : M));
       L += ol[s2] * f;
       ot += oo[s2] * f;
     }

@@ -499,13 +499,14 @@ __global__ void __launch_bounds__(DA_T) draft_attn_kernel(DraftAttn a) {
       float mx = m[i];
 #pragma unroll
       for (int u = 0; u < DA_U; ++u) mx = fmaxf(mx, s[i][u]);
-      const float c = mx == -INFINITY ? 0.f : expf(m[i] - mx);
+      const float mu = mx == -INFINITY ? 0.f : mx;   // no key yet: masked scores give 0, a NaN score stays NaN
+      const float c = expf(m[i] - mu);
       m[i] = mx;
       l[i] *= c;
 #pragma unroll
       for (int e = 0; e < 8; ++e) o[i][e] *= c;
 #pragma unroll
-      for (int u = 0; u < DA_U; ++u) s[i][u] = mx == -INFINITY ? 0.f : expf(s[i][u] - mx);
+      for (int u = 0; u < DA_U; ++u) s[i][u] = expf(s[i][u] - mu);
     }
 #pragma unroll
     for (int u = 0; u < DA_U; ++u) {
@@ -526,7 +527,7 @@ __global__ void __launch_bounds__(DA_T) draft_attn_kernel(DraftAttn a) {
     for (int x = 8; x <= 16; x <<= 1) {
       const float om = __shfl_xor_sync(0xffffffffu, m[i], x), ol = __shfl_xor_sync(0xffffffffu, l[i], x);
       const float mx = fmaxf(m[i], om);
-      const float c0 = mx == -INFINITY ? 0.f : expf(m[i] - mx), c1 = mx == -INFINITY ? 0.f : expf(om - mx);
+      const float mu = mx == -INFINITY ? 0.f : mx, c0 = expf(m[i] - mu), c1 = expf(om - mu);
       m[i] = mx;
       l[i] = l[i] * c0 + ol * c1;
 #pragma unroll
@@ -546,6 +547,7 @@ __global__ void __launch_bounds__(DA_T) draft_attn_kernel(DraftAttn a) {
   if (i >= nr || !s_ok[i]) return;
   float mx = -INFINITY, lt = 0.f, ot = 0.f;
   for (int w = 0; w < DA_T / 32; ++w) mx = fmaxf(mx, s_m[w][i]);
+  if (mx == -INFINITY) mx = 0.f;
   for (int w = 0; w < DA_T / 32; ++w) {
     const float f = expf(s_m[w][i] - mx);
     lt += s_l[w][i] * f;

@@ -376,3 +376,30 @@ def test_long_form_encoder_memory(built_lib, cuda):
     _report("long-form 5200 + 2100 frames", st)
     assert st.rows > 20
     assert_bounded(st)
+
+
+@pytest.mark.parametrize("dtype", ["fp32", "bf16"])
+def test_nan_score_of_one_frame_is_not_dropped(built_lib, cuda, dtype):
+    """A frame whose cross-attention score is not a number makes the row's
+    output NaN wherever the frame falls in the kernel's split of the keys, also
+    where it is alone: frame 5 of 30 holds a feature that overflows every key
+    component of head 0 (inf - inf in the score; its values stay finite)."""
+    import dataclasses
+    dims = dataclasses.replace(W.TINY, n_layers=1, d_model=128, n_heads=2, d_ffn=256, vocab=512, dtype=dtype)
+    blob = W.make_weights(dims).copy()
+    wk, wv = (W.weight_view(dims, blob, f"L0.{n}") for n in ("wck", "wcv"))
+    wk[:, 0] = 0.0
+    wk[:64, 0] = 3e38
+    wv[:, 0] = 0.0
+    enc = W.make_encoder_states(dims, [30], 30).copy()
+    enc[:, :, 0] = 0.0
+    sess = _session(dims, blob, 1, 2)()
+    prompt = W.make_prompt(dims, 1)
+    for bad in (False, True):
+        enc[0, 5, 0] = 10.0 if bad else 0.0
+        sess.encode_cache(enc, [30])
+        sess.prefill(prompt)
+        sess.verify(np.array([[3, 4]], dtype=np.int32), np.array([2], dtype=np.int32))
+        lg = sess.debug_logits(3).cpu().numpy()
+        assert np.isnan(lg).all() if bad else np.isfinite(lg).all()
+    assert sess.status() == 0
